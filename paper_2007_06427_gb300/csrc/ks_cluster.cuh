@@ -40,6 +40,7 @@ struct ClusterPlan {
     int nkmax;    // max 2 Ks + 1
     int rmax;     // max rows per rank
     int off_M, off_uh, off_rh, off_U, off_scr, off_part, off_red, off_tw, off_rin, off_tw_a;
+    int off_sc;   // scales of the double transforms of one call (max(ncmax, rt) ints)
     int off_tab;  // per-x-mode tables q_j, q_j^2 - q_j^4, q_j^4 (q_j^2 - 1)^2 (and the second in RA)
     int bytes;
     int u_global;  // 1: the rank's grid rows of u live in global memory (U array), not SMEM
@@ -146,13 +147,13 @@ __host__ __device__ inline int cluster_rows_per_rank(int ns, int C) {
 }
 
 // FFT of `cnt` columns stored [q][n] at `a` with `b` as scratch; the result is left in `a`.
-// nthr > 0: a double transform run by the first nthr threads only (see fft_batch), which alone
+// nthr > 0: a double transform run by the first nthr threads only (see fft_fx), which alone
 // call this; otherwise every thread of the block calls it.
 template <typename R>
 __device__ __forceinline__ void col_fft_inplace(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir,
-                                                const cpx<R>* tw, int nthr = 0) {
-    cpx<R>* r = nthr > 0 ? fft_col<R, true>(a, b, lg, cnt, dir, tw, nthr)
-                         : fft_col_warp<R, true>(a, b, lg, cnt, dir, tw);
+                                                const cpx<R>* tw, int* sc, int nthr = 0) {
+    cpx<R>* r = nthr > 0 ? fft_warp<R, true>(a, b, lg, cnt, dir, tw, sc, nthr)
+                         : fft_warp<R, true>(a, b, lg, cnt, dir, tw, sc);
     if (r != a) {
         const int n = cnt << lg;
         const int NT = nthr > 0 ? nthr : (int)blockDim.x;
@@ -244,6 +245,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
     Part* part = reinterpret_cast<Part*>(smem + cp.off_part);  // [2][nkx]: J, L2 partials
     double* red = reinterpret_cast<double*>(smem + cp.off_red);
     cpx<R>* tws = reinterpret_cast<cpx<R>*>(smem + cp.off_tw);
+    int* const fsc = reinterpret_cast<int*>(smem + cp.off_sc);
     // adjoint-precision views of the same buffers (phases are separated by barriers)
     cpx<RA>* Rin_a = reinterpret_cast<cpx<RA>*>(Rin);
     cpx<RA>* Mloc_a = reinterpret_cast<cpx<RA>*>(Mloc);
@@ -423,7 +425,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                                   : mk<R>(0, 0);
                 }
                 __syncthreads();
-                col_fft_inplace(Mloc, scr, lg, ncol >> 1, +1, tws);
+                col_fft_inplace(Mloc, scr, lg, ncol >> 1, +1, tws, fsc);
                 push_pairs(Mloc, Rin, true, -1);
             } else {
                 for (int i = wtid; i < ncol << lg; i += ntw) {
@@ -432,7 +434,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     Mloc[i] = (k >= -ks && k <= ks) ? uhl[q * nk + k + ks] : mk<R>(0, 0);
                 }
                 __syncthreads();
-                col_fft_inplace(Mloc, scr, lg, ncol, +1, tws);
+                col_fft_inplace(Mloc, scr, lg, ncol, +1, tws, fsc);
                 push_columns(Mloc, Rin, -1);
             }
         }
@@ -508,7 +510,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                         A[(size_t)pr * nx + J] = y;
                     }
                     __syncthreads();
-                    z = fft_pair_warp<R, true>(A, Bf, lgnx, np, +1, tws);
+                    z = fft_warp<R, true>(A, Bf, lgnx, np, +1, tws, fsc);
                     Y = (z == A) ? Bf : A;
                     for (int i = wtid; i < np * nx; i += ntw) {
                         const int pr = i >> lgnx, m = i & (nx - 1);
@@ -527,7 +529,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                         A[(size_t)r * nx + J] = zz;
                     }
                     __syncthreads();
-                    z = fft_warp<R, true>(A, Bf, lgnx, nr, +1, tws);
+                    z = fft_warp<R, true>(A, Bf, lgnx, nr, +1, tws, fsc);
                     Y = (z == A) ? Bf : A;
                     for (int i = wtid; i < np * nx; i += ntw) {
                         const int pr = i >> lgnx, m = i & (nx - 1);
@@ -539,7 +541,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     }
                 }
                 __syncthreads();
-                cpx<R>* F = fft_pair_warp<R, true>(Y, z, lgnx, np, -1, tws);
+                cpx<R>* F = fft_warp<R, true>(Y, z, lgnx, np, -1, tws, fsc);
                 const int lgp = lgnr - 1;
                 for (int i = wtid; i < (nkx << lgp); i += ntw) {
                     const int j = i >> lgp, pr = i & (np - 1);
@@ -566,7 +568,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     scr[i] = mk<R>(Mloc[((2 * pp) << lg) + n].y, hasb ? Mloc[((2 * pp + 1) << lg) + n].y : (R)0);
                 }
                 __syncthreads();
-                col_fft_inplace(scr, Mloc, lg, npair, -1, tws);
+                col_fft_inplace(scr, Mloc, lg, npair, -1, tws, fsc);
                 const R wTr = (R)wT;
                 for (int pp = 0; pp < npair; ++pp) {
                     const int ja = colj(2 * pp), jb = ja + 1;
@@ -613,9 +615,9 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                 }
                 __syncthreads();
                 // inverse of the pairs of i q r_hat (Mloc holds the spectra, scr is scratch)
-                push_pairs(fft_col_warp<RA, true>(Mloc_a, scr_a, lg, npair, +1, tws_a), Rin_a, false, 1);
+                push_pairs(fft_warp<RA, true>(Mloc_a, scr_a, lg, npair, +1, tws_a, fsc), Rin_a, false, 1);
             } else if (ncol > 0) {
-                col_fft_inplace(Mloc, scr, lg, ncol, -1, tws);
+                col_fft_inplace(Mloc, scr, lg, ncol, -1, tws, fsc);
                 const R wTr = (R)wT;
                 // columns in pairs: one block reduction for two columns' partials.  Element n of a
                 // column is accumulated by thread n mod COL_ACC_LANES, as in the item kernels, so
@@ -661,7 +663,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                 }
                 __syncthreads();
                 // inverse of i q r_hat (scr holds the spectra, Mloc is scratch), then push rho
-                push_columns(fft_col_warp<RA, true>(scr_a, Mloc_a, lg, ncol, +1, tws_a), Rin_a, 1);
+                push_columns(fft_warp<RA, true>(scr_a, Mloc_a, lg, ncol, +1, tws_a, fsc), Rin_a, 1);
             }
             xsync(1, bx_B);
 
@@ -695,7 +697,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     A[(size_t)pr * nx + J] = z;
                 }
                 wsync();
-                cpx<RA>* z = fft_pair_warp<RA, true>(A, Bf, lgnx, np, +1, tws_a, wn);
+                cpx<RA>* z = fft_warp<RA, true>(A, Bf, lgnx, np, +1, tws_a, fsc, wn);
                 cpx<RA>* Y = (z == A) ? Bf : A;
                 for (int i = wtid; i < np * nx; i += ntw) {
                     const int pr = i >> lgnx, m = i & (nx - 1);
@@ -704,7 +706,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                                   (RA)Ul[(size_t)(t0 + 2 * pr + 1) * nx + m] * rx.y);
                 }
                 wsync();
-                cpx<RA>* F = fft_pair_warp<RA, true>(Y, z, lgnx, np, -1, tws_a, wn);
+                cpx<RA>* F = fft_warp<RA, true>(Y, z, lgnx, np, -1, tws_a, fsc, wn);
                 for (int i = wtid; i < (nkx << lgp); i += ntw) {
                     const int j = i >> lgp, pr = i & (np - 1);
                     if (xi && j == 0) continue;
@@ -742,9 +744,9 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                                               hasb ? Mloc2_a[((2 * pp + 1) << lg) + n].y : (RA)0);
                         }
                         part_sync(nfft);
-                        col_fft_inplace(scr_a, Mloc2_a, lg, ncol >> 1, -1, tws_a, nfft);
+                        col_fft_inplace(scr_a, Mloc2_a, lg, ncol >> 1, -1, tws_a, fsc, nfft);
                     } else if (ncol > 0) {
-                        col_fft_inplace(Mloc2_a, scr_a, lg, ncol, -1, tws_a, nfft);
+                        col_fft_inplace(Mloc2_a, scr_a, lg, ncol, -1, tws_a, fsc, nfft);
                     }
                 }
             }
@@ -757,9 +759,9 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                                           hasb ? Mloc2_a[((2 * pp + 1) << lg) + n].y : (RA)0);
                     }
                     __syncthreads();
-                    col_fft_inplace(scr_a, Mloc2_a, lg, ncol >> 1, -1, tws_a);
+                    col_fft_inplace(scr_a, Mloc2_a, lg, ncol >> 1, -1, tws_a, fsc);
                 } else {
-                    col_fft_inplace(Mloc2_a, scr_a, lg, ncol, -1, tws_a);
+                    col_fft_inplace(Mloc2_a, scr_a, lg, ncol, -1, tws_a, fsc);
                 }
             }
             __syncthreads();
@@ -806,7 +808,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     Mloc2[i] = x;
                 }
                 __syncthreads();
-                push_pairs(fft_col_warp<R, true>(Mloc2, scr, lg, npair, +1, tws), Rin, true, 3);
+                push_pairs(fft_warp<R, true>(Mloc2, scr, lg, npair, +1, tws, fsc), Rin, true, 3);
             } else if (ncol > 0) {
                 const R wTr = (R)wT;
                 const R dt = (R)d.dtau;
@@ -876,7 +878,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     }
                 }
                 __syncthreads();
-                push_columns(fft_col_warp<R, true>(scr, Mloc2, lg, ncol, +1, tws), Rin, 3);
+                push_columns(fft_warp<R, true>(scr, Mloc2, lg, ncol, +1, tws, fsc), Rin, 3);
             }
             T = Tnext;
             wT = wTnext;

@@ -14,7 +14,7 @@
 // u_a^2 + i u_b^2); the state of each trajectory is its half spectrum v_j, j = 0..Kx, kept in
 // shared memory with the stage values of the scheme.  Global memory is touched at the start
 // (u0), at every saved instant (u and ||u||) and at the end.  The transforms take radix-2 passes
-// (fft_batch_r2): an FP64 warp instruction costs the same issue time with idle lanes, and a
+// (dns_fft): an FP64 warp instruction costs the same issue time with idle lanes, and a
 // radix-2 pass has twice the butterflies of a radix-4 pass at the same operation count per
 // point, so a single pair keeps a whole warp busy and four pairs fill the block's four warps.
 #include <cuda_runtime.h>
@@ -133,6 +133,44 @@ __device__ void dns_coefficients(double* coef, int nh, double L, double dt) {
     }
 }
 
+// The x-transforms of the run: cnt transforms of length n = 2^lg in double, radix-2 passes under the
+// conventions of fft_batch.  A run is chaotic, so its trajectory after a few hundred time units
+// hangs on the rounding of every transform: it keeps this arithmetic, where the descent's double
+// transforms are in fixed point.  With the twiddle product fused into the additions (v0 + w v1 as
+// four fused multiply-adds, v0 - w v1 as 2 v0 minus that) it costs 3 floating-point operations
+// per point per stage, as a fused radix-4 butterfly does, with twice the butterflies per pass.
+__device__ __forceinline__ cpx<double>* dns_fft(cpx<double>* a, cpx<double>* b, int lg, int cnt, int dir,
+                                                const cpx<double>* tw, int twsh) {
+    const int n = 1 << lg;
+    const int nb = n >> 1;
+    const int total = cnt * nb;
+    for (int span = 1; span < n; span <<= 1) {
+        const int tu = NMAX / (span * 2);
+        for (int i = threadIdx.x; i < total; i += blockDim.x) {
+            const int f = i >> (lg - 1);
+            const int j = i & (nb - 1);
+            const cpx<double>* s = a + (size_t)f * n;
+            cpx<double>* d = b + (size_t)f * n;
+            const cpx<double> v0 = s[j], v1 = s[j + nb];
+            const int jm = j & (span - 1);
+            const int od = ((j - jm) << 1) + jm;
+            if (span > 1) {
+                const cpx<double> t = cfma(v0, twid<double, true>(tw, jm * tu, dir, twsh), v1);
+                d[od] = t;
+                d[od + span] = twice_minus(v0, t);
+            } else {
+                d[od] = v0 + v1;
+                d[od + 1] = v0 - v1;
+            }
+        }
+        __syncthreads();
+        cpx<double>* t = a;
+        a = b;
+        b = t;
+    }
+    return a;
+}
+
 // spectrum `which` of trajectory t (t = 2 * pair + member) in the CTA's spectra block
 __device__ __forceinline__ cpx<double>* spec(cpx<double>* base, int nh, int t, int which) {
     return base + ((size_t)t * DNS_SPECS + which) * nh;
@@ -183,7 +221,7 @@ __device__ void dns_eval(const DnsArgs& a, int tr0, int ntraj, cpx<double>* fftb
         A[i] = z;
     }
     __syncthreads();
-    cpx<double>* Z = fft_batch_r2<double, true>(A, Bf, lgnx, np, +1, tw, 0, twsh);
+    cpx<double>* Z = dns_fft(A, Bf, lgnx, np, +1, tw, twsh);
     cpx<double>* Y = (Z == A) ? Bf : A;
     const double inx = 1.0 / (double)nx;  // exact: nx is a power of two
     const bool save = isave >= 0;
@@ -211,7 +249,7 @@ __device__ void dns_eval(const DnsArgs& a, int tr0, int ntraj, cpx<double>* fftb
             a.norms[(size_t)(tr0 + threadIdx.x) * a.nsave + isave] = sqrt(a.L * red[threadIdx.x] * inx);
     }
     if (dst < 0) return;
-    cpx<double>* F = fft_batch_r2<double, true>(Y, Z, lgnx, np, -1, tw, 0, twsh);
+    cpx<double>* F = dns_fft(Y, Z, lgnx, np, -1, tw, twsh);
     const double* g = coef + 6 * nh;
     for (int i = threadIdx.x; i < np * nh; i += blockDim.x) {
         const int pr = i / nh, j = i - pr * nh;
@@ -260,7 +298,7 @@ __global__ void __launch_bounds__(DNS_THREADS) k_dns(DnsArgs a) {
     }
     __syncthreads();
     {
-        cpx<double>* F = fft_batch_r2<double, true>(A, Bf, lgnx, np, -1, tw, 0, twsh);
+        cpx<double>* F = dns_fft(A, Bf, lgnx, np, -1, tw, twsh);
         for (int i = threadIdx.x; i < np * nh; i += blockDim.x) {
             const int pr = i / nh, j = i - pr * nh;
             const cpx<double> P = F[(size_t)pr * nx + j];

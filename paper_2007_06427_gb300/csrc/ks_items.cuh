@@ -233,7 +233,8 @@ struct Bufs {
     const int* prec;        // [B] 0 double, 1 float: the precision the loop currently runs in
     long long* steps;       // [B]
     double* sqrtJ;          // [B]
-    const cpx<R>* tw;       // [NMAX] exp(+2 pi i t / NMAX)
+    const cpx<R>* tw;       // float: [NMAX] exp(+2 pi i t / NMAX); double: [FX_TABLE] words of
+                            // ks_fx.cuh
     const R* qv;            // [nkx] q_j = 2 pi j / L in this precision
     const R* lin;           // [nkx] q_j^2 - q_j^4 (symbol of -u_xx - u_xxxx)
     const R* cq;            // [nkx] q_j^4 (q_j^2 - 1)^2 (x part of -Lambda_jk)
@@ -410,80 +411,24 @@ KS_HD cpx<R>* fft_batch(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir, const cp
     return a;
 }
 
-// Radix-2 variant of fft_batch (every pass a radix-2 pass, natural order in and out, same
-// conventions).  A pass has twice the butterflies of a radix-4 pass, so a double transform of
-// a single column keeps twice as many warps busy; with the twiddle product fused into the
-// additions (v0 + w v1 as four fused multiply-adds, v0 - w v1 as 2 v0 minus that) it costs 3
-// floating-point operations per point per radix-2 stage, as the fused radix-4 butterfly does.
-template <typename R, bool SWZ = false, bool SKI = false, bool SKO = false>
-KS_HD cpx<R>* fft_batch_r2(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir, const cpx<R>* tw,
-                           int nthr = 0, int twsh = 0) {
-#ifdef KS_HOST_EMULATION
-    const int NT = KS_NT;
-#else
-    const int NT = nthr > 0 ? nthr : KS_NT;
-#endif
-    const int n = 1 << lg;
-    const int nb = n >> 1;
-    const int total = cnt * nb;
-    for (int span = 1; span < n; span <<= 1) {
-        const int tu = NMAX / (span * 2);
-        const bool ski = SKI && span == 1, sko = SKO && 2 * span == n;
-        for (int i = KS_TID; i < total; i += NT) {
-            const int f = i >> (lg - 1);
-            const int j = i & (nb - 1);
-            const int si = ski ? row_skew<R>(f, n) : 0;
-            const int so = sko ? row_skew<R>(f, n) : 0;
-            const cpx<R>* s = a + (size_t)f * n;
-            cpx<R>* d = b + (size_t)f * n;
-            const cpx<R> v0 = s[j ^ si], v1 = s[(j + nb) ^ si];
-            const int jm = j & (span - 1);
-            const int od = ((j - jm) << 1) + jm;
-            if (span > 1) {
-                const cpx<R> t = cfma(v0, twid<R, SWZ>(tw, jm * tu, dir, twsh), v1);
-                d[od ^ so] = t;
-                d[(od + span) ^ so] = twice_minus(v0, t);
-            } else {
-                d[od ^ so] = v0 + v1;
-                d[(od + 1) ^ so] = v0 - v1;
-            }
-        }
-        if (nthr > 0) part_sync(nthr);
-        else KS_SYNC();
-        cpx<R>* t = a;
-        a = b;
-        b = t;
-    }
-    return a;
-}
+}  // namespace ks
 
-// The s-transforms (columns of the mixed array): in double, radix-2 passes (see fft_batch_r2)
-// unless the library is built with KS_COL_RADIX2=0; in float the radix-4 passes of fft_batch.
-// Every launch form calls this for its s-transforms, so they keep computing the same bits.
-#ifndef KS_COL_RADIX2
-#define KS_COL_RADIX2 1
-#endif
-template <typename R, bool SWZ = false>
-KS_HD cpx<R>* fft_col(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir, const cpx<R>* tw,
+#include "ks_fx.cuh"
+
+namespace ks {
+
+// The batched transform of every launch form: double in 64-bit fixed point (fft_fx, sc: room for
+// cnt scales), float in the radix-4 passes of fft_batch.  HOT: the phases of a tau-step, which take
+// the double transform inlined (256 ragged loops: 191 us a step, 229 through calls); the items at
+// the boundary of a call (analysis, synthesis, gradient) run once per call and share one copy of
+// it, which the launches of a call find in the instruction caches.
+template <typename R, bool HOT, bool SWZ = false, bool SKI = false, bool SKO = false>
+KS_HD cpx<R>* fft_any(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir, const cpx<R>* tw, int* sc,
                       int nthr = 0, int twsh = 0) {
-    if constexpr (sizeof(R) == 8 && KS_COL_RADIX2) return fft_batch_r2<R, SWZ>(a, b, lg, cnt, dir, tw, nthr, twsh);
-    else return fft_batch<R, SWZ>(a, b, lg, cnt, dir, tw, nthr, twsh);
-}
-
-// The x-transforms of row pairs (two real rows packed as one complex row: the forward
-// transforms of the products and of the analysis, the inverse ones of r_x and of the synthesis)
-// have half as many transforms as the batch has rows; in double they take radix-2 passes
-// unless the library is built with KS_PAIR_RADIX2=0.  The transform of z = u + i u_x, one per
-// row, keeps the radix-4 passes.  The choice depends on the transform's role only, so every
-// launch form computes the same bits.
-#ifndef KS_PAIR_RADIX2
-#define KS_PAIR_RADIX2 1
+#ifndef KS_HOST_EMULATION
+    if constexpr (sizeof(R) == 8 && !HOT) return fft_fx_call(a, b, lg, cnt, dir, tw, sc, nthr);
 #endif
-template <typename R, bool SWZ = false, bool SKI = false, bool SKO = false>
-KS_HD cpx<R>* fft_pair(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir, const cpx<R>* tw,
-                       int nthr = 0, int twsh = 0) {
-    if constexpr (sizeof(R) == 8 && KS_PAIR_RADIX2)
-        return fft_batch_r2<R, SWZ, SKI, SKO>(a, b, lg, cnt, dir, tw, nthr, twsh);
+    if constexpr (sizeof(R) == 8) return fft_fx(a, b, lg, cnt, dir, tw, sc, nthr);
     else return fft_batch<R, SWZ, SKI, SKO>(a, b, lg, cnt, dir, tw, nthr, twsh);
 }
 
@@ -493,11 +438,9 @@ KS_HD cpx<R>* fft_pair(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir, const cpx
 // the end.  Same arithmetic in the same order as fft_batch (bit-identical results), far fewer
 // block-wide barriers.  Device code only.
 //
-// Double: an FP64 warp instruction costs the same issue time with idle lanes, and a 64-point
-// radix-4 pass has only 16 butterflies per transform, so the double transform runs as
-// fft_batch itself (butterflies of all transforms spread over full warps).  A float transform
-// is latency-bound and keeps one transform per warp.  (Unrolling the float passes for fixed
-// lengths saved little inside the step and cost instruction-cache misses after a launch.)
+// The float transforms of the cluster kernel, which are latency-bound.  (Unrolling the passes
+// for fixed lengths saved little inside the step and cost instruction-cache misses after a
+// launch.)
 // ------------------------------------------------------------------------------------
 #ifndef KS_HOST_EMULATION
 // nthr > 0: only the first nthr threads (a multiple of 32) own transforms and call this; the
@@ -592,8 +535,13 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_al
 // transform of the cluster and persistent kernels reads the table through it): the values the
 // transforms read are unchanged, and the bytes fetched drop by NMAX / nm (8x for 128-point
 // columns).
+// Double: the prefix of the pass-ordered table of ks_fx.cuh, as it stands.
 template <typename X>
 __device__ __forceinline__ void load_twiddles(cpx<X>* dst, const cpx<X>* src, int nm) {
+    if constexpr (sizeof(X) == 8) {
+        for (int i = threadIdx.x; i < fx_table_len(nm); i += blockDim.x) cp_async<16>(dst + i, src + i);
+        return;
+    }
     const int st = NMAX / nm;
     for (int i = threadIdx.x; i < nm; i += blockDim.x)
         cp_async<sizeof(cpx<X>)>(dst + tw_swz<X>(i * st), src + (size_t)i * st);
@@ -604,36 +552,31 @@ __device__ __forceinline__ void load_twiddles(cpx<X>* dst, const cpx<X>* src, in
 // two, which the swizzle spreads over the banks as before.
 template <typename X>
 __device__ __forceinline__ void load_twiddles_compact(cpx<X>* dst, const cpx<X>* src, int nm) {
+    if constexpr (sizeof(X) == 8) {
+        load_twiddles(dst, src, nm);
+        return;
+    }
     const int st = NMAX / nm;
     for (int i = threadIdx.x; i < nm; i += blockDim.x)
         cp_async<sizeof(cpx<X>)>(dst + tw_swz<X>(i), src + (size_t)i * st);
 }
 
-template <typename R, bool SWZ = false, bool SKI = false, bool SKO = false>
-__device__ __forceinline__ cpx<R>* fft_warp(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir,
-                                            const cpx<R>* tw, int nthr = 0) {
-    if constexpr (sizeof(R) == 8) return fft_batch<R, SWZ, SKI, SKO>(a, b, lg, cnt, dir, tw, nthr);
-    else return fft_warp_any<R, SWZ, SKI, SKO>(a, b, lg, cnt, dir, tw, nthr);
-}
-
-// row-pair x-transforms of the cluster kernel: the double ones as fft_pair (block-wide), the float
-// ones warp-owned (the same arithmetic as fft_pair's radix-4 passes)
-template <typename R, bool SWZ = false, bool SKI = false, bool SKO = false>
-__device__ __forceinline__ cpx<R>* fft_pair_warp(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir,
-                                                 const cpx<R>* tw, int nthr = 0) {
-    if constexpr (sizeof(R) == 8) return fft_pair<R, SWZ, SKI, SKO>(a, b, lg, cnt, dir, tw, nthr);
-    else return fft_warp_any<R, SWZ, SKI, SKO>(a, b, lg, cnt, dir, tw, nthr);
-}
-
-// s-transforms of the cluster kernel: the double ones as fft_col (block-wide), the float ones
-// warp-owned (the same arithmetic as fft_col's radix-4 passes)
+// the transforms of the cluster kernel: the double ones block-wide (fft_fx), the float ones
+// warp-owned (the same arithmetic as fft_batch)
 template <typename R, bool SWZ = false>
-__device__ __forceinline__ cpx<R>* fft_col_warp(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir,
-                                                const cpx<R>* tw, int nthr = 0) {
-    if constexpr (sizeof(R) == 8) return fft_col<R, SWZ>(a, b, lg, cnt, dir, tw, nthr);
+__device__ __forceinline__ cpx<R>* fft_warp(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir,
+                                            const cpx<R>* tw, int* sc, int nthr = 0) {
+    if constexpr (sizeof(R) == 8) return fft_fx_call(a, b, lg, cnt, dir, tw, sc, nthr);
     else return fft_warp_any<R, SWZ>(a, b, lg, cnt, dir, tw, nthr);
 }
 #endif
+
+// Bytes of the table that load_twiddles (compact: load_twiddles_compact) fills for lengths up to nm.
+template <typename X>
+KS_HDX size_t twiddle_bytes(int nm, bool compact) {
+    if constexpr (sizeof(X) == 8) return (size_t)fx_table_len(nm) * sizeof(fxw);
+    else return (size_t)(compact ? nm : NMAX) * sizeof(cpx<X>);
+}
 
 // First xor distance of the reduction over the per-warp sums held by lanes 0..nw-1 of warp 0
 // (the other lanes hold zeros).  At a distance >= nw a lane below nw only meets lanes whose
@@ -1107,6 +1050,8 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
     cpx<R>* Bf = A + (size_t)nr * nx;
     cpx<R>* Mb = p.M + p.moff[b];
     R* Ub = p.U + p.goff[b];
+    int* sc = reinterpret_cast<int*>(Bf + (size_t)nr * nx);  // scales of double transforms
+    constexpr bool kHot = MODE == ROW_NONLIN || MODE == ROW_ADJ;
     R* Ib = p.io ? p.io + p.goff[b] : nullptr;
 
     if constexpr (MODE == ROW_ANALYZE) {
@@ -1119,13 +1064,13 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
             A[i] = mk<R>(ra[m], ra[nx + m]);
         }
         KS_SYNC();
-        cpx<R>* Y = fft_pair<R, SWZ, false, true>(A, Bf, lgnx, npairs, -1, p.tw, 0, p.twsh);
+        cpx<R>* Y = fft_any<R, kHot, SWZ, false, true>(A, Bf, lgnx, npairs, -1, p.tw, sc, 0, p.twsh);
         store_pair_spectra(d, Y, Mb, ns, n0, lgp);
         KS_SYNC();
     } else if constexpr (MODE == ROW_SYNTH) {
         load_pair_spectra(d, Mb, ns, n0, lgp, A);
         KS_SYNC();
-        cpx<R>* z = fft_pair<R, SWZ, true, false>(A, Bf, lgnx, npairs, +1, p.tw, 0, p.twsh);
+        cpx<R>* z = fft_any<R, kHot, SWZ, true, false>(A, Bf, lgnx, npairs, +1, p.tw, sc, 0, p.twsh);
         const int total = npairs * nx;
         for (int i = KS_TID; i < total; i += KS_NT) {
             const int pr = i >> lgnx;
@@ -1153,7 +1098,7 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                 A[(size_t)pr * nx + (J ^ row_skew<R>(pr, nx))] = y;
             }
             KS_SYNC();
-            cpx<R>* yv = fft_pair<R, SWZ, true, false>(A, Bf, lgnx, npairs, +1, p.tw, 0, p.twsh);
+            cpx<R>* yv = fft_any<R, kHot, SWZ, true, false>(A, Bf, lgnx, npairs, +1, p.tw, sc, 0, p.twsh);
             cpx<R>* Y = (yv == A) ? Bf : A;
             for (int i = KS_TID; i < total; i += KS_NT) {
                 const int pr = i >> lgnx;
@@ -1166,7 +1111,7 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                 Y[i] = mk<R>(ua * uxa, ub * uxb);
             }
             KS_SYNC();
-            cpx<R>* F = fft_pair<R, SWZ, false, true>(Y, yv, lgnx, npairs, -1, p.tw, 0, p.twsh);  // a4 (x-pass)
+            cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, yv, lgnx, npairs, -1, p.tw, sc, 0, p.twsh);  // a4 (x-pass)
             store_pair_spectra(d, F, Mb, ns, n0, lgp);
             KS_SYNC();
             return;
@@ -1186,7 +1131,7 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
             A[(size_t)r * nx + (J ^ row_skew<R>(r, nx))] = z;
         }
         KS_SYNC();
-        cpx<R>* z = fft_batch<R, SWZ, true, false>(A, Bf, lgnx, nr, +1, p.tw, 0, p.twsh);
+        cpx<R>* z = fft_any<R, kHot, SWZ, true, false>(A, Bf, lgnx, nr, +1, p.tw, sc, 0, p.twsh);
         cpx<R>* Y = (z == A) ? Bf : A;
         // keep u, form p = u u_x for the row pairs (a3)
         const int tp = npairs * nx;
@@ -1201,14 +1146,14 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
             Y[i] = mk<R>(za.x * za.y, zb.x * zb.y);
         }
         KS_SYNC();
-        cpx<R>* F = fft_pair<R, SWZ, false, true>(Y, z, lgnx, npairs, -1, p.tw, 0, p.twsh);  // a4 (x-pass)
+        cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, z, lgnx, npairs, -1, p.tw, sc, 0, p.twsh);  // a4 (x-pass)
         store_pair_spectra(d, F, Mb, ns, n0, lgp);
         KS_SYNC();
     } else if constexpr (MODE == ROW_ADJ) {
         // r_x rows from the column pass output rho = s-inverse of i q_j r_hat   (a7)
         load_pair_spectra(d, Mb, ns, n0, lgp, A);
         KS_SYNC();
-        cpx<R>* z = fft_pair<R, SWZ, true, false>(A, Bf, lgnx, npairs, +1, p.tw, 0, p.twsh);
+        cpx<R>* z = fft_any<R, kHot, SWZ, true, false>(A, Bf, lgnx, npairs, +1, p.tw, sc, 0, p.twsh);
         cpx<R>* Y = (z == A) ? Bf : A;
         const int tp = npairs * nx;
         for (int i = KS_TID; i < tp; i += KS_NT) {
@@ -1219,7 +1164,7 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
             Y[i] = mk<R>(ua[m] * rx.x, ua[nx + m] * rx.y);  // w = u r_x  (a8)
         }
         KS_SYNC();
-        cpx<R>* F = fft_pair<R, SWZ, false, true>(Y, z, lgnx, npairs, -1, p.tw, 0, p.twsh);
+        cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, z, lgnx, npairs, -1, p.tw, sc, 0, p.twsh);
         store_pair_spectra(d, F, Mb, ns, n0, lgp);
         KS_SYNC();
         // double: the loop's step scalars, once per loop (the column partials are complete since
@@ -1261,7 +1206,10 @@ enum ColMode {
 };
 
 // Shared-memory bytes a column item needs beyond its two transform buffers.
-constexpr int COL_RED_DOUBLES = 4 * (256 / 32 + 1) + 4;  // blocks of up to 256 threads
+constexpr int COL_RED_SC = 4 * (256 / 32 + 1);       // block sums of up to 256 threads, then the
+constexpr int COL_RED_DOUBLES = COL_RED_SC + 4;      // scale of the double transform
+// Bytes a row item of nr rows needs beyond its two transform buffers (scales).
+KS_HDX size_t row_extra_bytes(int nr) { return ((size_t)nr * sizeof(int) + 15) & ~(size_t)15; }
 
 
 // Threads that accumulate one column's J and L^dag_2 partial: element n of a column goes to
@@ -1339,6 +1287,8 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
     cpx<R>* A = reinterpret_cast<cpx<R>*>(smem);
     cpx<R>* Bf = A + ns;
     double* red = reinterpret_cast<double*>(Bf + ns);
+    int* sc = reinterpret_cast<int*>(red + COL_RED_SC);
+    constexpr bool kHot = MODE == COL_RESID || MODE == COL_UPDATE;
     cpx<R>* const M0 = p.M + p.moff[b];
     cpx<R>* const cola = M0 + (size_t)ja * ns;
     cpx<R>* const colb = M0 + (size_t)jb * ns;   // used only when hasb
@@ -1373,7 +1323,7 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
             A[i] = x;
         }
         KS_SYNC();
-        const cpx<R>* v = fft_col<R, SWZ>(A, Bf, lg, 1, +1, p.tw, 0, p.twsh);
+        const cpx<R>* v = fft_any<R, kHot, SWZ>(A, Bf, lg, 1, +1, p.tw, sc, 0, p.twsh);
         for (int i = KS_TID; i < ns; i += KS_NT) {
             cola[i] = mk<R>(0, v[i].x);
             if (hasb) colb[i] = mk<R>(0, v[i].y);
@@ -1385,7 +1335,7 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
         // RESID, UPDATE, GRAD: forward s-transform of the imaginary columns P or W of M, in one
         for (int i = KS_TID; i < ns; i += KS_NT) A[i] = mk<R>(cola[i].y, hasb ? colb[i].y : (R)0);
         KS_SYNC();
-        cpx<R>* F = fft_col<R, SWZ>(A, Bf, lg, 1, -1, p.tw, 0, p.twsh);
+        cpx<R>* F = fft_any<R, kHot, SWZ>(A, Bf, lg, 1, -1, p.tw, sc, 0, p.twsh);
         cpx<R>* X = (F == A) ? Bf : A;
         const R ins = p.insv[b];
         const R w_over_T = (R)wTc[b];
@@ -1429,7 +1379,7 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
                         if (hasb) acc[1].add(p.uh[bb + (k + ks)], p.rh[bb + (k + ks)], k);
                     }
                 }
-            const cpx<R>* v = fft_col<R, SWZ>(X, F, lg, 1, +1, p.tw, 0, p.twsh);
+            const cpx<R>* v = fft_any<R, kHot, SWZ>(X, F, lg, 1, +1, p.tw, sc, 0, p.twsh);
             for (int i = KS_TID; i < ns; i += KS_NT) {
                 cola[i] = mk<R>(v[i].x, 0);
                 if (hasb) colb[i] = mk<R>(v[i].y, 0);
@@ -1508,7 +1458,7 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
                 X[i] = x;
             }
             KS_SYNC();
-            const cpx<R>* v = fft_col<R, SWZ>(X, F, lg, 1, +1, p.tw, 0, p.twsh);
+            const cpx<R>* v = fft_any<R, kHot, SWZ>(X, F, lg, 1, +1, p.tw, sc, 0, p.twsh);
             for (int i = KS_TID; i < ns; i += KS_NT) {
                 cola[i] = mk<R>(0, v[i].x);
                 if (hasb) colb[i] = mk<R>(0, v[i].y);
@@ -1535,6 +1485,8 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
     cpx<R>* A = reinterpret_cast<cpx<R>*>(smem);
     cpx<R>* Bf = A + ns;
     double* red = reinterpret_cast<double*>(Bf + ns);
+    int* sc = reinterpret_cast<int*>(red + COL_RED_SC);
+    constexpr bool kHot = MODE == COL_RESID || MODE == COL_UPDATE;
     cpx<R>* col = p.M + p.moff[b] + (size_t)j * ns;
     const size_t bo = (size_t)p.boff[b] + (size_t)j * nk;
     const int B = d.B;
@@ -1564,14 +1516,14 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
             A[i] = (k >= -ks && k <= ks) ? src[bo + (k + ks)] : mk<R>(0, 0);
         }
         KS_SYNC();
-        cpx<R>* v = fft_col<R, SWZ>(A, Bf, lg, 1, +1, p.tw, 0, p.twsh);
+        cpx<R>* v = fft_any<R, kHot, SWZ>(A, Bf, lg, 1, +1, p.tw, sc, 0, p.twsh);
         for (int i = KS_TID; i < ns; i += KS_NT) col[i] = v[i];
         KS_SYNC();
     } else {
         // the remaining modes start with a forward s-transform of the column of M
         for (int i = KS_TID; i < ns; i += KS_NT) A[i] = col[i];
         KS_SYNC();
-        cpx<R>* F = fft_col<R, SWZ>(A, Bf, lg, 1, -1, p.tw, 0, p.twsh);
+        cpx<R>* F = fft_any<R, kHot, SWZ>(A, Bf, lg, 1, -1, p.tw, sc, 0, p.twsh);
         cpx<R>* X = (F == A) ? Bf : A;
         const R ins = p.insv[b];
 
@@ -1615,7 +1567,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                     const int k = (i < (ns >> 1)) ? i : i - ns;
                     if (k >= -ks && k <= ks) acc.add(p.uh[bo + (k + ks)], p.rh[bo + (k + ks)], k);
                 }
-            cpx<R>* v = fft_col<R, SWZ>(X, F, lg, 1, +1, p.tw, 0, p.twsh);
+            cpx<R>* v = fft_any<R, kHot, SWZ>(X, F, lg, 1, +1, p.tw, sc, 0, p.twsh);
             for (int i = KS_TID; i < ns; i += KS_NT) col[i] = v[i];
             block_reduce(acc, red);
             if (KS_TID == 0) {
@@ -1696,7 +1648,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                 Y[i] = x;
             }
             KS_SYNC();
-            cpx<R>* v = fft_col<R, SWZ>(Y, p.xi ? X : F, lg, 1, +1, p.tw, 0, p.twsh);
+            cpx<R>* v = fft_any<R, kHot, SWZ>(Y, p.xi ? X : F, lg, 1, +1, p.tw, sc, 0, p.twsh);
             for (int i = KS_TID; i < ns; i += KS_NT) col[i] = v[i];
             KS_SYNC();
         }

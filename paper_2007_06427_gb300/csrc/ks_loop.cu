@@ -620,9 +620,9 @@ int set_smem_attrs(ks_loop* h) {
 template <typename R>
 int setup_persistent(ks_loop* h) {
     const int pr = std::is_same<R, double>::value ? P64 : P32;
-    // the items' buffers, then the twiddle table (NMAX entries, swizzled positions)
+    // the items' buffers, then the twiddle table
     const size_t items_sm = std::max(h->lrow[pr].tw_off, h->lcol[pr].tw_off);  // 16-aligned
-    const size_t sm = items_sm + (size_t)NMAX * sizeof(cpx<R>);
+    const size_t sm = items_sm + twiddle_bytes<R>(std::max(h->d.nx, h->nsmax), false);
     h->ptw_off[pr] = (int)items_sm;
     KS_CUDA(cudaFuncSetAttribute(k_persist<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     int per_sm = 0, sms = 0, coop = 0;
@@ -673,8 +673,10 @@ ClusterPlan make_cluster_plan(const ks_loop* h, int C, int u_global, int smem_li
     off += al((size_t)2 * nkx * sizeof(double));
     cp.off_red = (int)off;
     off += al((size_t)COL_RED_DOUBLES * sizeof(double));
+    cp.off_sc = (int)off;
+    off += al((size_t)std::max(cp.ncmax, rt) * sizeof(int));
     cp.off_tw = (int)off;
-    off += al((size_t)NMAX * cs);
+    off += al(twiddle_bytes<R>(std::max(nx, cp.nsmax), false));
     cp.off_rin = (int)off;
     off += al((size_t)nkx * cp.rmax * cs);
     cp.off_tw_a = (int)off;
@@ -1148,11 +1150,9 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
     {
         std::vector<double> re, im;
         twiddles(re, im);
-        std::vector<cpx<double>> t64(NMAX);
+        const std::vector<fxw> t64 = fx_table();  // the double transforms' twiddles (ks_fx.cuh)
         std::vector<cpx<float>> t32(NMAX);
         for (int t = 0; t < NMAX; ++t) {
-            t64[t].x = re[t];
-            t64[t].y = im[t];
             t32[t].x = (float)re[t];
             t32[t].y = (float)im[t];
         }
@@ -1172,7 +1172,7 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
             i64v[b] = 1.0 / (double)h->ns[b];
             i32v[b] = (float)i64v[b];
         }
-        cpx<double>* p64 = nullptr;
+        fxw* p64 = nullptr;
         cpx<float>* p32 = nullptr;
         double *qq64 = nullptr, *ll64 = nullptr, *cc64 = nullptr, *ii64 = nullptr;
         float *qq32 = nullptr, *ll32 = nullptr, *cc32 = nullptr, *ii32 = nullptr;
@@ -1214,10 +1214,11 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
     const int ncolitems = B * h->d.nkx;
     for (int pr = 0; pr < 2; ++pr) {
         const size_t cs = pr == P64 ? sizeof(cpx<double>) : sizeof(cpx<float>);
-        const size_t tw_bytes = (size_t)std::max(h->d.nx, h->nsmax) * cs;  // compact table
+        const int nm = std::max(h->d.nx, h->nsmax);
+        const size_t tw_bytes = pr == P64 ? twiddle_bytes<double>(nm, true) : twiddle_bytes<float>(nm, true);
         Launch& lr = h->lrow[pr];
         lr.threads = h->d.nx >= 256 ? 256 : 128;
-        lr.tw_off = (2 * (size_t)h->rows_per_tile * h->d.nx * cs + 15) & ~(size_t)15;
+        lr.tw_off = 2 * (size_t)h->rows_per_tile * h->d.nx * cs + row_extra_bytes(h->rows_per_tile);  // 16-aligned
         lr.smem = lr.tw_off + tw_bytes;
         lr.grid = 152 * 16;
         Launch& lc = h->lcol[pr];

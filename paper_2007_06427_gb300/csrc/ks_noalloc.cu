@@ -34,7 +34,7 @@ constexpr size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // byte offsets of the pieces inside the scratch array (sized for the maxima above)
 constexpr size_t O_TW = 0;
-constexpr size_t O_QV = O_TW + al(sizeof(cpx<double>) * NMAX);
+constexpr size_t O_QV = O_TW + al(sizeof(fxw) * FX_TABLE);
 constexpr size_t O_LIN = O_QV + al(sizeof(double) * NA_NKX);
 constexpr size_t O_CQ = O_LIN + al(sizeof(double) * NA_NKX);
 constexpr size_t O_SCAL = O_CQ + al(sizeof(double) * NA_NKX);  // insv, T[2], wT[2], J, dJdT, sqrtJ
@@ -97,15 +97,26 @@ __global__ void k_na_prep(unsigned char* base, double L, int nx, int ns, double 
     }
 }
 
+// the twiddles that transforms of length up to nm read, into shared memory after the item's buffers
+__device__ __forceinline__ void na_stage_twiddles(Bufs<double>& p, unsigned char* smem, int tw_off, int nm) {
+    cpx<double>* tws = reinterpret_cast<cpx<double>*>(smem + tw_off);
+    load_twiddles(tws, p.tw, nm);
+    cp_async_wait();
+    __syncthreads();
+    p.tw = tws;
+}
+
 template <int MODE>
-__global__ void __launch_bounds__(NA_THREADS) k_na_rows(Dims d, Bufs<double> p, int nitems) {
+__global__ void __launch_bounds__(NA_THREADS) k_na_rows(Dims d, Bufs<double> p, int nitems, int tw_off, int nm) {
     extern __shared__ __align__(16) unsigned char smem[];
+    na_stage_twiddles(p, smem, tw_off, nm);
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) row_item<double, MODE>(d, p, it, smem);
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(NA_THREADS) k_na_cols(Dims d, Bufs<double> p, int nitems) {
+__global__ void __launch_bounds__(NA_THREADS) k_na_cols(Dims d, Bufs<double> p, int nitems, int tw_off, int nm) {
     extern __shared__ __align__(16) unsigned char smem[];
+    na_stage_twiddles(p, smem, tw_off, nm);
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) col_item<double, MODE>(d, p, it, smem, 0);
 }
 
@@ -114,34 +125,6 @@ __global__ void k_na_finalize(int nkx, double L, const double* Jpart, double* J)
         double s = 0.0;
         for (int c = 0; c < nkx; ++c) s += Jpart[c];
         *J = L * s;
-    }
-}
-
-// host-side twiddles exp(2 pi i t / NMAX), octant symmetric (held in static host storage)
-void na_twiddles(cpx<double>* tw) {
-    const int N = NMAX;
-    const double two_pi = 6.283185307179586476925286766559;
-    static double c[NMAX / 4 + 1], s[NMAX / 4 + 1];
-    for (int t = 0; t <= N / 8; ++t) {
-        c[t] = std::cos(two_pi * t / N);
-        s[t] = std::sin(two_pi * t / N);
-    }
-    for (int t = N / 8 + 1; t <= N / 4; ++t) {
-        c[t] = s[N / 4 - t];
-        s[t] = c[N / 4 - t];
-    }
-    for (int t = 0; t < N; ++t) {
-        const int qd = t / (N / 4), r = t % (N / 4);
-        const double a = c[r], b = s[r];
-        double re, im;
-        switch (qd) {
-            case 0: re = a; im = b; break;
-            case 1: re = -b; im = a; break;
-            case 2: re = -a; im = -b; break;
-            default: re = b; im = -a; break;
-        }
-        tw[t].x = re;
-        tw[t].y = im;
     }
 }
 
@@ -210,12 +193,12 @@ int na_setup(int dev, unsigned char** base) {
         cudaGetLastError();
         return na_fail(KS_ERR_CUDA, "cudaGetSymbolAddress of the scratch array failed");
     }
-    static cpx<double> tw[NMAX];
-    na_twiddles(tw);
-    e = cudaMemcpy(static_cast<unsigned char*>(ptr) + O_TW, tw, sizeof(tw), cudaMemcpyHostToDevice);
+    const std::vector<fxw> tw = fx_table();
+    e = cudaMemcpy(static_cast<unsigned char*>(ptr) + O_TW, tw.data(), tw.size() * sizeof(fxw), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return na_fail(KS_ERR_CUDA, "twiddle upload failed");
-    const int rs = (int)(2 * NA_ROWS * NA_NXMAX * sizeof(cpx<double>));
-    const int cs = (int)(2 * NA_NSMAX * sizeof(cpx<double>) + COL_RED_DOUBLES * sizeof(double));
+    const int rs = (int)(2 * NA_ROWS * NA_NXMAX * sizeof(cpx<double>) + row_extra_bytes(NA_ROWS) + twiddle_bytes<double>(NA_NSMAX, true));
+    const int cs = (int)(2 * NA_NSMAX * sizeof(cpx<double>) + COL_RED_DOUBLES * sizeof(double) +
+                         twiddle_bytes<double>(NA_NSMAX, true));
     if (cudaFuncSetAttribute(k_na_rows<ROW_ANALYZE>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs) ||
         cudaFuncSetAttribute(k_na_rows<ROW_NONLIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs) ||
         cudaFuncSetAttribute(k_na_rows<ROW_SYNTH>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs) ||
@@ -318,21 +301,22 @@ extern "C" int ks_residual_noalloc(double L, int nx, int ns, const double* u, do
 
     const int nrow = ns / NA_ROWS;
     const int ncol = d.nkx;
-    const size_t rs = 2 * (size_t)NA_ROWS * nx * sizeof(cpx<double>);
-    const size_t cs = 2 * (size_t)ns * sizeof(cpx<double>) + COL_RED_DOUBLES * sizeof(double);
+    const int rt = (int)(2 * (size_t)NA_ROWS * nx * sizeof(cpx<double>) + row_extra_bytes(NA_ROWS));
+    const int ct = (int)(2 * (size_t)ns * sizeof(cpx<double>) + COL_RED_DOUBLES * sizeof(double));
+    const size_t rs = rt + twiddle_bytes<double>(nx, true), cs = ct + twiddle_bytes<double>(ns, true);
     k_na_prep<<<1, NA_THREADS, 0, s>>>(base, L, nx, ns, T);
     // project u onto the band (a4 applied to the input), then a1-a6 and the synthesis of r
     p.io = const_cast<double*>(u);
-    k_na_rows<ROW_ANALYZE><<<nrow, NA_THREADS, rs, s>>>(d, p, nrow);
-    k_na_cols<COL_ANALYZE><<<ncol, NA_THREADS, cs, s>>>(d, p, ncol);
-    k_na_cols<COL_SYNTH_U><<<ncol, NA_THREADS, cs, s>>>(d, p, ncol);
-    k_na_rows<ROW_NONLIN><<<nrow, NA_THREADS, rs, s>>>(d, p, nrow);
-    k_na_cols<COL_RESID><<<ncol, NA_THREADS, cs, s>>>(d, p, ncol);
+    k_na_rows<ROW_ANALYZE><<<nrow, NA_THREADS, rs, s>>>(d, p, nrow, rt, nx);
+    k_na_cols<COL_ANALYZE><<<ncol, NA_THREADS, cs, s>>>(d, p, ncol, ct, ns);
+    k_na_cols<COL_SYNTH_U><<<ncol, NA_THREADS, cs, s>>>(d, p, ncol, ct, ns);
+    k_na_rows<ROW_NONLIN><<<nrow, NA_THREADS, rs, s>>>(d, p, nrow, rt, nx);
+    k_na_cols<COL_RESID><<<ncol, NA_THREADS, cs, s>>>(d, p, ncol, ct, ns);
     k_na_finalize<<<1, 32, 0, s>>>(ncol, L, reinterpret_cast<const double*>(base + O_JP), J);
     if (r) {
         p.io = r;
-        k_na_cols<COL_SYNTH_R><<<ncol, NA_THREADS, cs, s>>>(d, p, ncol);
-        k_na_rows<ROW_SYNTH><<<nrow, NA_THREADS, rs, s>>>(d, p, nrow);
+        k_na_cols<COL_SYNTH_R><<<ncol, NA_THREADS, cs, s>>>(d, p, ncol, ct, ns);
+        k_na_rows<ROW_SYNTH><<<nrow, NA_THREADS, rs, s>>>(d, p, nrow, rt, nx);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return na_fail(KS_ERR_CUDA, cudaGetErrorString(e));
