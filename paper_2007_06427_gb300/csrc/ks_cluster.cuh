@@ -586,14 +586,14 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                                 const R bk = -(R)k * wTr;
                                 const cpx<R> pa = xi_split_a(ck, cm);
                                 const cpx<R> ua = uhl[(2 * pp) * nk + k + ks];
-                                const cpx<R> ra = mk<R>(lin_a * ua.x - bk * ua.y - pa.x, lin_a * ua.y + bk * ua.x - pa.y);
+                                const cpx<R> ra = symbol_add(lin_a, bk, ua, neg(pa));
                                 rhl[(2 * pp) * nk + k + ks] = ra;
                                 acc[0].add(ua, ra, k);
                                 cpx<R> xb = mk<R>(0, 0);
                                 if (hasb) {
                                     const cpx<R> pb = xi_split_b(ck, cm);
                                     const cpx<R> ub = uhl[(2 * pp + 1) * nk + k + ks];
-                                    const cpx<R> rb = mk<R>(lin_b * ub.x - bk * ub.y - pb.x, lin_b * ub.y + bk * ub.x - pb.y);
+                                    const cpx<R> rb = symbol_add(lin_b, bk, ub, neg(pb));
                                     rhl[(2 * pp + 1) * nk + k + ks] = rb;
                                     acc[1].add(ub, rb, k);
                                     xb = mk<R>(-q_b * rb.y, q_b * rb.x);
@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                                     const cpx<R> ph = Mloc[(q << lg) + n];
                                     const cpx<R> u = uhl[q * nk + k + ks];
                                     const R bk = -(R)k * wTr;
-                                    const cpx<R> r = mk<R>(a_lin * u.x - bk * u.y - ph.x, a_lin * u.y + bk * u.x - ph.y);
+                                    const cpx<R> r = symbol_add(a_lin, bk, u, neg(ph));
                                     rhl[q * nk + k + ks] = r;
                                     acc[t].add(u, r, k);
                                     x = mk<R>(-rq * r.y, rq * r.x);
@@ -787,17 +787,16 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                         const int ja = colj(2 * pp), jb = ja + 1;
                         const cpx<RA> ck = scr_a[i], cm = scr_a[(pp << lg) + ((ns - n) & (ns - 1))];
                         const RA bk = (RA)k * wTa;
-                        const R kk2 = (R)k * (R)k;
                         auto update = [&](int q, int j, cpx<RA> wh) {
                             const RA a_lin = s_lina[j];
                             const cpx<R> rr = rhl[q * nk + k + ks];
                             const cpx<RA> r = mk<RA>((RA)rr.x, (RA)rr.y);
-                            const cpx<RA> Ga = mk<RA>(a_lin * r.x - bk * r.y + wh.x, a_lin * r.y + bk * r.x + wh.y);
+                            const cpx<RA> Ga = symbol_add(a_lin, bk, r, wh);
                             const cpx<R> G = mk<R>((R)Ga.x, (R)Ga.y);
                             R f = dt;
-                            if (d.scheme == 1) f = dt / ((R)1 + dt * (kk2 * wT2 + s_cq[j]));
+                            if (d.scheme == 1) f = imex_factor(dt, k, wT2, s_cq[j]);
                             cpx<R> u = uhl[q * nk + k + ks];
-                            u = u - scale(G, f);
+                            u = step_along(u, G, f);
                             uhl[q * nk + k + ks] = u;
                             return u;
                         };
@@ -821,7 +820,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     const cpx<R> rr = rhl[q * nk + k + ks];
                     const cpx<RA> r = mk<RA>((RA)rr.x, (RA)rr.y);
                     const RA bk = (RA)k * wTa;
-                    const cpx<RA> G = mk<RA>(a_lin * r.x - bk * r.y + wh.x, a_lin * r.y + bk * r.x + wh.y);
+                    const cpx<RA> G = symbol_add(a_lin, bk, r, wh);
                     return mk<R>((R)G.x, (R)G.y);
                 };
                 // double state with more than one element per thread: the band by (k, -k) pairs,
@@ -836,15 +835,12 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     for (int i = wtid; i < ncol * nh; i += ntw) {
                         const int q = i / nh, k = i - q * nh;
                         R f = dt;
-                        if (d.scheme == 1) {
-                            const R kk2 = (R)k * (R)k;
-                            f = dt / ((R)1 + dt * (kk2 * wT2 + s_cq[rank + q * C]));
-                        }
+                        if (d.scheme == 1) f = imex_factor(dt, k, wT2, s_cq[rank + q * C]);
                         auto upd = [&](int kk, int n) {
                             const int e = (q << lg) + n;
                             const cpx<R> G = g_hat(e, q, kk);
                             cpx<R> u = uhl[q * nk + kk + ks];
-                            u = u - scale(G, f);
+                            u = step_along(u, G, f);
                             uhl[q * nk + kk + ks] = u;
                             scr[e] = u;
                         };
@@ -865,12 +861,9 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                             const int j = rank + q * C;
                             const cpx<R> G = g_hat(i, q, k);
                             R f = dt;
-                            if (d.scheme == 1) {
-                                const R kk2 = (R)k * (R)k;
-                                f = dt / ((R)1 + dt * (kk2 * wT2 + s_cq[j]));
-                            }
+                            if (d.scheme == 1) f = imex_factor(dt, k, wT2, s_cq[j]);
                             cpx<R> u = uhl[q * nk + k + ks];
-                            u = u - scale(G, f);
+                            u = step_along(u, G, f);
                             uhl[q * nk + k + ks] = u;
                             x = u;
                         }

@@ -74,26 +74,62 @@ template <typename R>
 KS_HD cpx<R> operator+(cpx<R> a, cpx<R> b) { return mk<R>(a.x + b.x, a.y + b.y); }
 template <typename R>
 KS_HD cpx<R> operator-(cpx<R> a, cpx<R> b) { return mk<R>(a.x - b.x, a.y - b.y); }
+// fused multiply-add a * b + c with one rounding, in either precision
+KS_HD double fmx(double a, double b, double c) { return fma(a, b, c); }
+KS_HD float fmx(float a, float b, float c) { return fmaf(a, b, c); }
+// a * b rounded, never fused into an addition that follows
+KS_HD float mul_rn(float a, float b) {
+#ifdef KS_HOST_EMULATION
+    return a * b;
+#else
+    return __fmul_rn(a, b);
+#endif
+}
+KS_HD double mul_rn(double a, double b) {
+#ifdef KS_HOST_EMULATION
+    return a * b;
+#else
+    return __dmul_rn(a, b);
+#endif
+}
+// The products below fuse explicitly: left to the compiler, which of two products a sum fuses can
+// differ from kernel to kernel, and the launch forms would no longer agree bit for bit.
 template <typename R>
 KS_HD cpx<R> cmul(cpx<R> a, cpx<R> b) {
-    return mk<R>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+    return mk<R>(fmx(a.x, b.x, -mul_rn(a.y, b.y)), fmx(a.x, b.y, mul_rn(a.y, b.x)));
 }
 template <typename R>
 KS_HD cpx<R> conj(cpx<R> a) { return mk<R>(a.x, -a.y); }
+template <typename R>
+KS_HD cpx<R> neg(cpx<R> a) { return mk<R>(-a.x, -a.y); }
 template <typename R>
 KS_HD cpx<R> scale(cpx<R> a, R s) { return mk<R>(a.x * s, a.y * s); }
 // multiply by i*sgn (sgn = +1 or -1)
 template <typename R>
 KS_HD cpx<R> mul_i(cpx<R> a, int sgn) { return sgn > 0 ? mk<R>(-a.y, a.x) : mk<R>(a.y, -a.x); }
 
-// fused multiply-add a * b + c with one rounding, in either precision
-KS_HD double fmx(double a, double b, double c) { return fma(a, b, c); }
-KS_HD float fmx(float a, float b, float c) { return fmaf(a, b, c); }
-
 // v0 + w v (complex) as four fused multiply-adds
 template <typename R>
 KS_HD cpx<R> cfma(cpx<R> v0, cpx<R> w, cpx<R> v) {
     return mk<R>(fmx(w.x, v.x, fmx(-w.y, v.y, v0.x)), fmx(w.x, v.y, fmx(w.y, v.x, v0.y)));
+}
+
+// (a + i b) v + c (complex): r_hat with c = -p_hat and b = -omega_k / T, G_hat with c = w_hat and
+// b = omega_k / T
+template <typename R>
+KS_HD cpx<R> symbol_add(R a, R b, cpx<R> v, cpx<R> c) {
+    return mk<R>(fmx(a, v.x, -mul_rn(b, v.y)) + c.x, fmx(a, v.y, mul_rn(b, v.x)) + c.y);
+}
+// u - f G
+template <typename R>
+KS_HD cpx<R> step_along(cpx<R> u, cpx<R> G, R f) {
+    return mk<R>(fmx(-f, G.x, u.x), fmx(-f, G.y, u.y));
+}
+// dtau / (1 - dtau Lambda), Lambda = -(k omega/T)^2 - q^4 (q^2 - 1)^2 (wT2 = (2 pi / T)^2, cq the x part)
+template <typename R>
+KS_HD R imex_factor(R dt, int k, R wT2, R cq) {
+    const R kk2 = (R)k * (R)k;
+    return dt / fmx(dt, fmx(kk2, wT2, cq), (R)1);
 }
 
 // 2 a - b (complex) as two fused multiply-adds
@@ -143,7 +179,7 @@ KS_HD ff ff_add(ff a, ff b) {
     return two_sum(s.hi, e);
 }
 KS_HD ff two_prod(float a, float b) {
-    const float p = a * b;
+    const float p = mul_rn(a, b);
     ff r;
     r.hi = p;
     r.lo = fmaf(a, b, -p);
@@ -168,8 +204,8 @@ template <>
 struct ColAcc<double> {
     double J = 0.0, L = 0.0;
     KS_HD void add(cpx<double> u, cpx<double> r, int k) {
-        J += r.x * r.x + r.y * r.y;
-        L += (double)k * (u.x * r.y - u.y * r.x);
+        J += fmx(r.x, r.x, mul_rn(r.y, r.y));
+        L = fmx((double)k, fmx(u.x, r.y, -mul_rn(u.y, r.x)), L);
     }
     KS_HD double part_J(double wj) const { return wj * J; }
     KS_HD double part_L(double wj) const { return wj * L; }
@@ -1354,14 +1390,14 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
                     // r_hat = (a + i bk) u_hat - p_hat for both columns                     (a5)
                     const cpx<R> pa = scale(xi_split_a(ck, cm), ins);
                     const cpx<R> ua = p.uh[ba + (k + ks)];
-                    const cpx<R> ra = mk<R>(lin_a * ua.x - bk * ua.y - pa.x, lin_a * ua.y + bk * ua.x - pa.y);
+                    const cpx<R> ra = symbol_add(lin_a, bk, ua, neg(pa));
                     p.rh[ba + (k + ks)] = ra;
                     if (fused) acc[0].add(ua, ra, k);         // a6
                     cpx<R> xb = zero;
                     if (hasb) {
                         const cpx<R> pb = scale(xi_split_b(ck, cm), ins);
                         const cpx<R> ub = p.uh[bb + (k + ks)];
-                        const cpx<R> rb = mk<R>(lin_b * ub.x - bk * ub.y - pb.x, lin_b * ub.y + bk * ub.x - pb.y);
+                        const cpx<R> rb = symbol_add(lin_b, bk, ub, neg(pb));
                         p.rh[bb + (k + ks)] = rb;
                         if (fused) acc[1].add(ub, rb, k);
                         xb = mk<R>(-q_b * rb.y, q_b * rb.x);   // i q_j r_hat                 (a7)
@@ -1409,7 +1445,7 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
             const cpx<R> r = p.rh[(second ? bb : ba) + (k + ks)];
             const R a_lin = second ? lin_b : lin_a;
             const R bk = (R)k * w_over_T;
-            return mk<R>(a_lin * r.x - bk * r.y + wh.x, a_lin * r.y + bk * r.x + wh.y);
+            return symbol_add(a_lin, bk, r, wh);
         };
 
         if constexpr (MODE == COL_GRAD) {
@@ -1440,17 +1476,16 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
                     R fa = dt, fb = dt;
                     if (d.scheme == 1) {
                         // IMEX: dtau / (1 - dtau Lambda), Lambda = -(omega/T)^2 - q^4 (q^2-1)^2  (a10)
-                        const R kk2 = (R)k * (R)k;
-                        fa = dt / ((R)1 + dt * (kk2 * wT2 + cq_a));
-                        fb = dt / ((R)1 + dt * (kk2 * wT2 + cq_b));
+                        fa = imex_factor(dt, k, wT2, cq_a);
+                        fb = imex_factor(dt, k, wT2, cq_b);
                     }
                     cpx<R> ua = p.uh[ba + (k + ks)];
-                    ua = ua - scale(g_at(i, k, false), fa);
+                    ua = step_along(ua, g_at(i, k, false), fa);
                     p.uh[ba + (k + ks)] = ua;
                     cpx<R> ub = zero;
                     if (hasb) {
                         ub = p.uh[bb + (k + ks)];
-                        ub = ub - scale(g_at(i, k, true), fb);
+                        ub = step_along(ub, g_at(i, k, true), fb);
                         p.uh[bb + (k + ks)] = ub;
                     }
                     x = xi_join_imag(ua, ub);
@@ -1554,7 +1589,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                     const cpx<R> u = p.uh[bo + (k + ks)];
                     const R bk = -(R)k * w_over_T;            // -omega_k / T
                     // r_hat = (a + i bk) u_hat - p_hat                                    (a5)
-                    const cpx<R> r = mk<R>(a_lin * u.x - bk * u.y - ph.x, a_lin * u.y + bk * u.x - ph.y);
+                    const cpx<R> r = symbol_add(a_lin, bk, u, neg(ph));
                     p.rh[bo + (k + ks)] = r;
                     if (fused) acc.add(u, r, k);              // a6: |r|^2, k Im(conj(u) r)
                     x = mk<R>(-rq * r.y, rq * r.x);           // i q_j r_hat                 (a7)
@@ -1582,7 +1617,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                     const cpx<R> wh = scale(F[i], ins);
                     const cpx<R> r = p.rh[bo + (k + ks)];
                     const R bk = (R)k * w_over_T;             // +omega_k / T
-                    const cpx<R> G = mk<R>(a_lin * r.x - bk * r.y + wh.x, a_lin * r.y + bk * r.x + wh.y);
+                    const cpx<R> G = symbol_add(a_lin, bk, r, wh);
                     if (p.xi) X[i] = G;
                     else p.gh[bo + (k + ks)] = G;
                 }
@@ -1613,7 +1648,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                         const cpx<R> wh = scale(F[i], ins);
                         const cpx<R> r = p.rh[bo + (k + ks)];
                         const R bk = (R)k * w_over_T;
-                        X[i] = mk<R>(a_lin * r.x - bk * r.y + wh.x, a_lin * r.y + bk * r.x + wh.y);
+                        X[i] = symbol_add(a_lin, bk, r, wh);
                     }
                 }
                 KS_SYNC();
@@ -1632,16 +1667,15 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                         const cpx<R> r = p.rh[bo + (k + ks)];
                         const R bk = (R)k * w_over_T;
                         // G_hat = (a + i omega/T) r_hat + F[P(u r_x)]                      (a9)
-                        G = mk<R>(a_lin * r.x - bk * r.y + wh.x, a_lin * r.y + bk * r.x + wh.y);
+                        G = symbol_add(a_lin, bk, r, wh);
                     }
                     R f = dt;
                     if (d.scheme == 1) {
                         // IMEX: dtau / (1 - dtau Lambda), Lambda = -(omega/T)^2 - q^4 (q^2-1)^2  (a10)
-                        const R kk2 = (R)k * (R)k;
-                        f = dt / ((R)1 + dt * (kk2 * wT2 + cqj));
+                        f = imex_factor(dt, k, wT2, cqj);
                     }
                     cpx<R> u = p.uh[bo + (k + ks)];
-                    u = u - scale(G, f);
+                    u = step_along(u, G, f);
                     p.uh[bo + (k + ks)] = u;
                     x = u;
                 }

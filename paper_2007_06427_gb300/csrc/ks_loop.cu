@@ -17,6 +17,7 @@
 #include "ks_cluster.cuh"
 #include "ks_items.cuh"
 #include "ks_loop.h"
+#include "ks_reg.cuh"
 
 using namespace ks;
 
@@ -336,6 +337,12 @@ struct ks_loop {
     Work st;   // resident descent state
     Work api;  // scratch for ks_residual / ks_adjoint_grad
     Launch lrow[2], lcol[2];
+    // float phases with the transforms in registers (ks_reg.cuh): tiles, or none where a length is
+    // not covered
+    int rg_nrow = 0, rg_ncol = 0, rg_ntab = 0;
+    RgTile* d_rg_rows = nullptr;
+    RgCol* d_rg_cols = nullptr;
+    rgv* d_rg_tab = nullptr;
     bool state_set = false;
     std::vector<void*> allocs;
     // profiling: per-kind event pairs around every launch when enabled
@@ -569,9 +576,81 @@ struct LaunchScope {
 
 std::string prec_suffix(int pr) { return pr == 0 ? "_f64" : "_f32"; }
 
+// The float phases of a step take the register kernels wherever their lengths are covered, except
+// in the centre-symmetric subspace (whose transforms pair rows and columns differently).  The two
+// row phases agree on the layout of U, so they must come from the same family: the choice depends
+// on nothing that changes between them.
+bool use_rg(const ks_loop* h) { return h->rg_nrow > 0 && !h->xi; }
+
+template <int MODE>
+int launch_rg_rows(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
+    const int n = h->rg_nrow, per = RG_THREADS / 32, g = (n + per - 1) / per;
+    LaunchScope ls(h, s, std::string(kRowNames[MODE]) + prec_suffix(P32));
+    switch (h->d.lgnx) {
+    case 5: k_rg_rows<MODE, 5><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
+    case 6: k_rg_rows<MODE, 6><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
+    case 7: k_rg_rows<MODE, 7><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
+    case 8: k_rg_rows<MODE, 8><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
+    default: k_rg_rows<MODE, 9><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
+    }
+    KS_CUDA(cudaGetLastError());
+    ls.done();
+    return KS_OK;
+}
+
+template <int MODE>
+int launch_rg_cols(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
+    const int n = h->rg_ncol, per = RG_THREADS / 64, g = (n + per - 1) / per;
+    LaunchScope ls(h, s, std::string(kColNames[MODE]) + prec_suffix(P32));
+    const size_t smem = (size_t)h->rg_ntab * sizeof(rgv) + (size_t)per * RG_XBYTES;
+    k_rg_cols<MODE><<<g, RG_THREADS, smem, s>>>(h->d, p, h->d_rg_cols, n, h->d_rg_tab, h->rg_ntab);
+    KS_CUDA(cudaGetLastError());
+    ls.done();
+    return KS_OK;
+}
+
+// Tiles and twiddles of the register kernels: row lengths 32 .. 512, column lengths 32 .. 1024.
+int setup_rg(ks_loop* h) {
+    const int nx = h->d.nx;
+    if (nx < 32 || nx > 512) return KS_OK;
+    for (int n : h->ns)
+        if (n < 32) return KS_OK;
+    std::vector<RgTile> rows;
+    const int step = 1024 / nx;  // 2 F rows, F = 32 / (nx / 16) pairs a warp
+    for (int b = 0; b < h->d.B; ++b)
+        for (int n0 = 0; n0 < h->ns[b]; n0 += step) rows.push_back(RgTile{b, n0});
+    std::vector<RgCol> cols;  // in colorder: the 1024-point loops come first
+    for (int b : h->colorder) {
+        const int F = std::max(1, 512 / h->ns[b]);
+        for (int j = 0; j < h->d.nkx; j += F) {
+            cols.push_back(RgCol{b, j});
+            if (h->ns[b] == 1024) cols.push_back(RgCol{-1, 0});
+        }
+    }
+    if (cols.size() & 1) cols.push_back(RgCol{-1, 0});
+    std::vector<rgv> tab(RG_TABLE);
+    std::vector<double> re, im;
+    twiddles(re, im);
+    for (int lg = 5; lg <= LGNMAX; ++lg)
+        for (int e = 0; e < rg_len(lg); ++e) {
+            int t, m;
+            rg_entry(lg, e, t, m);
+            tab[rg_at(lg) + e] = rgv{(float)re[t * (NMAX / m)], (float)im[t * (NMAX / m)]};
+        }
+    KS_TRY(upload(h, &h->d_rg_rows, rows));
+    KS_TRY(upload(h, &h->d_rg_cols, cols));
+    KS_TRY(upload(h, &h->d_rg_tab, tab));
+    h->rg_nrow = (int)rows.size();
+    h->rg_ncol = (int)cols.size() / 2;
+    h->rg_ntab = rg_at(ilog2(h->nsmax) + 1);
+    return KS_OK;
+}
+
 template <typename R, int MODE>
 int launch_rows(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const int pr = std::is_same<R, double>::value ? P64 : P32;
+    if constexpr (std::is_same<R, float>::value && (MODE == ROW_NONLIN || MODE == ROW_ADJ))
+        if (use_rg(h)) return launch_rg_rows<MODE>(h, p, s);
     const Launch& l = h->lrow[pr];
     const int n = (int)h->rows.size();
     LaunchScope ls(h, s, std::string(kRowNames[MODE]) + prec_suffix(pr));
@@ -585,6 +664,8 @@ int launch_rows(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
 template <typename R, int MODE>
 int launch_cols(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const int pr = std::is_same<R, double>::value ? P64 : P32;
+    if constexpr (std::is_same<R, float>::value && (MODE == COL_RESID || MODE == COL_UPDATE))
+        if (use_rg(h)) return launch_rg_cols<MODE>(h, p, s);
     const Launch& l = h->lcol[pr];
     const int n = col_item_count(h->d, h->xi, MODE);
     LaunchScope ls(h, s, std::string(kColNames[MODE]) + prec_suffix(pr));
@@ -1228,6 +1309,7 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
         lc.grid = 152 * 16;
     }
     if ((rc = set_smem_attrs<double>(h)) || (rc = set_smem_attrs<float>(h))) return cleanup(rc);
+    if (h->need[P32] && (rc = setup_rg(h))) return cleanup(rc);
     if ((rc = setup_persistent<double>(h)) || (rc = setup_persistent<float>(h))) return cleanup(rc);
     if ((rc = setup_cluster<double, double>(h)) || (rc = setup_cluster<float, float>(h)) ||
         (h->mode == KS_MIXED && (rc = setup_cluster<double, float>(h))))
