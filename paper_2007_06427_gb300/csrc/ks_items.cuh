@@ -288,6 +288,15 @@ struct Bufs {
     int own_frozen_only;    // cluster kernel: 1 = carry T forward only for frozen loops of this
                             // precision (the other precision's launch runs concurrently and
                             // carries its own)
+    // the launches at the boundary of a call carry its small duties with them:
+    const double* Tin;      // ROW_ANALYZE: periods to install (T, 2 pi / T at parity 0), or null
+    int* prec_out;          // ROW_ANALYZE with Tin: fresh descent state (status, steps, sqrtJ zero, this
+    int prec_new;           // precision), or null
+    const float* iof;       // ROW_ANALYZE, double: float grid to analyse in place of io, or null
+    cpx<float>* uhf;        // COL_ANALYZE: band rounded to float, stored in place of uh, or null
+    int fin;                // ROW_SYNTH: 1: also form J, dJ/dT and sqrt(J) from the column partials
+    double* Jout;           // [B] (fin), each nullable
+    double* dJdTout;
     int step_scalars;       // 1 (tau-steps): the ROW_ADJ launch forms each running loop's step
                             // scalars (loop_scalars, loops_scalars) for the COL_UPDATE items
                             // that follow
@@ -977,6 +986,20 @@ KS_HD void loop_scalars(const Dims& d, const Bufs<R>& p, int b, int par) {
     }
 }
 
+// J = L sum_j Jpart and dJ/dT = 2 L^dag_2 = 2 (2 pi L / T^2) sum_j L2part of loop b, by one warp.
+template <typename P>
+KS_HD void loop_costs(const P* Jpart, const P* L2part, int nkx, double L, double T, double* J,
+                      double* dJdT, double* sqrtJ) {
+    double sj, sl;
+    sum_partials(Jpart, L2part, nkx, sj, sl);
+    if ((KS_TID & 31) == 0) {
+        const double Jb = L * sj;
+        if (J) *J = Jb;
+        if (dJdT) *dJdT = 2.0 * L * 2.0 * 3.14159265358979323846 * sl / (T * T);
+        if (sqrtJ) *sqrtJ = sqrt(Jb);
+    }
+}
+
 // is the loop processed by this kernel set?
 template <typename R>
 KS_HD bool loop_live(const Bufs<R>& p, int b) {
@@ -1096,8 +1119,13 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
         for (int i = KS_TID; i < total; i += KS_NT) {
             const int pr = i >> lgnx;
             const int m = i & (nx - 1);
-            const R* ra = Ib + (size_t)(n0 + 2 * pr) * nx;
-            A[i] = mk<R>(ra[m], ra[nx + m]);
+            const size_t at = (size_t)(n0 + 2 * pr) * nx + m;
+            if (sizeof(R) == 8 && p.iof) {
+                const float* ra = p.iof + p.goff[b] + at;
+                A[i] = mk<R>((R)ra[0], (R)ra[nx]);
+            } else {
+                A[i] = mk<R>(Ib[at], Ib[at + nx]);
+            }
         }
         KS_SYNC();
         cpx<R>* Y = fft_any<R, kHot, SWZ, false, true>(A, Bf, lgnx, npairs, -1, p.tw, sc, 0, p.twsh);
@@ -1238,8 +1266,16 @@ enum ColMode {
     COL_SYNTH_G = 3,  // band G_hat -> M
     COL_RESID = 4,    // M = P -> r_hat, partials, M = s-inverse of i q r_hat
     COL_UPDATE = 5,   // M = W -> G_hat, update u_hat and T, M = s-inverse of new u_hat
-    COL_GRAD = 6      // M = W -> G_hat band (no update)
+    COL_GRAD = 6,     // M = W -> G_hat band (no update)
+    // the column phases of ks_residual and ks_adjoint_grad outside the subspace, where two that
+    // follow one another on the same column are one
+    COL_ANALYZE_U = 7,  // COL_ANALYZE, then COL_SYNTH_U
+    COL_RESID_R = 8,    // r_hat and partials of COL_RESID, then COL_SYNTH_R (in place of i q r_hat's inverse)
+    COL_RESID_J = 9,    // r_hat and partials alone
+    COL_GRAD_G = 10     // COL_GRAD, then COL_SYNTH_G
 };
+KS_HDX constexpr bool col_resid(int MODE) { return MODE == COL_RESID || MODE == COL_RESID_R || MODE == COL_RESID_J; }
+KS_HDX constexpr bool col_grad(int MODE) { return MODE == COL_GRAD || MODE == COL_GRAD_G; }
 
 // Shared-memory bytes a column item needs beyond its two transform buffers.
 constexpr int COL_RED_SC = 4 * (256 / 32 + 1);       // block sums of up to 256 threads, then the
@@ -1530,7 +1566,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
     const double* wTc = p.wT + (size_t)par * B;
     double* wTn = p.wT + (size_t)(par ^ 1) * B;
 
-    if constexpr (MODE == COL_RESID || MODE == COL_GRAD) {
+    if constexpr (col_resid(MODE) || col_grad(MODE)) {
         if (!loop_live(p, b)) return;
     }
     if constexpr (MODE == COL_UPDATE) {
@@ -1567,8 +1603,29 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                 const int k = kk - ks;
                 cpx<R> v = scale(F[k & (ns - 1)], ins);
                 if (p.xi) v = (j == 0) ? mk<R>(0, 0) : xi_pair(v, scale(F[(-k) & (ns - 1)], ins));
-                p.uh[bo + kk] = v;
+                if (p.uhf) p.uhf[bo + kk] = mk<float>((float)v.x, (float)v.y);
+                else p.uh[bo + kk] = v;
             }
+            KS_SYNC();
+            return;
+        }
+        // the inverse s-transform of the spectrum in X to the column of M
+        auto back = [&](cpx<R>* Y, cpx<R>* other) {
+            KS_SYNC();
+            const cpx<R>* v = fft_any<R, kHot, SWZ>(Y, other, lg, 1, +1, p.tw, sc, 0, p.twsh);
+            for (int i = KS_TID; i < ns; i += KS_NT) col[i] = v[i];
+        };
+        if constexpr (MODE == COL_ANALYZE_U) {
+            for (int i = KS_TID; i < ns; i += KS_NT) {
+                const int k = (i < (ns >> 1)) ? i : i - ns;
+                cpx<R> v = mk<R>(0, 0);
+                if (k >= -ks && k <= ks) {
+                    v = scale(F[i], ins);
+                    p.uh[bo + (k + ks)] = v;
+                }
+                X[i] = v;
+            }
+            back(X, F);
             KS_SYNC();
             return;
         }
@@ -1578,7 +1635,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
         const R rq = p.qv[j];
         const double wj = (j == 0) ? 1.0 : 2.0;  // x-conjugate pairs counted twice
 
-        if constexpr (MODE == COL_RESID) {
+        if constexpr (col_resid(MODE)) {
             ColAcc<R> acc;
             const bool fused = KS_ACC_FUSED;
             for (int i = KS_TID; i < ns; i += KS_NT) {
@@ -1592,7 +1649,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                     const cpx<R> r = symbol_add(a_lin, bk, u, neg(ph));
                     p.rh[bo + (k + ks)] = r;
                     if (fused) acc.add(u, r, k);              // a6: |r|^2, k Im(conj(u) r)
-                    x = mk<R>(-rq * r.y, rq * r.x);           // i q_j r_hat                 (a7)
+                    x = MODE == COL_RESID_R ? r : mk<R>(-rq * r.y, rq * r.x);  // i q_j r_hat    (a7)
                 }
                 X[i] = x;
             }
@@ -1602,26 +1659,29 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                     const int k = (i < (ns >> 1)) ? i : i - ns;
                     if (k >= -ks && k <= ks) acc.add(p.uh[bo + (k + ks)], p.rh[bo + (k + ks)], k);
                 }
-            cpx<R>* v = fft_any<R, kHot, SWZ>(X, F, lg, 1, +1, p.tw, sc, 0, p.twsh);
-            for (int i = KS_TID; i < ns; i += KS_NT) col[i] = v[i];
+            if constexpr (MODE != COL_RESID_J) back(X, F);
             block_reduce(acc, red);
             if (KS_TID == 0) {
                 p.Jpart[(size_t)b * nkx + j] = acc.part_J(wj);
                 p.L2part[(size_t)b * nkx + j] = acc.part_L(wj);
             }
             KS_SYNC();
-        } else if constexpr (MODE == COL_GRAD) {
+        } else if constexpr (col_grad(MODE)) {
             for (int i = KS_TID; i < ns; i += KS_NT) {
                 const int k = (i < (ns >> 1)) ? i : i - ns;
+                cpx<R> x = mk<R>(0, 0);
                 if (k >= -ks && k <= ks) {
                     const cpx<R> wh = scale(F[i], ins);
                     const cpx<R> r = p.rh[bo + (k + ks)];
                     const R bk = (R)k * w_over_T;             // +omega_k / T
                     const cpx<R> G = symbol_add(a_lin, bk, r, wh);
                     if (p.xi) X[i] = G;
-                    else p.gh[bo + (k + ks)] = G;
+                    else if constexpr (MODE == COL_GRAD) p.gh[bo + (k + ks)] = G;
+                    x = G;
                 }
+                if constexpr (MODE == COL_GRAD_G) X[i] = x;
             }
+            if constexpr (MODE == COL_GRAD_G) back(X, F);
             KS_SYNC();
             if (p.xi) {
                 // gradient within the Xi subspace: the projected G_hat

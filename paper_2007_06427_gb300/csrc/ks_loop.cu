@@ -46,6 +46,27 @@ template <typename R, int MODE>
 __global__ void __launch_bounds__(256) k_rows(Dims d, Bufs<R> p, int nitems, int tw_off, int nm) {
     extern __shared__ __align__(16) unsigned char smem[];
     const Bufs<R> q = stage_twiddles(p, smem, tw_off, nm);
+    if constexpr (MODE == ROW_ANALYZE) {
+        if (p.Tin)
+            for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < d.B; b += gridDim.x * blockDim.x) {
+                const double T = p.Tin[b];
+                p.T[b] = T;
+                p.wT[b] = 2.0 * 3.14159265358979323846 / T;
+                if (p.prec_out) {
+                    p.status[b] = 0;
+                    p.steps[b] = 0;
+                    p.sqrtJ[b] = 0.0;
+                    p.prec_out[b] = p.prec_new;
+                }
+            }
+    }
+    if constexpr (MODE == ROW_SYNTH) {
+        // loop b on block b mod blocks, its last warp: the partials are complete
+        if (p.fin && (int)threadIdx.x >= (int)blockDim.x - 32)
+            for (int b = blockIdx.x; b < d.B; b += gridDim.x)
+                loop_costs(p.Jpart + (size_t)b * d.nkx, p.L2part + (size_t)b * d.nkx, d.nkx, d.L, p.T[b],
+                           p.Jout ? p.Jout + b : nullptr, p.dJdTout ? p.dJdTout + b : nullptr, nullptr);
+    }
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) row_item<R, MODE, true>(d, q, it, smem);
     if constexpr (MODE == ROW_ADJ) loops_scalars(d, q, q.par, blockIdx.x, gridDim.x);
 }
@@ -55,13 +76,6 @@ __global__ void __launch_bounds__(256) k_cols(Dims d, Bufs<R> p, int nitems, int
     extern __shared__ __align__(16) unsigned char smem[];
     const Bufs<R> q = stage_twiddles(p, smem, tw_off, nm);
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) col_item<R, MODE, true>(d, q, it, smem, q.par);
-}
-
-// float grid -> double grid
-__global__ void k_grid_f2d(const float* src, double* dst, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        dst[i] = (double)src[i];
 }
 
 // double band -> float band (every loop)
@@ -174,25 +188,17 @@ __global__ void __launch_bounds__(128, 6) k_persist(Dims d, Bufs<R> p, int nstep
     }
 }
 
-// J = L sum_j Jpart, dJ/dT = 2 L^dag_2 = 2 (2 pi L / T^2) sum_j L2part, per loop.
-// only loops with prec[b] == myprec are written when mask != 0.
+// J, dJ/dT and sqrt(J) of every loop (loop_costs), a warp per loop; only loops with
+// prec[b] == myprec are written when mask != 0.
 template <typename P>
 __global__ void k_finalize(int B, int nkx, double L, const P* Jpart, const P* L2part,
                            const double* T, const int* prec, int myprec, int mask, double* J,
                            double* dJdT, double* sqrtJ) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (b >= B) return;
     if (mask && prec[b] != myprec) return;
-    double sj = 0.0, sl = 0.0;
-    for (int c = 0; c < nkx; ++c) {
-        sj += widen(Jpart[(size_t)b * nkx + c]);
-        sl += widen(L2part[(size_t)b * nkx + c]);
-    }
-    const double Tb = T[b];
-    const double Jb = L * sj;
-    if (J) J[b] = Jb;
-    if (dJdT) dJdT[b] = 2.0 * L * 2.0 * 3.14159265358979323846 * sl / (Tb * Tb);
-    if (sqrtJ) sqrtJ[b] = sqrt(Jb);
+    loop_costs(Jpart + (size_t)b * nkx, L2part + (size_t)b * nkx, nkx, L, T[b], J ? J + b : nullptr,
+               dJdT ? dJdT + b : nullptr, sqrtJ ? sqrtJ + b : nullptr);
 }
 
 // float band -> double band for the loops flagged in sel[b] (mixed-precision switch).
@@ -263,6 +269,7 @@ struct Work {
     int* sel = nullptr;        // [B] selection flags (switch)
     int par = 0;
     bool mix_valid[2] = {false, false};
+    bool loaded = false;  // M was primed by the load of the state, under the symmetry knob of then
 };
 
 struct Launch {
@@ -529,7 +536,8 @@ Bufs<R> make_bufs(ks_loop* h, const Work& w, int pr, int check_active, double to
 
 const char* const kRowNames[] = {"rows_analyze", "rows_nonlin", "rows_adj", "rows_synth"};
 const char* const kColNames[] = {"cols_analyze", "cols_synth_u", "cols_synth_r", "cols_synth_g",
-                                 "cols_resid", "cols_update", "cols_grad"};
+                                 "cols_resid", "cols_update", "cols_grad", "cols_analyze_u",
+                                 "cols_resid_r", "cols_resid_j", "cols_grad_g"};
 
 int kind_id(ks_loop* h, const std::string& name) {
     for (size_t i = 0; i < h->kind_names.size(); ++i)
@@ -557,9 +565,9 @@ struct LaunchScope {
     cudaStream_t s;
     int kind = -1;
     cudaEvent_t a = nullptr;
-    LaunchScope(ks_loop* h_, cudaStream_t s_, const std::string& name) : h(h_), s(s_) {
+    LaunchScope(ks_loop* h_, cudaStream_t s_, const char* name, const char* suffix = "") : h(h_), s(s_) {
         if (h->prof) {
-            kind = kind_id(h, name);
+            kind = kind_id(h, std::string(name) + suffix);
             a = take_event(h);
             cudaEventRecord(a, s);
         }
@@ -574,7 +582,7 @@ struct LaunchScope {
     }
 };
 
-std::string prec_suffix(int pr) { return pr == 0 ? "_f64" : "_f32"; }
+const char* prec_suffix(int pr) { return pr == 0 ? "_f64" : "_f32"; }
 
 // The float phases of a step take the register kernels wherever their lengths are covered, except
 // in the centre-symmetric subspace (whose transforms pair rows and columns differently).  The two
@@ -585,7 +593,7 @@ bool use_rg(const ks_loop* h) { return h->rg_nrow > 0 && !h->xi; }
 template <int MODE>
 int launch_rg_rows(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
     const int n = h->rg_nrow, per = RG_THREADS / 32, g = (n + per - 1) / per;
-    LaunchScope ls(h, s, std::string(kRowNames[MODE]) + prec_suffix(P32));
+    LaunchScope ls(h, s, kRowNames[MODE], prec_suffix(P32));
     switch (h->d.lgnx) {
     case 5: k_rg_rows<MODE, 5><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
     case 6: k_rg_rows<MODE, 6><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
@@ -601,7 +609,7 @@ int launch_rg_rows(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
 template <int MODE>
 int launch_rg_cols(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
     const int n = h->rg_ncol, per = RG_THREADS / 64, g = (n + per - 1) / per;
-    LaunchScope ls(h, s, std::string(kColNames[MODE]) + prec_suffix(P32));
+    LaunchScope ls(h, s, kColNames[MODE], prec_suffix(P32));
     const size_t smem = (size_t)h->rg_ntab * sizeof(rgv) + (size_t)per * RG_XBYTES;
     k_rg_cols<MODE><<<g, RG_THREADS, smem, s>>>(h->d, p, h->d_rg_cols, n, h->d_rg_tab, h->rg_ntab);
     KS_CUDA(cudaGetLastError());
@@ -653,7 +661,7 @@ int launch_rows(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
         if (use_rg(h)) return launch_rg_rows<MODE>(h, p, s);
     const Launch& l = h->lrow[pr];
     const int n = (int)h->rows.size();
-    LaunchScope ls(h, s, std::string(kRowNames[MODE]) + prec_suffix(pr));
+    LaunchScope ls(h, s, kRowNames[MODE], prec_suffix(pr));
     k_rows<R, MODE><<<std::min(n, l.grid), l.threads, l.smem, s>>>(h->d, p, n, (int)l.tw_off,
                                                                      std::max(h->d.nx, h->nsmax));
     KS_CUDA(cudaGetLastError());
@@ -668,7 +676,7 @@ int launch_cols(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
         if (use_rg(h)) return launch_rg_cols<MODE>(h, p, s);
     const Launch& l = h->lcol[pr];
     const int n = col_item_count(h->d, h->xi, MODE);
-    LaunchScope ls(h, s, std::string(kColNames[MODE]) + prec_suffix(pr));
+    LaunchScope ls(h, s, kColNames[MODE], prec_suffix(pr));
     k_cols<R, MODE><<<std::min(n, l.grid), l.threads, l.smem, s>>>(h->d, p, n, (int)l.tw_off,
                                                                      std::max(h->d.nx, h->nsmax));
     KS_CUDA(cudaGetLastError());
@@ -693,6 +701,10 @@ int set_smem_attrs(ks_loop* h) {
     KS_ATTR((k_cols<R, COL_RESID>), cs);
     KS_ATTR((k_cols<R, COL_UPDATE>), cs);
     KS_ATTR((k_cols<R, COL_GRAD>), cs);
+    KS_ATTR((k_cols<R, COL_ANALYZE_U>), cs);
+    KS_ATTR((k_cols<R, COL_RESID_R>), cs);
+    KS_ATTR((k_cols<R, COL_RESID_J>), cs);
+    KS_ATTR((k_cols<R, COL_GRAD_G>), cs);
 #undef KS_ATTR
     return KS_OK;
 }
@@ -949,7 +961,7 @@ int run_cluster(ks_loop* h, Work& w, int pr, long long nsteps, double tol, doubl
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    LaunchScope ls(h, s, std::string("cluster") + prec_suffix(pr) + (slot == 2 ? "_adj_f32" : ""));
+    LaunchScope ls(h, s, "cluster", slot == 2 ? "_f64_adj_f32" : prec_suffix(pr));
     KS_CUDA(cudaLaunchKernelEx(&cfg, cluster_fn<R, RA>(h->xi != 0, cp.mb), h->d, p,
                                ta, cp, (int)nsteps, w.par,
                                w.mix_valid[pr] ? 1 : 0));
@@ -972,31 +984,43 @@ int run_persist(ks_loop* h, Work& w, int pr, long long nsteps, double tol, doubl
     int tw_off = h->ptw_off[pr];
     int nm = std::max(h->d.nx, h->nsmax);  // longest transform
     void* args[] = {&d, &p, &ns_i, &par0, &nrow, &ncol, &bar, &tw_off, &nm};
-    LaunchScope ls(h, s, std::string("persist") + prec_suffix(pr));
+    LaunchScope ls(h, s, "persist", prec_suffix(pr));
     KS_CUDA(cudaLaunchCooperativeKernel((const void*)k_persist<R>, dim3(h->pgrid[pr]), dim3(COL_ACC_LANES),
                                         args, h->psmem[pr], s));
     ls.done();
     return KS_OK;
 }
 
-// grid -> band (u_hat) for every loop, from io
-template <typename R>
-int run_analyze(ks_loop* h, Work& w, int pr, R* io, cudaStream_t s) {
-    Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, io);
-    KS_TRY((launch_rows<R, ROW_ANALYZE>(h, p, s)));
-    KS_TRY((launch_cols<R, COL_ANALYZE>(h, p, s)));
-    w.mix_valid[pr] = false;
+// grid -> band (u_hat) for every loop, always in double: from io or, when iof is given, from a
+// float grid, and then to the float band alone.  Tin: the loops' periods (device), installed by
+// the same launches.  prec_new >= 0: so is a fresh descent state of that precision.  prime: M also
+// gets the s-inverse of u_hat (double band).
+int run_analyze(ks_loop* h, Work& w, double* io, const float* iof, const double* Tin, bool prime,
+                int prec_new, cudaStream_t s) {
+    Bufs<double> p = make_bufs<double>(h, w, P64, 0, 0.0, 0.0, io);
+    p.Tin = Tin;
+    p.prec_out = prec_new >= 0 ? w.prec : nullptr;
+    p.prec_new = prec_new;
+    p.iof = iof;
+    p.uhf = iof ? (cpx<float>*)w.uh[P32] : nullptr;
+    KS_TRY((launch_rows<double, ROW_ANALYZE>(h, p, s)));
+    const bool fuse = prime && !iof && !h->xi;
+    if (fuse) KS_TRY((launch_cols<double, COL_ANALYZE_U>(h, p, s)));
+    else KS_TRY((launch_cols<double, COL_ANALYZE>(h, p, s)));
+    w.mix_valid[P64] = w.loaded = fuse;
+    if (iof) w.mix_valid[P32] = false;
     return KS_OK;
 }
 
-// band (u_hat / r_hat / G_hat) -> grid io, every loop
+// band (u_hat / r_hat / G_hat) -> grid io, every loop; have: M holds its s-inverse already
 template <typename R, int CMODE>
-int run_synth(ks_loop* h, Work& w, int pr, R* io, cudaStream_t s) {
+int run_synth(ks_loop* h, Work& w, int pr, R* io, cudaStream_t s, bool have = false) {
     Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, io);
-    KS_TRY((launch_cols<R, CMODE>(h, p, s)));
-    KS_TRY((launch_rows<R, ROW_SYNTH>(h, p, s)));
-    w.mix_valid[pr] = false;
-    return KS_OK;
+    if (!have) {
+        KS_TRY((launch_cols<R, CMODE>(h, p, s)));
+        w.mix_valid[pr] = false;
+    }
+    return launch_rows<R, ROW_SYNTH>(h, p, s);
 }
 
 // M = s-inverse of u_hat (the input of ROW_NONLIN)
@@ -1019,37 +1043,52 @@ int run_step(ks_loop* h, Work& w, int pr, double tol, double switch_tol, cudaStr
     return KS_OK;
 }
 
-// residual pass (no update): J partials and r_hat for every loop of the workspace
-template <typename R>
+// residual pass (no update): J partials and r_hat for every loop of the workspace; M holds the
+// s-inverse of u_hat when mix_valid says so.  CMODE: COL_RESID (M = the input of ROW_ADJ),
+// COL_RESID_R (M = s-inverse of r_hat) or COL_RESID_J (the rest alone); in the subspace COL_RESID
+// stands in for all.
+template <typename R, int CMODE>
 int run_residual(ks_loop* h, Work& w, int pr, cudaStream_t s) {
     Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, (R*)nullptr);
-    KS_TRY((launch_cols<R, COL_SYNTH_U>(h, p, s)));
-    KS_TRY((launch_rows<R, ROW_NONLIN>(h, p, s)));
-    KS_TRY((launch_cols<R, COL_RESID>(h, p, s)));
+    if (!w.mix_valid[pr]) KS_TRY((launch_cols<R, COL_SYNTH_U>(h, p, s)));
     w.mix_valid[pr] = false;
+    KS_TRY((launch_rows<R, ROW_NONLIN>(h, p, s)));
+    if (h->xi) KS_TRY((launch_cols<R, COL_RESID>(h, p, s)));
+    else KS_TRY((launch_cols<R, CMODE>(h, p, s)));
     return KS_OK;
 }
 
+// M = the s-inverse of G_hat, for the synthesis of G
 template <typename R>
 int run_gradient(ks_loop* h, Work& w, int pr, cudaStream_t s) {
-    KS_TRY(run_residual<R>(h, w, pr, s));
+    KS_TRY((run_residual<R, COL_RESID>(h, w, pr, s)));
     Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, (R*)nullptr);
     KS_TRY((launch_rows<R, ROW_ADJ>(h, p, s)));
+    if (!h->xi) return launch_cols<R, COL_GRAD_G>(h, p, s);
     KS_TRY((launch_cols<R, COL_GRAD>(h, p, s)));
-    return KS_OK;
+    return launch_cols<R, COL_SYNTH_G>(h, p, s);
 }
 
-int run_finalize(ks_loop* h, Work& w, const double* T, int myprec, int mask,
-                 cudaStream_t s) {
+// M (the s-inverse of r_hat or G_hat) -> grid io, and J, dJ/dT (each nullable) in the same launch
+template <typename R>
+int run_rows_out(ks_loop* h, Work& w, int pr, R* io, double* J, double* dJdT, cudaStream_t s) {
+    Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, io);
+    p.fin = 1;
+    p.Jout = J;
+    p.dJdTout = dJdT;
+    return launch_rows<R, ROW_SYNTH>(h, p, s);
+}
+
+int run_finalize(ks_loop* h, Work& w, const double* T, int myprec, int mask, cudaStream_t s,
+                 double* J = nullptr, double* dJdT = nullptr) {
     const int B = h->d.B;
     LaunchScope ls(h, s, "finalize");
     if (myprec == P64)
-        k_finalize<double><<<(B + 127) / 128, 128, 0, s>>>(B, h->d.nkx, h->d.L, w.Jpart, w.L2part, T,
-                                                            w.prec, myprec, mask, w.J, w.dJdT, w.sqrtJ);
+        k_finalize<double><<<(B + 3) / 4, 128, 0, s>>>(B, h->d.nkx, h->d.L, w.Jpart, w.L2part, T, w.prec, myprec,
+                                                        mask, J, dJdT, w.sqrtJ);
     else
-        k_finalize<ff><<<(B + 127) / 128, 128, 0, s>>>(B, h->d.nkx, h->d.L, (const ff*)w.Jpart,
-                                                        (const ff*)w.L2part, T, w.prec, myprec, mask,
-                                                        w.J, w.dJdT, w.sqrtJ);
+        k_finalize<ff><<<(B + 3) / 4, 128, 0, s>>>(B, h->d.nkx, h->d.L, (const ff*)w.Jpart, (const ff*)w.L2part, T,
+                                                    w.prec, myprec, mask, J, dJdT, w.sqrtJ);
     KS_CUDA(cudaGetLastError());
     ls.done();
     return KS_OK;
@@ -1085,7 +1124,9 @@ int check_handle(ks_loop* h) {
 // The projection onto the band always runs in double: a float field is widened first and the
 // projected band is rounded to float afterwards, so the band of a float handle carries only
 // the rounding of its coefficients, not the transform noise of a float analysis.
-int load_state(ks_loop* h, Work& w, int pr, const void* u, const double* T, cudaStream_t s) {
+// prime: M gets the s-inverse of u_hat as well where that costs no launch.
+int load_state(ks_loop* h, Work& w, int pr, const void* u, const double* T, bool prime, int prec_new,
+               cudaStream_t s) {
     const size_t gb = (size_t)h->ngrid * elem_size(pr);
     void* io = w.io[pr];
     if (is_device_ptr(u)) {
@@ -1093,25 +1134,13 @@ int load_state(ks_loop* h, Work& w, int pr, const void* u, const double* T, cuda
     } else {
         KS_TRY(copy_in(io, u, gb, s));
     }
-    KS_TRY(copy_in(w.T, T, h->d.B * sizeof(double), s));
-    w.par = 0;
-    k_prep_wT<<<(h->d.B + 127) / 128, 128, 0, s>>>(w.T, w.wT, h->d.B);
-    KS_CUDA(cudaGetLastError());
-    if (pr == P64) {
-        KS_TRY(run_analyze<double>(h, w, P64, (double*)io, s));
-    } else {
-        const long long n = h->ngrid;
-        const int g = (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 152 * 8));
-        k_grid_f2d<<<g, 256, 0, s>>>((const float*)io, (double*)w.io[P64], n);
-        KS_CUDA(cudaGetLastError());
-        KS_TRY(run_analyze<double>(h, w, P64, (double*)w.io[P64], s));
-        const long long nb = h->nband;
-        k_band_d2f<<<(int)std::max<long long>(1, std::min<long long>((nb + 255) / 256, 152 * 8)), 256, 0, s>>>(
-            (const cpx<double>*)w.uh[P64], (cpx<float>*)w.uh[P32], nb);
-        KS_CUDA(cudaGetLastError());
-        w.mix_valid[P32] = false;
+    if (!is_device_ptr(T)) {
+        KS_TRY(copy_in(w.T, T, h->d.B * sizeof(double), s));
+        T = w.T;
     }
-    return KS_OK;
+    w.par = 0;
+    if (pr == P64) return run_analyze(h, w, (double*)io, nullptr, T, prime, prec_new, s);
+    return run_analyze(h, w, nullptr, (const float*)io, T, prime, prec_new, s);
 }
 
 // copy a device result buffer to the caller's pointer (device or host)
@@ -1349,6 +1378,27 @@ extern "C" int ks_destroy(ks_loop_t h) {
     return KS_OK;
 }
 
+namespace {
+
+// where a result of B doubles goes: the caller's buffer when it is on the device
+double* out_ptr(double* user, double* own) { return user && is_device_ptr(user) ? user : own; }
+
+template <typename R>
+int residual_call(ks_loop* h, Work& w, int pr, void* r, double* J, cudaStream_t s) {
+    if (!r) {
+        KS_TRY((run_residual<R, COL_RESID_J>(h, w, pr, s)));
+        return J ? run_finalize(h, w, w.T, pr, 0, s, J) : KS_OK;
+    }
+    KS_TRY((run_residual<R, COL_RESID_R>(h, w, pr, s)));
+    if (h->xi) {
+        Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, (R*)nullptr);
+        KS_TRY((launch_cols<R, COL_SYNTH_R>(h, p, s)));
+    }
+    return run_rows_out<R>(h, w, pr, (R*)r, J, nullptr, s);
+}
+
+}  // namespace
+
 extern "C" int ks_residual(ks_loop_t h, const void* u, const double* T, void* r, double* J,
                            void* stream) {
     g_err.clear();
@@ -1357,20 +1407,14 @@ extern "C" int ks_residual(ks_loop_t h, const void* u, const double* T, void* r,
     cudaStream_t s = (cudaStream_t)stream;
     const int pr = h->api_prec;
     Work& w = h->api;
-    KS_TRY(load_state(h, w, pr, u, T, s));
-    if (pr == P64) KS_TRY(run_residual<double>(h, w, pr, s));
-    else KS_TRY(run_residual<float>(h, w, pr, s));
-    KS_TRY(run_finalize(h, w, w.T, pr, 0, s));
-    const int B = h->d.B;
-    if (r) {
-        void* dst = is_device_ptr(r) ? r : w.io[pr];
-        if (pr == P64) KS_TRY((run_synth<double, COL_SYNTH_R>(h, w, pr, (double*)dst, s)));
-        else KS_TRY((run_synth<float, COL_SYNTH_R>(h, w, pr, (float*)dst, s)));
-        if (dst != r) KS_TRY(copy_out(r, dst, (size_t)h->ngrid * elem_size(pr), s));
-    }
-    KS_TRY(copy_out(J, w.J, B * sizeof(double), s));
-    if ((r && !is_device_ptr(r)) || (J && !is_device_ptr(J)) || !is_device_ptr(u))
-        KS_CUDA(cudaStreamSynchronize(s));
+    KS_TRY(load_state(h, w, pr, u, T, true, -1, s));
+    void* dst = !r || is_device_ptr(r) ? r : w.io[pr];
+    double* Jd = J ? out_ptr(J, w.J) : nullptr;
+    if (pr == P64) KS_TRY(residual_call<double>(h, w, pr, dst, Jd, s));
+    else KS_TRY(residual_call<float>(h, w, pr, dst, Jd, s));
+    if (dst != r) KS_TRY(copy_out(r, dst, (size_t)h->ngrid * elem_size(pr), s));
+    if (Jd != J) KS_TRY(copy_out(J, Jd, h->d.B * sizeof(double), s));
+    if (dst != r || Jd != J || !is_device_ptr(u)) KS_CUDA(cudaStreamSynchronize(s));
     return KS_OK;
 }
 
@@ -1382,17 +1426,19 @@ extern "C" int ks_adjoint_grad(ks_loop_t h, const void* u, const double* T, void
     cudaStream_t s = (cudaStream_t)stream;
     const int pr = h->api_prec;
     Work& w = h->api;
-    KS_TRY(load_state(h, w, pr, u, T, s));
-    if (pr == P64) KS_TRY(run_gradient<double>(h, w, pr, s));
-    else KS_TRY(run_gradient<float>(h, w, pr, s));
-    KS_TRY(run_finalize(h, w, w.T, pr, 0, s));
+    KS_TRY(load_state(h, w, pr, u, T, true, -1, s));
     void* dst = is_device_ptr(G) ? G : w.io[pr];
-    if (pr == P64) KS_TRY((run_synth<double, COL_SYNTH_G>(h, w, pr, (double*)dst, s)));
-    else KS_TRY((run_synth<float, COL_SYNTH_G>(h, w, pr, (float*)dst, s)));
+    double* dJd = dJdT ? out_ptr(dJdT, w.dJdT) : nullptr;
+    if (pr == P64) {
+        KS_TRY(run_gradient<double>(h, w, pr, s));
+        KS_TRY(run_rows_out<double>(h, w, pr, (double*)dst, nullptr, dJd, s));
+    } else {
+        KS_TRY(run_gradient<float>(h, w, pr, s));
+        KS_TRY(run_rows_out<float>(h, w, pr, (float*)dst, nullptr, dJd, s));
+    }
     if (dst != G) KS_TRY(copy_out(G, dst, (size_t)h->ngrid * elem_size(pr), s));
-    KS_TRY(copy_out(dJdT, w.dJdT, h->d.B * sizeof(double), s));
-    if (!is_device_ptr(G) || (dJdT && !is_device_ptr(dJdT)) || !is_device_ptr(u))
-        KS_CUDA(cudaStreamSynchronize(s));
+    if (dJd != dJdT) KS_TRY(copy_out(dJdT, dJd, h->d.B * sizeof(double), s));
+    if (dst != G || dJd != dJdT || !is_device_ptr(u)) KS_CUDA(cudaStreamSynchronize(s));
     return KS_OK;
 }
 
@@ -1472,22 +1518,18 @@ int set_state_full(ks_loop* h, const void* u, const double* T, cudaStream_t s) {
     const int pr0 = start_prec(h);
     if (h->mode == KS_MIXED) {
         // the caller's field is double: project in double, round the band to float
-        KS_TRY(load_state(h, w, P64, u, T, s));
+        KS_TRY(load_state(h, w, P64, u, T, false, pr0, s));
         const long long n = h->nband;
         k_band_d2f<<<(int)std::min<long long>((n + 255) / 256, 152 * 8), 256, 0, s>>>(
             (const cpx<double>*)w.uh[P64], (cpx<float>*)w.uh[P32], n);
         KS_CUDA(cudaGetLastError());
     } else {
-        KS_TRY(load_state(h, w, pr0, u, T, s));
+        KS_TRY(load_state(h, w, pr0, u, T, true, pr0, s));
     }
-    KS_CUDA(cudaMemsetAsync(w.status, 0, B * sizeof(int), s));
-    KS_CUDA(cudaMemsetAsync(w.steps, 0, B * sizeof(long long), s));
-    KS_CUDA(cudaMemsetAsync(w.sqrtJ, 0, B * sizeof(double), s));
     h->h_prec.assign(B, pr0);
-    KS_CUDA(cudaMemcpyAsync(w.prec, h->h_prec.data(), B * sizeof(int), cudaMemcpyHostToDevice, s));
     h->h_status.assign(B, KS_RUNNING);
     h->h_steps.assign(B, 0);
-    w.mix_valid[P64] = w.mix_valid[P32] = false;
+    if (h->mode == KS_MIXED) w.mix_valid[P64] = w.mix_valid[P32] = false;
     h->state_set = true;
     h->hist_steps.assign(B, {});
     h->hist_sqrtJ.assign(B, {});
@@ -1654,6 +1696,7 @@ void drop_graphs(ks_loop* h) {
 // four-launch form their graphs hold the two chains as parallel branches.
 int steps_impl(ks_loop* h, long long n, double tol, cudaStream_t s, bool device_switch = true) {
     Work& w = h->st;
+    if (n > 0) w.loaded = false;
     bool live[2] = {false, false};
     for (int b = 0; b < h->d.B; ++b)
         if (h->h_status[b] == KS_RUNNING) live[h->h_prec[b]] = true;
@@ -1748,6 +1791,15 @@ int set_status(ks_loop* h, cudaStream_t s) {
     return KS_OK;
 }
 
+// M of the resident state holds the s-inverse of every loop's u_hat: the steps leave it so for the
+// loops that still run (a loop that froze has other values there)
+bool mix_usable(const ks_loop* h, const Work& w, int pr) {
+    if (&w != &h->st || !w.mix_valid[pr]) return false;
+    for (int b = 0; b < h->d.B; ++b)
+        if (h->h_status[b] != KS_RUNNING || h->h_prec[b] != pr) return false;
+    return true;
+}
+
 // evaluate J at the current resident state of every loop (per precision) into sqrtJ
 int final_eval(ks_loop* h, cudaStream_t s) {
     Work& w = h->st;
@@ -1757,9 +1809,10 @@ int final_eval(ks_loop* h, cudaStream_t s) {
         for (int b = 0; b < h->d.B; ++b) any |= (h->h_prec[b] == pr);
         if (!any) continue;
         const double* Tc = w.T + (size_t)w.par * h->d.B;
-        if (pr == P64) KS_TRY(run_residual<double>(h, w, pr, s));
-        else KS_TRY(run_residual<float>(h, w, pr, s));
-        KS_TRY(run_finalize(h, w, Tc, pr, 1, s));
+        if (!mix_usable(h, w, pr)) w.mix_valid[pr] = false;
+        if (pr == P64) KS_TRY((run_residual<double, COL_RESID_J>(h, w, pr, s)));
+        else KS_TRY((run_residual<float, COL_RESID_J>(h, w, pr, s)));
+        KS_TRY(run_finalize(h, w, Tc, pr, 1, s, w.J));
     }
     return KS_OK;
 }
@@ -1786,7 +1839,8 @@ int monitor_f64(ks_loop* h, cudaStream_t s, std::vector<double>& out, bool doubl
     a.par = 0;
     k_prep_wT<<<(B + 127) / 128, 128, 0, s>>>(a.T, a.wT, B);
     KS_CUDA(cudaGetLastError());
-    KS_TRY(run_residual<double>(h, a, P64, s));
+    a.mix_valid[P64] = false;
+    KS_TRY((run_residual<double, COL_RESID_J>(h, a, P64, s)));
     KS_TRY(run_finalize(h, a, a.T, P64, 0, s));
     out.resize(B);
     KS_CUDA(cudaMemcpyAsync(out.data(), a.sqrtJ, B * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1822,7 +1876,8 @@ int polish_probe(ks_loop* h, cudaStream_t s, const std::vector<int>& sel, long l
     a.mix_valid[P64] = false;
     KS_TRY(form_steps(h, a, P64, form_of(h, P64), n, 0.0, 0.0, s, false));
     const double* Tc = a.T + (size_t)a.par * B;
-    KS_TRY(run_residual<double>(h, a, P64, s));
+    a.mix_valid[P64] = false;
+    KS_TRY((run_residual<double, COL_RESID_J>(h, a, P64, s)));
     KS_TRY(run_finalize(h, a, Tc, P64, 0, s));
     out.resize(B);
     Tout.resize(B);
@@ -1938,7 +1993,8 @@ int extrapolate_round(ks_loop* h, cudaStream_t s, const std::vector<double>& val
     a.par = 0;
     k_prep_wT<<<(B + 127) / 128, 128, 0, s>>>(a.T, a.wT, B);
     KS_CUDA(cudaGetLastError());
-    KS_TRY(run_residual<double>(h, a, P64, s));
+    a.mix_valid[P64] = false;
+    KS_TRY((run_residual<double, COL_RESID_J>(h, a, P64, s)));
     KS_TRY(run_finalize(h, a, a.T, P64, 0, s));
     std::vector<double> sqe(B);
     KS_CUDA(cudaMemcpyAsync(sqe.data(), a.sqrtJ, B * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -2005,8 +2061,9 @@ int get_state_impl(ks_loop* h, void* u, double* T, cudaStream_t s) {
         } else {
             const int pr = (h->mode == KS_FP32) ? P32 : P64;
             void* dst = is_device_ptr(u) ? u : w.io[pr];
-            if (pr == P64) KS_TRY((run_synth<double, COL_SYNTH_U>(h, w, pr, (double*)dst, s)));
-            else KS_TRY((run_synth<float, COL_SYNTH_U>(h, w, pr, (float*)dst, s)));
+            const bool have = mix_usable(h, w, pr);
+            if (pr == P64) KS_TRY((run_synth<double, COL_SYNTH_U>(h, w, pr, (double*)dst, s, have)));
+            else KS_TRY((run_synth<float, COL_SYNTH_U>(h, w, pr, (float*)dst, s, have)));
             if (dst != u) KS_TRY(copy_out(u, dst, (size_t)h->ngrid * elem_size(pr), s));
         }
     }
@@ -2252,6 +2309,7 @@ extern "C" int ks_descend(ks_loop_t h, void* u, double* T, long long max_steps, 
     }
     // final residual at the resident state (in double for every loop of a mixed descent),
     // step-cap status for the loops still running
+    KS_TRY(get_state_impl(h, u, T, s));  // first: it reads M, which the evaluation overwrites
     KS_TRY(final_eval(h, s));
     KS_TRY(readback(h, s));
     if (monitor) {
@@ -2261,7 +2319,6 @@ extern "C" int ks_descend(ks_loop_t h, void* u, double* T, long long max_steps, 
     for (int b = 0; b < B; ++b)
         if (h->h_status[b] == KS_RUNNING || h->h_status[b] == ST_SWITCH) h->h_status[b] = KS_STEP_CAP;
     KS_TRY(set_status(h, s));
-    KS_TRY(get_state_impl(h, u, T, s));
     Work& w = h->st;
     KS_TRY(copy_out(steps, w.steps, B * sizeof(long long), s));
     KS_TRY(copy_out(sqrtJ, w.sqrtJ, B * sizeof(double), s));
@@ -2358,6 +2415,7 @@ extern "C" int ks_set_option(ks_loop_t h, const char* key, long long value) {
         h->extrap_drop = (double)value * 1e-6;
     } else if (k == "symmetry") {
         if (value < 0 || value > 1) return fail(KS_ERR_ARG, "symmetry must be 0 (none) or 1 (Xi)");
+        if (h->st.loaded && h->xi != (int)value) h->st.mix_valid[P64] = false;
         h->xi = (int)value;
     } else if (k == "stall_window") {
         if (value < 1) return fail(KS_ERR_ARG, "stall_window must be >= 1");
