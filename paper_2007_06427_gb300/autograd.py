@@ -39,29 +39,30 @@ class KSLoopJ(torch.autograd.Function):
         gu = gT = None
         gJ = gJ.to(torch.float64)
         if ctx.needs_input_grad[0]:
-            fac = grid_factor(loop, u.device)                       # 2 L / (Nx Ns_b) per point
-            per_loop = torch.repeat_interleave(gJ, loop_sizes(loop, u.device))
-            gu = G * (fac * per_loop).to(G.dtype)
+            per_loop = (gJ * loop_factor(loop, u.device)).to(G.dtype)
+            gu = G * per_loop.index_select(0, loop_index(loop, u.device))
         if ctx.needs_input_grad[1]:
             gT = dJdT * gJ
         return gu, gT, None
 
 
-def loop_sizes(loop, device):
-    key = ("sizes", str(device))
+def loop_index(loop, device):
+    """Loop of each packed grid value (a gather by it needs no host read of the lengths)."""
+    key = ("index", str(device))
     cache = loop.__dict__.setdefault("_cache", {})
     if key not in cache:
-        cache[key] = torch.tensor([n * loop.nx for n in loop.ns], dtype=torch.int64, device=device)
+        sizes = torch.tensor([n * loop.nx for n in loop.ns], dtype=torch.int64, device=device)
+        cache[key] = torch.repeat_interleave(torch.arange(loop.batch, device=device), sizes)
     return cache[key]
 
 
-def grid_factor(loop, device):
-    key = ("fac", str(device))
+def loop_factor(loop, device):
+    """2 L / (Nx Ns_b) per loop."""
+    key = ("factor", str(device))
     cache = loop.__dict__.setdefault("_cache", {})
     if key not in cache:
-        f = torch.tensor([2.0 * loop.L / (loop.nx * n) for n in loop.ns], dtype=torch.float64,
-                         device=device)
-        cache[key] = torch.repeat_interleave(f, loop_sizes(loop, device))
+        cache[key] = torch.tensor([2.0 * loop.L / (loop.nx * n) for n in loop.ns], dtype=torch.float64,
+                                  device=device)
     return cache[key]
 
 
