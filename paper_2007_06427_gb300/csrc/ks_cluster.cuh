@@ -261,7 +261,8 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
     cpx<RA>* tws_a = kSame ? reinterpret_cast<cpx<RA>*>(tws) : reinterpret_cast<cpx<RA>*>(smem + cp.off_tw_a);
     // 1/(2 Nx) of the row split; per loop it is multiplied by 1/Ns, the normalisation of the
     // forward s-transform that the column phases would otherwise apply (both powers of two, so
-    // the product is exact and scaling before the transform gives the same bits as after it)
+    // the product is exact and scaling before the transform gives the same bits as after it); a
+    // double transform applies both itself (norm)
     const R h0 = (R)d.hx;
     const RA h0_a = (RA)d.hx;
     // the per-x-mode tables, read in every phase, live in shared memory
@@ -541,7 +542,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     }
                 }
                 __syncthreads();
-                cpx<R>* F = fft_warp<R, true>(Y, z, lgnx, np, -1, tws, fsc);
+                cpx<R>* F = fft_warp<R, true>(Y, z, lgnx, np, -1, tws, fsc, 0, lgnx + 1 + lg);
                 const int lgp = lgnr - 1;
                 for (int i = wtid; i < (nkx << lgp); i += ntw) {
                     const int j = i >> lgp, pr = i & (np - 1);
@@ -549,8 +550,8 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     const cpx<R> yj = F[(size_t)pr * nx + j];
                     const cpx<R> ym = conj(F[(size_t)pr * nx + ((nx - j) & (nx - 1))]);
                     const cpx<R> sm = yj + ym, df = yj - ym;
-                    xput(Mloc + (size_t)own_slot(j) * ns + n0 + 2 * pr, own_rank(j), 0, scale(sm, h),
-                         mk<R>(df.y * h, -df.x * h));
+                    xput(Mloc + (size_t)own_slot(j) * ns + n0 + 2 * pr, own_rank(j), 0, norm(sm, h),
+                         norm(mk<R>(df.y, -df.x), h));
                 }
                 __syncthreads();
                 t0 += nr;
@@ -706,15 +707,15 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                                   (RA)Ul[(size_t)(t0 + 2 * pr + 1) * nx + m] * rx.y);
                 }
                 wsync();
-                cpx<RA>* F = fft_warp<RA, true>(Y, z, lgnx, np, -1, tws_a, fsc, wn);
+                cpx<RA>* F = fft_warp<RA, true>(Y, z, lgnx, np, -1, tws_a, fsc, wn, lgnx + 1 + lg);
                 for (int i = wtid; i < (nkx << lgp); i += ntw) {
                     const int j = i >> lgp, pr = i & (np - 1);
                     if (xi && j == 0) continue;
                     const cpx<RA> yj = F[(size_t)pr * nx + j];
                     const cpx<RA> ym = conj(F[(size_t)pr * nx + ((nx - j) & (nx - 1))]);
                     const cpx<RA> sm = yj + ym, df = yj - ym;
-                    xput(Mloc2_a + (size_t)own_slot(j) * ns + n0 + 2 * pr, own_rank(j), 2, scale(sm, h_a),
-                         mk<RA>(df.y * h_a, -df.x * h_a));
+                    xput(Mloc2_a + (size_t)own_slot(j) * ns + n0 + 2 * pr, own_rank(j), 2, norm(sm, h_a),
+                         norm(mk<RA>(df.y, -df.x), h_a));
                 }
                 wsync();
                 t0 += nr;

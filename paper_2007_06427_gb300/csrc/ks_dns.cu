@@ -13,10 +13,7 @@
 // two real fields of a pair share one complex x-transform (u_a + i u_b, and the products
 // u_a^2 + i u_b^2); the state of each trajectory is its half spectrum v_j, j = 0..Kx, kept in
 // shared memory with the stage values of the scheme.  Global memory is touched at the start
-// (u0), at every saved instant (u and ||u||) and at the end.  The transforms take radix-2 passes
-// (dns_fft): an FP64 warp instruction costs the same issue time with idle lanes, and a
-// radix-2 pass has twice the butterflies of a radix-4 pass at the same operation count per
-// point, so a single pair keeps a whole warp busy and four pairs fill the block's four warps.
+// (u0), at every saved instant (u and ||u||) and at the end.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -36,7 +33,7 @@ namespace {
 constexpr int DNS_THREADS = 128;
 constexpr int DNS_PAIRS_MAX = 4;
 constexpr int DNS_CONTOUR = 32;  // points on the upper half of the contour circle
-constexpr int DNS_SPECS = 7;     // v, a, s (stage b then c), Nv, Na, Nb, Nc per trajectory
+constexpr int DNS_SPECS = 6;     // v, a, s (stage b then c), Nv, Na, Nb per trajectory
 constexpr int DNS_COEFS = 7;     // E, E2, Q, f1, f2, f3, g per x-mode
 
 struct DnsArgs {
@@ -133,34 +130,46 @@ __device__ void dns_coefficients(double* coef, int nh, double L, double dt) {
     }
 }
 
-// The x-transforms of the run: cnt transforms of length n = 2^lg in double, radix-2 passes under the
+// The x-transforms of the run: transforms of length n = 2^lg in double, radix-2 passes under the
 // conventions of fft_batch.  A run is chaotic, so its trajectory after a few hundred time units
-// hangs on the rounding of every transform: it keeps this arithmetic, where the descent's double
+// hangs on the rounding of every operation: it keeps this arithmetic, where the descent's double
 // transforms are in fixed point.  With the twiddle product fused into the additions (v0 + w v1 as
-// four fused multiply-adds, v0 - w v1 as 2 v0 minus that) it costs 3 floating-point operations
-// per point per stage, as a fused radix-4 butterfly does, with twice the butterflies per pass.
-__device__ __forceinline__ cpx<double>* dns_fft(cpx<double>* a, cpx<double>* b, int lg, int cnt, int dir,
-                                                const cpx<double>* tw, int twsh) {
-    const int n = 1 << lg;
-    const int nb = n >> 1;
-    const int total = cnt * nb;
-    for (int span = 1; span < n; span <<= 1) {
+// four fused multiply-adds, v0 - w v1 as 2 v0 minus that) it costs 3 operations per point and stage.
+//
+// A run is a chain of dependent passes, and an FP64 warp instruction holds its pipe for 64 clocks
+// whatever lanes are active, so a butterfly is shared by two threads, one per component: three
+// dependent FP64 instructions a pass where one thread takes six, on twice the warps.  The values
+// are the same.
+//
+// One component of a butterfly's outputs (c = 0 real, 1 imaginary).
+__device__ __forceinline__ void dns_bfly(cpx<double> v0, cpx<double> v1, cpx<double> w, int c, double& o0,
+                                         double& o1) {
+    const double z = c ? v0.y : v0.x, a = c ? v1.y : v1.x, b = c ? v1.x : v1.y, s = c ? w.y : -w.y;
+    o0 = fma(w.x, a, fma(s, b, z));
+    o1 = fma(2.0, z, -o0);
+}
+
+// Passes first <= span < last of cnt transforms at a (b scratch); returns where the data is.
+__device__ __forceinline__ cpx<double>* dns_passes(cpx<double>* a, cpx<double>* b, int lg, int cnt, int dir,
+                                                   const cpx<double>* tw, int twsh, int first, int last) {
+    const int n = 1 << lg, nb = n >> 1;
+    for (int span = first; span < last; span <<= 1) {
         const int tu = NMAX / (span * 2);
-        for (int i = threadIdx.x; i < total; i += blockDim.x) {
-            const int f = i >> (lg - 1);
-            const int j = i & (nb - 1);
-            const cpx<double>* s = a + (size_t)f * n;
-            cpx<double>* d = b + (size_t)f * n;
-            const cpx<double> v0 = s[j], v1 = s[j + nb];
-            const int jm = j & (span - 1);
-            const int od = ((j - jm) << 1) + jm;
+        for (int i = threadIdx.x; i < cnt << lg; i += blockDim.x) {
+            const int f = i >> lg, j = (i >> 1) & (nb - 1), c = i & 1;
+            const cpx<double>* s = a + (f << lg);
+            double* d = reinterpret_cast<double*>(b + (f << lg)) + c;
+            const int jm = j & (span - 1), od = ((j - jm) << 1) + jm;
             if (span > 1) {
-                const cpx<double> t = cfma(v0, twid<double, true>(tw, jm * tu, dir, twsh), v1);
-                d[od] = t;
-                d[od + span] = twice_minus(v0, t);
+                double o0, o1;
+                dns_bfly(s[j], s[j + nb], twid<double, true>(tw, jm * tu, dir, twsh), c, o0, o1);
+                d[2 * od] = o0;
+                d[2 * (od + span)] = o1;
             } else {
-                d[od] = v0 + v1;
-                d[od + 1] = v0 - v1;
+                const double v0 = reinterpret_cast<const double*>(s + j)[c];
+                const double v1 = reinterpret_cast<const double*>(s + j + nb)[c];
+                d[2 * od] = v0 + v1;
+                d[2 * od + 2] = v0 - v1;
             }
         }
         __syncthreads();
@@ -176,7 +185,7 @@ __device__ __forceinline__ cpx<double>* spec(cpx<double>* base, int nh, int t, i
     return base + ((size_t)t * DNS_SPECS + which) * nh;
 }
 
-enum { SV = 0, SA = 1, SS = 2, SNV = 3, SNA = 4, SNB = 5, SNC = 6 };
+enum { SV = 0, SA = 1, SS = 2, SNV = 3, SNA = 4, SNB = 5 };
 
 // Sum of y over the nx points of each trajectory of the CTA (component 0: member a, 1: b),
 // warp w reduces trajectories w, w + warps, ...; fixed order for a given nx.
@@ -193,52 +202,60 @@ __device__ void dns_norms(const cpx<double>* Y, int nx, int ntraj, double* red) 
 }
 
 // One evaluation for every trajectory of the CTA: the grid field of spectrum `src` (inverse
-// x-transform of the pair u_a + i u_b), optionally saved, and, when dst >= 0, the nonlinear
-// term N_j = -(i q_j / 2) F[u^2]_j on the retained modes (forward transform of the pair
-// u_a^2 + i u_b^2, split into the two members).
-__device__ void dns_eval(const DnsArgs& a, int tr0, int ntraj, cpx<double>* fftb, cpx<double>* specs,
-                         const cpx<double>* tw, const double* coef, double* red, int src, int dst,
-                         long long isave, bool end) {
+// x-transform of the pair u_a + i u_b), optionally saved, and, unless `end`, the nonlinear term
+// N_j = -(i q_j / 2) F[u^2]_j on the retained modes (forward transform of the pair u_a^2 + i u_b^2,
+// split into the two members), handed to use(t, j, c, N): component c of mode j of trajectory t.
+// The first pass forms the pair's spectrum as it reads it, the last inverse pass squares what it
+// writes, so that neither takes a round trip of its own.
+template <typename Use>
+__device__ __forceinline__ void dns_eval(const DnsArgs& a, int tr0, int ntraj, cpx<double>* fftb,
+                                         cpx<double>* specs, const cpx<double>* tw, const double* coef,
+                                         double* red, int src, long long isave, bool end, Use use) {
     const int nx = a.nx, lgnx = a.lgnx, kx = a.kx, nh = a.nh;
-    const int np = (ntraj + 1) >> 1;
+    const int np = (ntraj + 1) >> 1, nb = nx >> 1;
     const int twsh = LGNMAX - lgnx;
     cpx<double>* A = fftb;
     cpx<double>* Bf = fftb + (size_t)a.pairs * nx;
     for (int i = threadIdx.x; i < np * nx; i += blockDim.x) {
-        const int pr = i >> lgnx, J = i & (nx - 1);
+        const int pr = i >> lgnx, j = (i >> 1) & (nb - 1), c = i & 1;
         const int ta = 2 * pr, tb = ta + 1;
         const bool hb = tb < ntraj;
-        cpx<double> z = mk<double>(0, 0);
-        if (J <= kx) {
-            const cpx<double> va = spec(specs, nh, ta, src)[J];
-            const cpx<double> vb = hb ? spec(specs, nh, tb, src)[J] : mk<double>(0, 0);
-            z = mk<double>(va.x - vb.y, va.y + vb.x);               // v_a + i v_b
-        } else if (J >= nx - kx) {
-            const cpx<double> va = spec(specs, nh, ta, src)[nx - J];
-            const cpx<double> vb = hb ? spec(specs, nh, tb, src)[nx - J] : mk<double>(0, 0);
-            z = mk<double>(va.x + vb.y, -va.y + vb.x);              // conj v_a + i conj v_b
-        }
-        A[i] = z;
+        const double* sa = reinterpret_cast<const double*>(spec(specs, nh, ta, src));
+        const double* sb = reinterpret_cast<const double*>(spec(specs, nh, tb, src));
+        auto z = [&](int J) {  // component c of v_a + i v_b, or of conj v_a + i conj v_b
+            if (J <= kx) {
+                const double x = sa[2 * J + c], y = hb ? sb[2 * J + 1 - c] : 0.0;
+                return c ? x + y : x - y;
+            }
+            if (J >= nx - kx) {
+                const double x = sa[2 * (nx - J) + c], y = hb ? sb[2 * (nx - J) + 1 - c] : 0.0;
+                return c ? -x + y : x + y;
+            }
+            return 0.0;
+        };
+        const double v0 = z(j), v1 = z(j + nb);
+        double* d = reinterpret_cast<double*>(A + (pr << lgnx) + 2 * j) + c;
+        d[0] = v0 + v1;
+        d[2] = v0 - v1;
     }
     __syncthreads();
-    cpx<double>* Z = dns_fft(A, Bf, lgnx, np, +1, tw, twsh);
-    cpx<double>* Y = (Z == A) ? Bf : A;
+    cpx<double>* Z = dns_passes(A, Bf, lgnx, np, +1, tw, twsh, 2, nb);
+    cpx<double>* Y = Z == A ? Bf : A;
     const double inx = 1.0 / (double)nx;  // exact: nx is a power of two
     const bool save = isave >= 0;
-    for (int i = threadIdx.x; i < np * nx; i += blockDim.x) {
-        const int pr = i >> lgnx, m = i & (nx - 1);
-        const double ua = Z[i].x * inx, ub = Z[i].y * inx;
-        Y[i] = mk<double>(ua * ua, ub * ub);
-        if (save) {
-            const int ta = tr0 + 2 * pr, tb = ta + 1;
-            if (a.u_saved) {
-                a.u_saved[((size_t)ta * a.nsave + isave) * nx + m] = ua;
-                if (2 * pr + 1 < ntraj) a.u_saved[((size_t)tb * a.nsave + isave) * nx + m] = ub;
-            }
-        }
-        if (end && a.u_end) {
-            a.u_end[(size_t)(tr0 + 2 * pr) * nx + m] = ua;
-            if (2 * pr + 1 < ntraj) a.u_end[(size_t)(tr0 + 2 * pr + 1) * nx + m] = ub;
+    for (int i = threadIdx.x; i < np * nx; i += blockDim.x) {  // the pass of span nb
+        const int pr = i >> lgnx, j = (i >> 1) & (nb - 1), c = i & 1;
+        double o[2];
+        dns_bfly(Z[(pr << lgnx) + j], Z[(pr << lgnx) + j + nb],
+                 twid<double, true>(tw, j * (NMAX / nx), +1, twsh), c, o[0], o[1]);
+        const int t = 2 * pr + c;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int m = j + q * nb;
+            const double u = o[q] * inx;
+            reinterpret_cast<double*>(Y + (pr << lgnx) + m)[c] = u * u;
+            if (save && a.u_saved && t < ntraj) a.u_saved[((size_t)(tr0 + t) * a.nsave + isave) * nx + m] = u;
+            if (end && a.u_end && t < ntraj) a.u_end[(size_t)(tr0 + t) * nx + m] = u;
         }
     }
     __syncthreads();
@@ -248,19 +265,17 @@ __device__ void dns_eval(const DnsArgs& a, int tr0, int ntraj, cpx<double>* fftb
         if ((int)threadIdx.x < ntraj)
             a.norms[(size_t)(tr0 + threadIdx.x) * a.nsave + isave] = sqrt(a.L * red[threadIdx.x] * inx);
     }
-    if (dst < 0) return;
-    cpx<double>* F = dns_fft(Y, Z, lgnx, np, -1, tw, twsh);
+    if (end) return;
+    const cpx<double>* F = dns_passes(Y, Z, lgnx, np, -1, tw, twsh, 1, nx);
     const double* g = coef + 6 * nh;
-    for (int i = threadIdx.x; i < np * nh; i += blockDim.x) {
-        const int pr = i / nh, j = i - pr * nh;
-        const cpx<double> P = F[(size_t)pr * nx + j];
-        const cpx<double> Pm = conj(F[(size_t)pr * nx + ((nx - j) & (nx - 1))]);
-        const cpx<double> sm = P + Pm, df = P - Pm;
-        // W_a = (P + conj P_-j) / 2, W_b = (P - conj P_-j) / (2i); N = i g W
-        const cpx<double> Wa = mk<double>(0.5 * sm.x, 0.5 * sm.y);
-        const cpx<double> Wb = mk<double>(0.5 * df.y, -0.5 * df.x);
-        spec(specs, nh, 2 * pr, dst)[j] = mk<double>(-g[j] * Wa.y, g[j] * Wa.x);
-        if (2 * pr + 1 < ntraj) spec(specs, nh, 2 * pr + 1, dst)[j] = mk<double>(-g[j] * Wb.y, g[j] * Wb.x);
+    for (int i = threadIdx.x; i < ntraj * nh * 2; i += blockDim.x) {
+        const int c = i & 1, t = (i >> 1) / nh, j = (i >> 1) - t * nh;
+        const cpx<double> P = F[((t >> 1) << lgnx) + j], Q = F[((t >> 1) << lgnx) + ((nx - j) & (nx - 1))];
+        // W_a = (P + conj Q) / 2, W_b = (P - conj Q) / (2 i); N = i g W
+        const double h = (c ^ (t & 1)) ? P.x : P.y, k = (c ^ (t & 1)) ? Q.x : Q.y;
+        // a: W.x = (P.x + Q.x) / 2, W.y = (P.y - Q.y) / 2; b: W.x = (P.y + Q.y) / 2, W.y = -(P.x - Q.x) / 2
+        const double W = c ? 0.5 * (h + k) : ((t & 1) ? -0.5 : 0.5) * (h - k);
+        use(t, j, c, (c ? g[j] : -g[j]) * W);
     }
     __syncthreads();
 }
@@ -298,7 +313,7 @@ __global__ void __launch_bounds__(DNS_THREADS) k_dns(DnsArgs a) {
     }
     __syncthreads();
     {
-        cpx<double>* F = dns_fft(A, Bf, lgnx, np, -1, tw, twsh);
+        cpx<double>* F = dns_passes(A, Bf, lgnx, np, -1, tw, twsh, 1, nx);
         for (int i = threadIdx.x; i < np * nh; i += blockDim.x) {
             const int pr = i / nh, j = i - pr * nh;
             const cpx<double> P = F[(size_t)pr * nx + j];
@@ -322,51 +337,36 @@ __global__ void __launch_bounds__(DNS_THREADS) k_dns(DnsArgs a) {
     const double* f1 = coef + 3 * nh;
     const double* f2 = coef + 4 * nh;
     const double* f3 = coef + 5 * nh;
-    const int nsp = ntraj * nh;
+    auto at = [&](int t, int which, int j, int c) -> double& {
+        return reinterpret_cast<double*>(spec(specs, nh, t, which) + j)[c];
+    };
     for (long long n = 0; n < a.nsteps; ++n) {
         const long long isave = (n % a.save_every == 0) ? n / a.save_every : -1;
-        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SV, SNV, isave, false);
-        for (int i = threadIdx.x; i < nsp; i += blockDim.x) {  // a = E2 v + Q Nv
-            const int t = i / nh, j = i - t * nh;
-            const cpx<double> v = spec(specs, nh, t, SV)[j], N = spec(specs, nh, t, SNV)[j];
-            spec(specs, nh, t, SA)[j] = mk<double>(E2[j] * v.x + Q[j] * N.x, E2[j] * v.y + Q[j] * N.y);
-        }
-        __syncthreads();
-        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SA, SNA, -1, false);
-        for (int i = threadIdx.x; i < nsp; i += blockDim.x) {  // b = E2 v + Q Na
-            const int t = i / nh, j = i - t * nh;
-            const cpx<double> v = spec(specs, nh, t, SV)[j], N = spec(specs, nh, t, SNA)[j];
-            spec(specs, nh, t, SS)[j] = mk<double>(E2[j] * v.x + Q[j] * N.x, E2[j] * v.y + Q[j] * N.y);
-        }
-        __syncthreads();
-        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SS, SNB, -1, false);
-        for (int i = threadIdx.x; i < nsp; i += blockDim.x) {  // c = E2 a + Q (2 Nb - Nv)
-            const int t = i / nh, j = i - t * nh;
-            const cpx<double> av = spec(specs, nh, t, SA)[j];
-            const cpx<double> Nb = spec(specs, nh, t, SNB)[j], Nv = spec(specs, nh, t, SNV)[j];
-            const cpx<double> d2 = mk<double>(2.0 * Nb.x - Nv.x, 2.0 * Nb.y - Nv.y);
-            spec(specs, nh, t, SS)[j] = mk<double>(E2[j] * av.x + Q[j] * d2.x, E2[j] * av.y + Q[j] * d2.y);
-        }
-        __syncthreads();
-        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SS, SNC, -1, false);
+        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SV, isave, false, [&](int t, int j, int c, double N) {
+            at(t, SNV, j, c) = N;
+            at(t, SA, j, c) = E2[j] * at(t, SV, j, c) + Q[j] * N;  // a = E2 v + Q Nv
+        });
+        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SA, -1, false, [&](int t, int j, int c, double N) {
+            at(t, SNA, j, c) = N;
+            at(t, SS, j, c) = E2[j] * at(t, SV, j, c) + Q[j] * N;  // b = E2 v + Q Na
+        });
+        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SS, -1, false, [&](int t, int j, int c, double N) {
+            at(t, SNB, j, c) = N;
+            const double d2 = 2.0 * N - at(t, SNV, j, c);          // c = E2 a + Q (2 Nb - Nv)
+            at(t, SS, j, c) = E2[j] * at(t, SA, j, c) + Q[j] * d2;
+        });
         // v' = E v + f1 Nv + 2 f2 (Na + Nb) + f3 Nc; in the subspace the real parts are zeroed
-        for (int i = threadIdx.x; i < nsp; i += blockDim.x) {
-            const int t = i / nh, j = i - t * nh;
-            const cpx<double> v = spec(specs, nh, t, SV)[j];
-            const cpx<double> Nv = spec(specs, nh, t, SNV)[j], Na = spec(specs, nh, t, SNA)[j];
-            const cpx<double> Nb = spec(specs, nh, t, SNB)[j], Nc = spec(specs, nh, t, SNC)[j];
+        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SS, -1, false, [&](int t, int j, int c, double N) {
             const double w2 = 2.0 * f2[j];
-            cpx<double> vn = mk<double>(E[j] * v.x + f1[j] * Nv.x + w2 * (Na.x + Nb.x) + f3[j] * Nc.x,
-                                        E[j] * v.y + f1[j] * Nv.y + w2 * (Na.y + Nb.y) + f3[j] * Nc.y);
-            if (a.symmetric) vn.x = 0.0;
-            spec(specs, nh, t, SV)[j] = vn;
-        }
-        __syncthreads();
+            const double v = at(t, SV, j, c), Nv = at(t, SNV, j, c), Na = at(t, SNA, j, c), Nb = at(t, SNB, j, c);
+            const double vn = E[j] * v + f1[j] * Nv + w2 * (Na + Nb) + f3[j] * N;
+            at(t, SV, j, c) = a.symmetric && c == 0 ? 0.0 : vn;
+        });
     }
     const bool save_last = (a.nsteps % a.save_every == 0);
     if (save_last || a.u_end)
-        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SV, -1,
-                 save_last ? a.nsteps / a.save_every : -1, true);
+        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SV, save_last ? a.nsteps / a.save_every : -1, true,
+                 [](int, int, int, double) {});
 }
 
 // Loop l of a segment cut: field at instants t_a + T_l n / Ns_l (n = 0..Ns_l - 1) by linear
@@ -485,11 +485,18 @@ extern "C" int ks_dns(double L, int nx, int batch, double dt, long long nsteps, 
     a.symmetric = symmetric ? 1 : 0;
     a.nsteps = nsteps;
     a.nsave = nsteps / save_every + 1;
-    // pairs per CTA: enough butterflies for the block (nx / 2 radix-2 butterflies per pair and
-    // pass), within the shared memory of one CTA
+    // pairs per CTA: no more than spread the batch over the SMs (a pass is a chain of dependent
+    // instructions, whatever the pairs; 64 trajectories of 64 modes: 25.9 us a step on 8 CTAs), than
+    // give the block's threads two butterfly components each, or than fit its shared memory
     int pairs = std::max(1, std::min(DNS_PAIRS_MAX, (2 * DNS_THREADS) / nx));
     while (pairs > 1 && dns_plan(nx, a.nh, pairs).bytes > 200 * 1024) --pairs;
-    pairs = std::min(pairs, (batch + 1) / 2);
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
+        cudaGetLastError();
+        return dns_fail(KS_ERR_CUDA, "no usable CUDA device");
+    }
+    const int npairs = (batch + 1) / 2;
+    pairs = std::min(pairs, (npairs + sms - 1) / sms);
     a.pairs = pairs;
     const DnsPlan pl = dns_plan(nx, a.nh, pairs);
     if (pl.bytes > 227 * 1024) return dns_fail(KS_ERR_ARG, "nx too large for the shared-memory plan");

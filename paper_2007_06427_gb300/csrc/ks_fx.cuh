@@ -20,7 +20,7 @@
 // points, where the rounding of the results to double is all of it, 0.6 at 1024).
 //
 // A transform that holds an infinity or a NaN returns NaN in every element (each output depends on
-// each input); inputs below 2^-950 count as zero.
+// each input); inputs below 2^-913 count as zero.
 #pragma once
 
 #include <vector>
@@ -265,7 +265,7 @@ KS_HD int fx_ref(unsigned maxhi, unsigned sum) {
     while (bits < 32 && (sum >> bits)) ++bits;
     const int E = bits - 19 + e0;
     if (e0 == 0x7ff || E > 2046) return FX_NAN;
-    return e0 < 80 ? FX_ZERO : E;
+    return e0 < 110 ? FX_ZERO : E;  // the smallest result keeps a positive exponent, scaled down too
 }
 
 #ifndef KS_HOST_EMULATION
@@ -278,12 +278,13 @@ __device__ __forceinline__ T fx_reduce(T v, int g, Op op) {
         if (o < g) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
-// Scale of the transform whose inputs the g lanes hold, N each (called by whole warps).
+// Scale of the transform whose inputs the g lanes hold, N = 2 or 4 each (called by whole warps).
+// The order of the float sum, ((0, 1), (2, 3)) and then the xor tree, is the same for two lanes of
+// two inputs, for a lane of four and in fx_scales.
 template <int N>
 __device__ __forceinline__ int fx_group_scale(const cpx<double> (&v)[N], int g) {
-    float S = 0.f;
-#pragma unroll
-    for (int q = 0; q < N; ++q) S += fx_abs(v[q]);
+    float S = fx_abs(v[0]) + fx_abs(v[1]);
+    if constexpr (N == 4) S += fx_abs(v[2]) + fx_abs(v[3]);
     S = fx_reduce(S, g, [](float a, float b) { return a + b; });
     int E = fx_ref(S);
     if (__any_sync(0xffffffffu, !fx_sum_ok(S))) {
@@ -341,8 +342,9 @@ KS_HD double fx_out_int(long long v, unsigned del) {
 #else
     const int lz = __clzll((long long)m);
 #endif
-    const unsigned long long M = m << (lz & 63);
-    const unsigned long long q = (M >> 11) + ((M >> 10) & 1);  // leading bit at 52, or 53 after rounding
+    const unsigned long long M = m << (lz & 63) >> 1;  // |v| < 2^63: exact, leading bit at 62
+    // to nearest, ties to even, as the instruction: leading bit at 52, or 53 after rounding
+    const unsigned long long q = (M + 0x1ff + ((M >> 10) & 1)) >> 10;
     const unsigned hi = (unsigned)(q >> 32) + ((unsigned)(1085 - lz) << 20) + (((unsigned)(s >> 32)) & 0x80000000u) + del;
     const unsigned h = m != 0 ? hi : 0;
 #ifdef KS_HOST_EMULATION
@@ -354,6 +356,9 @@ KS_HD double fx_out_int(long long v, unsigned del) {
     return __hiloint2double((int)h, (int)(unsigned)q);
 #endif
 }
+
+// The scale of results that come out multiplied by 2^-down.
+KS_HD int fx_down(int E, int down) { return E >= FX_ZERO ? E : E - down; }
 
 // One result at scale E; flip: 2^31 for the conjugate.
 KS_HD cpx<double> fx_result(fxc v, int E, unsigned flip) {
@@ -379,7 +384,7 @@ KS_HD int fx_pos(int i) {
 // to double.
 template <int SPAN, bool LAST, bool FINE = false>
 KS_HD void fx_pass4(const fxc* a, fxc* b, int lg, int total, unsigned flip, const cpx<double>* tw,
-                    const int* sc, int NT) {
+                    const int* sc, int NT, int down) {
     constexpr int LI = SPAN == 4 ? 1 : SPAN == 16 ? 2 : 0, LO = (LAST || SPAN != 4) ? 0 : 2;
     const int nb = 1 << (lg - 2);
     for (int i = KS_TID; i < total; i += NT) {
@@ -396,7 +401,7 @@ KS_HD void fx_pass4(const fxc* a, fxc* b, int lg, int total, unsigned flip, cons
         const fxc o1{t1.x - t3.y, t1.y + t3.x}, o3{t1.x + t3.y, t1.y - t3.x};
         if constexpr (LAST) {
             cpx<double>* e = reinterpret_cast<cpx<double>*>(d) + od;
-            const int E = sc[f];
+            const int E = fx_down(sc[f], down);
             e[0] = fx_result(o0, E, flip);
             e[SPAN] = fx_result(o1, E, flip);
             e[2 * SPAN] = fx_result(o2, E, flip);
@@ -413,12 +418,12 @@ KS_HD void fx_pass4(const fxc* a, fxc* b, int lg, int total, unsigned flip, cons
 // The radix-2 pass that ends a transform of length 2 SPAN (SPAN = 4, 16, 64 or 256).
 template <int SPAN>
 KS_HD void fx_pass2(const fxc* a, fxc* b, int cnt, unsigned flip, const cpx<double>* tw,
-                    const int* sc, int NT) {
+                    const int* sc, int NT, int down) {
     constexpr int LI = SPAN == 4 ? 1 : SPAN == 16 ? 2 : 0, n = 2 * SPAN;
     for (int i = KS_TID; i < cnt * SPAN; i += NT) {
         const int f = i / SPAN, j = i & (SPAN - 1);
         const fxc* s = a + f * n;
-        const int E = sc[f];
+        const int E = fx_down(sc[f], down);
         const fxc v0 = s[fx_pos<LI>(j)];
         const fxc v1 = fx_mul<false>(s[fx_pos<LI>(j + SPAN)], fx_tw(tw, fx_r2_at(SPAN) + j));
         const fxc x = v0 + v1, y = v0 - v1;
@@ -428,6 +433,116 @@ KS_HD void fx_pass2(const fxc* a, fxc* b, int cnt, unsigned flip, const cpx<doub
     }
 }
 
+#ifndef KS_HOST_EMULATION
+// ---- two threads per butterfly ------------------------------------------------------------------
+// Where a call has fewer butterflies than half its threads (single loops, whose blocks hold one or
+// two columns or row pairs), two neighbouring lanes share a butterfly: lane c = 0 computes the real
+// parts, c = 1 the imaginary ones, from the same inputs.  The integers are the same, in half the
+// instructions a lane: two 64-point transforms take 2640 clocks a block, 3070 with one thread a butterfly
+// (32 points: 1970 against 2310).
+
+// component c of fx_mul<false>: a, b the value's components, w the halves (hi, lo) of the twiddle
+// that multiply them (c = 0: re, im; c = 1: im, re)
+__device__ __forceinline__ long long fx_mul_part(long long a, long long b, int2 wa, int2 wb, int c) {
+    const int al = (int)a, ah = fx_top(a) + (int)((unsigned)al >> 31);
+    const int bl = (int)b, bh = fx_top(b) + (int)((unsigned)bl >> 31);
+    const int a1 = fx_top(fx_wide(al, wa.x)), a2 = fx_top(fx_wide(ah, wa.y));
+    const int b1 = fx_top(fx_wide(bl, wb.x)) + 2 * c, b2 = fx_top(fx_wide(bh, wb.y));
+    const long long A = fx_wide(ah, wa.x) + a1 + a2, B = fx_wide(bh, wb.x) + b1 + b2;
+    const long long x = (c ? -B : B) - A;
+    return x + x;
+}
+__device__ __forceinline__ long long fx_shfl1(long long v) {
+    const int lo = __shfl_xor_sync(0xffffffffu, (int)v, 1), hi = __shfl_xor_sync(0xffffffffu, fx_top(v), 1);
+    return (long long)(((unsigned long long)(unsigned)hi << 32) | (unsigned)lo);
+}
+__device__ __forceinline__ double fx_result_part(long long v, int E, unsigned flip) {
+    if (E >= FX_ZERO) return E == FX_ZERO ? 0.0 : NAN;
+    return fx_out(v, fx_del(E) + flip);
+}
+
+template <int SPAN, bool LAST>
+__device__ __forceinline__ void fx_split4(const fxc* a, fxc* b, int lg, int total, unsigned flip,
+                                          const cpx<double>* tw, const int* sc, int NT, int down) {
+    constexpr int LI = SPAN == 4 ? 1 : SPAN == 16 ? 2 : 0, LO = (LAST || SPAN != 4) ? 0 : 2;
+    const int nb = 1 << (lg - 2), c = threadIdx.x & 1;
+    for (int i0 = threadIdx.x; (i0 & ~31) < 2 * total; i0 += NT) {  // by whole warps
+        const int i = min(i0 >> 1, total - 1);
+        const int f = i >> (lg - 2), j = i & (nb - 1);
+        const fxc* s = a + ((unsigned)f << lg);
+        const int jm = j & (SPAN - 1), od = ((j - jm) << 2) + jm;
+        const int2* w = reinterpret_cast<const int2*>(tw) + 2 * (fx_r4_at(SPAN) + 3 * jm);
+        const long long v0 = reinterpret_cast<const long long*>(s + fx_pos<LI>(j))[c];
+        const fxc v1 = s[fx_pos<LI>(j + nb)], v2 = s[fx_pos<LI>(j + 2 * nb)], v3 = s[fx_pos<LI>(j + 3 * nb)];
+        const long long a1 = fx_mul_part(v1.x, v1.y, w[c], w[c ^ 1], c);
+        const long long a2 = fx_mul_part(v2.x, v2.y, w[2 + c], w[2 + (c ^ 1)], c);
+        const long long a3 = fx_mul_part(v3.x, v3.y, w[4 + c], w[4 + (c ^ 1)], c);
+        const long long t0 = v0 + a2, t1 = v0 - a2, t2 = a1 + a3;
+        const long long u3 = fx_shfl1(a1 - a3), t3 = c ? u3 : -u3;  // i t3
+        const long long o[4] = {t0 + t2, t1 + t3, t0 - t2, t1 - t3};
+        if (i0 >= 2 * total) continue;
+        if constexpr (LAST) {
+            double* e = reinterpret_cast<double*>(b + ((unsigned)f << lg) + od) + c;
+            const int E = fx_down(sc[f], down);
+            const unsigned fl = c ? flip : 0u;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) e[2 * q * SPAN] = fx_result_part(o[q], E, fl);
+        } else {
+            long long* d = reinterpret_cast<long long*>(b + ((unsigned)f << lg)) + c;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) d[2 * fx_pos<LO>(od + q * SPAN)] = o[q];
+        }
+    }
+}
+
+template <int SPAN>
+__device__ __forceinline__ void fx_split2(const fxc* a, fxc* b, int cnt, unsigned flip, const cpx<double>* tw,
+                                          const int* sc, int NT, int down) {
+    constexpr int LI = SPAN == 4 ? 1 : SPAN == 16 ? 2 : 0, n = 2 * SPAN;
+    const int c = threadIdx.x & 1;
+    for (int i = threadIdx.x; i < cnt * 2 * SPAN; i += NT) {
+        const int f = i / (2 * SPAN), j = (i >> 1) & (SPAN - 1);
+        const fxc* s = a + f * n;
+        const int2* w = reinterpret_cast<const int2*>(tw) + 2 * (fx_r2_at(SPAN) + j);
+        const long long v0 = reinterpret_cast<const long long*>(s + fx_pos<LI>(j))[c];
+        const fxc v1 = s[fx_pos<LI>(j + SPAN)];
+        const long long p = fx_mul_part(v1.x, v1.y, w[c], w[c ^ 1], c);
+        double* d = reinterpret_cast<double*>(b + f * n + j) + c;
+        const int E = fx_down(sc[f], down);
+        const unsigned fl = c ? flip : 0u;
+        d[0] = fx_result_part(v0 + p, E, fl);
+        d[2 * SPAN] = fx_result_part(v0 - p, E, fl);
+    }
+}
+
+// The first pass (n <= 64: 2 n / 4 lanes hold a transform).
+__device__ __forceinline__ void fx_split_first(const cpx<double>* a, fxc* b, int lg, int total, unsigned flip,
+                                               int* sc, int NT) {
+    const int nb = 1 << (lg - 2), c = threadIdx.x & 1;
+    for (int i0 = threadIdx.x; (i0 & ~31) < 2 * total; i0 += NT) {
+        const int i = min(i0 >> 1, total - 1);
+        const int f = i >> (lg - 2), j = i & (nb - 1);
+        const cpx<double>* s = a + ((unsigned)f << lg) + j;
+        const cpx<double> m[2] = {s[2 * c * nb], s[(2 * c + 1) * nb]};
+        const int E = fx_group_scale(m, 2 * nb);
+        long long x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            x[q] = fx_in(reinterpret_cast<const double*>(s + q * nb)[c], E, c ? flip : 0u);
+        const long long t0 = x[0] + x[2], t1 = x[0] - x[2], t2 = x[1] + x[3];
+        const long long u3 = fx_shfl1(x[1] - x[3]), t3 = c ? u3 : -u3;
+        if (i0 >= 2 * total) continue;
+        if (j == 0 && c == 0) sc[f] = E;
+        const int o = fx_pos<1>(j << 2);
+        long long* d = reinterpret_cast<long long*>(b + ((unsigned)f << lg)) + c;
+        d[2 * o] = t0 + t2;
+        d[2 * (o ^ 1)] = t1 + t3;
+        d[2 * (o ^ 2)] = t0 - t2;
+        d[2 * (o ^ 3)] = t1 - t3;
+    }
+}
+#endif
+
 // cnt transforms of length n = 2^lg (n >= 8), stored contiguously in a, b scratch of the same
 // size: the conventions of fft_batch.  Radix-4 passes, a radix-2 pass last when lg is odd; the
 // first pass converts its input to integers, the last one converts back.  The passes have the
@@ -435,8 +550,12 @@ KS_HD void fx_pass2(const fxc* a, fxc* b, int cnt, unsigned flip, const cpx<doub
 // scales.  Lengths up to 128 form the scale in the first pass, among the n / 4 lanes that hold
 // the transform; longer ones in a pass of their own before it (a transform per warp).  The
 // arithmetic does not depend on the thread count.  True when the result is in b.
+// down: the results come out multiplied by 2^-down (a normalisation that costs nothing here).
+// SPLIT: lengths up to 64 take two threads a butterfly when there are threads for it (128 points: 3490
+// clocks for two transforms against 3370 with one thread, 256: 4630 against 4360, so not there).
+template <bool SPLIT>
 KS_HD bool fx_run(cpx<double>* a, cpx<double>* b, int lg, int cnt, int dir,
-                  const cpx<double>* tw, int* sc, int nthr) {
+                  const cpx<double>* tw, int* sc, int nthr, int down) {
 #ifdef KS_HOST_EMULATION
     const int NT = KS_NT;
     const bool pre = true;
@@ -456,6 +575,12 @@ KS_HD bool fx_run(cpx<double>* a, cpx<double>* b, int lg, int cnt, int dir,
     }
     fxc* fa = reinterpret_cast<fxc*>(a);
     fxc* fb = reinterpret_cast<fxc*>(b);
+#ifndef KS_HOST_EMULATION
+    const bool split = SPLIT && 2 * total <= NT && lg <= 6;
+    if (split) {
+        fx_split_first(a, fb, lg, total, flip, sc, NT);
+    } else
+#endif
     // span 1: no twiddles.  By whole warps: lanes past the end hold the last butterfly and store
     // nothing (the lanes of a transform are all in or all out).
     for (int i0 = KS_TID; (i0 & ~31) < total; i0 += NT) {
@@ -485,53 +610,75 @@ KS_HD bool fx_run(cpx<double>* a, cpx<double>* b, int lg, int cnt, int dir,
     }
     sync();
     // the data is in b now; the passes alternate
+#ifndef KS_HOST_EMULATION
+    if constexpr (SPLIT) {
+        if (split) {
+            if (lg == 3) {
+                fx_split2<4>(fb, fa, cnt, flip, tw, sc, NT, down);
+                sync();
+                return false;
+            }
+            if (lg == 4) {
+                fx_split4<4, true>(fb, fa, lg, total, flip, tw, sc, NT, down);
+                sync();
+                return false;
+            }
+            fx_split4<4, false>(fb, fa, lg, total, flip, tw, sc, NT, down);
+            sync();
+            if (lg == 5) fx_split2<16>(fa, fb, cnt, flip, tw, sc, NT, down);
+            else fx_split4<16, true>(fa, fb, lg, total, flip, tw, sc, NT, down);
+            sync();
+            return true;
+        }
+    }
+#endif
     switch (lg) {
     case 10:
-        fx_pass4<4, false, true>(fb, fa, lg, total, flip, tw, sc, NT);
+        fx_pass4<4, false, true>(fb, fa, lg, total, flip, tw, sc, NT, down);
         sync();
-        fx_pass4<16, false, true>(fa, fb, lg, total, flip, tw, sc, NT);
+        fx_pass4<16, false, true>(fa, fb, lg, total, flip, tw, sc, NT, down);
         sync();
-        fx_pass4<64, false, true>(fb, fa, lg, total, flip, tw, sc, NT);
+        fx_pass4<64, false, true>(fb, fa, lg, total, flip, tw, sc, NT, down);
         sync();
-        fx_pass4<256, true, true>(fa, fb, lg, total, flip, tw, sc, NT);
+        fx_pass4<256, true, true>(fa, fb, lg, total, flip, tw, sc, NT, down);
         sync();
         return true;
     case 3:
-        fx_pass2<4>(fb, fa, cnt, flip, tw, sc, NT);
+        fx_pass2<4>(fb, fa, cnt, flip, tw, sc, NT, down);
         sync();
         return false;
     case 4:
-        fx_pass4<4, true>(fb, fa, lg, total, flip, tw, sc, NT);
+        fx_pass4<4, true>(fb, fa, lg, total, flip, tw, sc, NT, down);
         sync();
         return false;
     }
-    fx_pass4<4, false>(fb, fa, lg, total, flip, tw, sc, NT);
+    fx_pass4<4, false>(fb, fa, lg, total, flip, tw, sc, NT, down);
     sync();
     switch (lg) {
     case 5:
-        fx_pass2<16>(fa, fb, cnt, flip, tw, sc, NT);
+        fx_pass2<16>(fa, fb, cnt, flip, tw, sc, NT, down);
         sync();
         return true;
     case 6:
-        fx_pass4<16, true>(fa, fb, lg, total, flip, tw, sc, NT);
+        fx_pass4<16, true>(fa, fb, lg, total, flip, tw, sc, NT, down);
         sync();
         return true;
     }
-    fx_pass4<16, false>(fa, fb, lg, total, flip, tw, sc, NT);
+    fx_pass4<16, false>(fa, fb, lg, total, flip, tw, sc, NT, down);
     sync();
     switch (lg) {
     case 7:
-        fx_pass2<64>(fb, fa, cnt, flip, tw, sc, NT);
+        fx_pass2<64>(fb, fa, cnt, flip, tw, sc, NT, down);
         sync();
         return false;
     case 8:
-        fx_pass4<64, true>(fb, fa, lg, total, flip, tw, sc, NT);
+        fx_pass4<64, true>(fb, fa, lg, total, flip, tw, sc, NT, down);
         sync();
         return false;
     }
-    fx_pass4<64, false>(fb, fa, lg, total, flip, tw, sc, NT);
+    fx_pass4<64, false>(fb, fa, lg, total, flip, tw, sc, NT, down);
     sync();
-    fx_pass2<256>(fa, fb, cnt, flip, tw, sc, NT);
+    fx_pass2<256>(fa, fb, cnt, flip, tw, sc, NT, down);
     sync();
     return true;
 }
@@ -541,11 +688,11 @@ KS_HD bool fx_run(cpx<double>* a, cpx<double>* b, int lg, int cnt, int dir,
 // step then share their instructions.  The buffers are passed as offsets into the block's dynamic shared memory, so the
 // accesses stay in the shared space.
 static __device__ __noinline__ bool fx_call(int ao, int bo, int lg, int cnt, int dir, int two, int sco,
-                                          int nthr) {
+                                          int nthr, int down) {
     extern __shared__ __align__(16) unsigned char smem[];
-    return fx_run(reinterpret_cast<cpx<double>*>(smem + ao), reinterpret_cast<cpx<double>*>(smem + bo),
+    return fx_run<true>(reinterpret_cast<cpx<double>*>(smem + ao), reinterpret_cast<cpx<double>*>(smem + bo),
                   lg, cnt, dir, reinterpret_cast<const cpx<double>*>(smem + two),
-                  reinterpret_cast<int*>(smem + sco), nthr);
+                  reinterpret_cast<int*>(smem + sco), nthr, down);
 }
 __device__ __forceinline__ int fx_off(const void* p) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -556,13 +703,14 @@ __device__ __forceinline__ int fx_off(const void* p) {
 // the transform under the conventions of fft_batch; on the device every buffer, the table (its
 // prefix, see FX_TABLE) included, is in shared memory.  fft_fx_call: through the shared copy.
 KS_HD cpx<double>* fft_fx(cpx<double>* a, cpx<double>* b, int lg, int cnt, int dir,
-                          const cpx<double>* tw, int* sc, int nthr = 0) {
-    return fx_run(a, b, lg, cnt, dir, tw, sc, nthr) ? b : a;
+                          const cpx<double>* tw, int* sc, int nthr = 0, int down = 0) {
+    return fx_run<false>(a, b, lg, cnt, dir, tw, sc, nthr, down) ? b : a;
 }
 #ifndef KS_HOST_EMULATION
 __device__ __forceinline__ cpx<double>* fft_fx_call(cpx<double>* a, cpx<double>* b, int lg, int cnt,
-                                                    int dir, const cpx<double>* tw, int* sc, int nthr = 0) {
-    return fx_call(fx_off(a), fx_off(b), lg, cnt, dir, fx_off(tw), fx_off(sc), nthr) ? b : a;
+                                                    int dir, const cpx<double>* tw, int* sc, int nthr = 0,
+                                                    int down = 0) {
+    return fx_call(fx_off(a), fx_off(b), lg, cnt, dir, fx_off(tw), fx_off(sc), nthr, down) ? b : a;
 }
 #endif
 

@@ -462,6 +462,14 @@ KS_HD cpx<R>* fft_batch(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir, const cp
 
 namespace ks {
 
+// The normalisations of the forward transforms are powers of two.  A double transform takes them in
+// its conversion (down, for nothing); the results of a float one are multiplied by norm<float>(g),
+// and those of a double one left as they are.  Either way exact, so the same bits.
+template <typename R>
+KS_HD cpx<R> norm(cpx<R> v, R g) {
+    return sizeof(R) == 8 ? v : scale(v, g);
+}
+
 // The batched transform of every launch form: double in 64-bit fixed point (fft_fx, sc: room for
 // cnt scales), float in the radix-4 passes of fft_batch.  HOT: the phases of a tau-step, which take
 // the double transform inlined (256 ragged loops: 191 us a step, 229 through calls); the items at
@@ -469,11 +477,11 @@ namespace ks {
 // it, which the launches of a call find in the instruction caches.
 template <typename R, bool HOT, bool SWZ = false, bool SKI = false, bool SKO = false>
 KS_HD cpx<R>* fft_any(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir, const cpx<R>* tw, int* sc,
-                      int nthr = 0, int twsh = 0) {
+                      int nthr = 0, int twsh = 0, int down = 0) {
 #ifndef KS_HOST_EMULATION
-    if constexpr (sizeof(R) == 8 && !HOT) return fft_fx_call(a, b, lg, cnt, dir, tw, sc, nthr);
+    if constexpr (sizeof(R) == 8 && !HOT) return fft_fx_call(a, b, lg, cnt, dir, tw, sc, nthr, down);
 #endif
-    if constexpr (sizeof(R) == 8) return fft_fx(a, b, lg, cnt, dir, tw, sc, nthr);
+    if constexpr (sizeof(R) == 8) return fft_fx(a, b, lg, cnt, dir, tw, sc, nthr, down);
     else return fft_batch<R, SWZ, SKI, SKO>(a, b, lg, cnt, dir, tw, nthr, twsh);
 }
 
@@ -610,8 +618,8 @@ __device__ __forceinline__ void load_twiddles_compact(cpx<X>* dst, const cpx<X>*
 // warp-owned (the same arithmetic as fft_batch)
 template <typename R, bool SWZ = false>
 __device__ __forceinline__ cpx<R>* fft_warp(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir,
-                                            const cpx<R>* tw, int* sc, int nthr = 0) {
-    if constexpr (sizeof(R) == 8) return fft_fx_call(a, b, lg, cnt, dir, tw, sc, nthr);
+                                            const cpx<R>* tw, int* sc, int nthr = 0, int down = 0) {
+    if constexpr (sizeof(R) == 8) return fft_fx_call(a, b, lg, cnt, dir, tw, sc, nthr, down);
     else return fft_warp_any<R, SWZ>(a, b, lg, cnt, dir, tw, nthr);
 }
 #endif
@@ -1067,9 +1075,8 @@ KS_HD void load_pair_spectra(const Dims& d, const cpx<R>* Mb, int ns, int n0, in
     }
 }
 
-// From Y = FFT(y_a + i y_b) (forward, unscaled, row-skewed) extract the half spectra of the two
-// real rows,
-// scaled by 1/Nx, for j = 0..Kx, and store them to M[j][n0 + 2 pr + {0,1}].
+// From Y = FFT(y_a + i y_b) (forward, row-skewed; in double scaled by 1 / (2 Nx) already) extract the
+// half spectra of the two real rows, scaled by 1/Nx, for j = 0..Kx, and store them to M[j][n0 + 2 pr + {0,1}].
 template <typename R>
 KS_HD void store_pair_spectra(const Dims& d, const cpx<R>* Y, cpx<R>* Mb, int ns, int n0,
                               int lgp) {
@@ -1086,8 +1093,8 @@ KS_HD void store_pair_spectra(const Dims& d, const cpx<R>* Y, cpx<R>* Mb, int ns
         const cpx<R> sm = yj + ym;  // 2 X^a
         const cpx<R> df = yj - ym;  // 2 i X^b
         cpx<R>* col = Mb + (size_t)j * ns + n0 + 2 * pr;
-        col[0] = scale(sm, h);
-        col[1] = mk<R>(df.y * h, -df.x * h);
+        col[0] = norm(sm, h);
+        col[1] = norm(mk<R>(df.y, -df.x), h);
     }
 }
 
@@ -1128,7 +1135,7 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
             }
         }
         KS_SYNC();
-        cpx<R>* Y = fft_any<R, kHot, SWZ, false, true>(A, Bf, lgnx, npairs, -1, p.tw, sc, 0, p.twsh);
+        cpx<R>* Y = fft_any<R, kHot, SWZ, false, true>(A, Bf, lgnx, npairs, -1, p.tw, sc, 0, p.twsh, lgnx + 1);
         store_pair_spectra(d, Y, Mb, ns, n0, lgp);
         KS_SYNC();
     } else if constexpr (MODE == ROW_SYNTH) {
@@ -1175,7 +1182,7 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                 Y[i] = mk<R>(ua * uxa, ub * uxb);
             }
             KS_SYNC();
-            cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, yv, lgnx, npairs, -1, p.tw, sc, 0, p.twsh);  // a4 (x-pass)
+            cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, yv, lgnx, npairs, -1, p.tw, sc, 0, p.twsh, lgnx + 1);  // a4 (x-pass)
             store_pair_spectra(d, F, Mb, ns, n0, lgp);
             KS_SYNC();
             return;
@@ -1210,7 +1217,7 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
             Y[i] = mk<R>(za.x * za.y, zb.x * zb.y);
         }
         KS_SYNC();
-        cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, z, lgnx, npairs, -1, p.tw, sc, 0, p.twsh);  // a4 (x-pass)
+        cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, z, lgnx, npairs, -1, p.tw, sc, 0, p.twsh, lgnx + 1);  // a4 (x-pass)
         store_pair_spectra(d, F, Mb, ns, n0, lgp);
         KS_SYNC();
     } else if constexpr (MODE == ROW_ADJ) {
@@ -1228,7 +1235,7 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
             Y[i] = mk<R>(ua[m] * rx.x, ua[nx + m] * rx.y);  // w = u r_x  (a8)
         }
         KS_SYNC();
-        cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, z, lgnx, npairs, -1, p.tw, sc, 0, p.twsh);
+        cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, z, lgnx, npairs, -1, p.tw, sc, 0, p.twsh, lgnx + 1);
         store_pair_spectra(d, F, Mb, ns, n0, lgp);
         KS_SYNC();
         // double: the loop's step scalars, once per loop (the column partials are complete since
@@ -1407,7 +1414,7 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
         // RESID, UPDATE, GRAD: forward s-transform of the imaginary columns P or W of M, in one
         for (int i = KS_TID; i < ns; i += KS_NT) A[i] = mk<R>(cola[i].y, hasb ? colb[i].y : (R)0);
         KS_SYNC();
-        cpx<R>* F = fft_any<R, kHot, SWZ>(A, Bf, lg, 1, -1, p.tw, sc, 0, p.twsh);
+        cpx<R>* F = fft_any<R, kHot, SWZ>(A, Bf, lg, 1, -1, p.tw, sc, 0, p.twsh, lg);
         cpx<R>* X = (F == A) ? Bf : A;
         const R ins = p.insv[b];
         const R w_over_T = (R)wTc[b];
@@ -1424,14 +1431,14 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
                     const cpx<R> ck = F[i], cm = F[(ns - i) & (ns - 1)];
                     const R bk = -(R)k * w_over_T;            // -omega_k / T
                     // r_hat = (a + i bk) u_hat - p_hat for both columns                     (a5)
-                    const cpx<R> pa = scale(xi_split_a(ck, cm), ins);
+                    const cpx<R> pa = norm(xi_split_a(ck, cm), ins);
                     const cpx<R> ua = p.uh[ba + (k + ks)];
                     const cpx<R> ra = symbol_add(lin_a, bk, ua, neg(pa));
                     p.rh[ba + (k + ks)] = ra;
                     if (fused) acc[0].add(ua, ra, k);         // a6
                     cpx<R> xb = zero;
                     if (hasb) {
-                        const cpx<R> pb = scale(xi_split_b(ck, cm), ins);
+                        const cpx<R> pb = norm(xi_split_b(ck, cm), ins);
                         const cpx<R> ub = p.uh[bb + (k + ks)];
                         const cpx<R> rb = symbol_add(lin_b, bk, ub, neg(pb));
                         p.rh[bb + (k + ks)] = rb;
@@ -1477,7 +1484,7 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
         // G_hat = (a + i omega/T) r_hat + F[P(u r_x)] for both columns at mode k              (a9)
         auto g_at = [&](int i, int k, bool second) {
             const cpx<R> ck = F[i], cm = F[(ns - i) & (ns - 1)];
-            const cpx<R> wh = scale(second ? xi_split_b(ck, cm) : xi_split_a(ck, cm), ins);
+            const cpx<R> wh = norm(second ? xi_split_b(ck, cm) : xi_split_a(ck, cm), ins);
             const cpx<R> r = p.rh[(second ? bb : ba) + (k + ks)];
             const R a_lin = second ? lin_b : lin_a;
             const R bk = (R)k * w_over_T;
@@ -1594,15 +1601,15 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
         // the remaining modes start with a forward s-transform of the column of M
         for (int i = KS_TID; i < ns; i += KS_NT) A[i] = col[i];
         KS_SYNC();
-        cpx<R>* F = fft_any<R, kHot, SWZ>(A, Bf, lg, 1, -1, p.tw, sc, 0, p.twsh);
+        cpx<R>* F = fft_any<R, kHot, SWZ>(A, Bf, lg, 1, -1, p.tw, sc, 0, p.twsh, lg);
         cpx<R>* X = (F == A) ? Bf : A;
         const R ins = p.insv[b];
 
         if constexpr (MODE == COL_ANALYZE) {
             for (int kk = KS_TID; kk < nk; kk += KS_NT) {
                 const int k = kk - ks;
-                cpx<R> v = scale(F[k & (ns - 1)], ins);
-                if (p.xi) v = (j == 0) ? mk<R>(0, 0) : xi_pair(v, scale(F[(-k) & (ns - 1)], ins));
+                cpx<R> v = norm(F[k & (ns - 1)], ins);
+                if (p.xi) v = (j == 0) ? mk<R>(0, 0) : xi_pair(v, norm(F[(-k) & (ns - 1)], ins));
                 if (p.uhf) p.uhf[bo + kk] = mk<float>((float)v.x, (float)v.y);
                 else p.uh[bo + kk] = v;
             }
@@ -1620,7 +1627,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                 const int k = (i < (ns >> 1)) ? i : i - ns;
                 cpx<R> v = mk<R>(0, 0);
                 if (k >= -ks && k <= ks) {
-                    v = scale(F[i], ins);
+                    v = norm(F[i], ins);
                     p.uh[bo + (k + ks)] = v;
                 }
                 X[i] = v;
@@ -1642,7 +1649,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                 const int k = (i < (ns >> 1)) ? i : i - ns;
                 cpx<R> x = mk<R>(0, 0);
                 if (k >= -ks && k <= ks) {
-                    const cpx<R> ph = scale(F[i], ins);
+                    const cpx<R> ph = norm(F[i], ins);
                     const cpx<R> u = p.uh[bo + (k + ks)];
                     const R bk = -(R)k * w_over_T;            // -omega_k / T
                     // r_hat = (a + i bk) u_hat - p_hat                                    (a5)
@@ -1671,7 +1678,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                 const int k = (i < (ns >> 1)) ? i : i - ns;
                 cpx<R> x = mk<R>(0, 0);
                 if (k >= -ks && k <= ks) {
-                    const cpx<R> wh = scale(F[i], ins);
+                    const cpx<R> wh = norm(F[i], ins);
                     const cpx<R> r = p.rh[bo + (k + ks)];
                     const R bk = (R)k * w_over_T;             // +omega_k / T
                     const cpx<R> G = symbol_add(a_lin, bk, r, wh);
@@ -1705,7 +1712,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                 for (int i = KS_TID; i < ns; i += KS_NT) {
                     const int k = (i < (ns >> 1)) ? i : i - ns;
                     if (k >= -ks && k <= ks) {
-                        const cpx<R> wh = scale(F[i], ins);
+                        const cpx<R> wh = norm(F[i], ins);
                         const cpx<R> r = p.rh[bo + (k + ks)];
                         const R bk = (R)k * w_over_T;
                         X[i] = symbol_add(a_lin, bk, r, wh);
@@ -1723,7 +1730,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                     if (p.xi) {
                         G = (j == 0) ? mk<R>(0, 0) : xi_pair(X[i], X[(ns - i) & (ns - 1)]);
                     } else {
-                        const cpx<R> wh = scale(F[i], ins);
+                        const cpx<R> wh = norm(F[i], ins);
                         const cpx<R> r = p.rh[bo + (k + ks)];
                         const R bk = (R)k * w_over_T;
                         // G_hat = (a + i omega/T) r_hat + F[P(u r_x)]                      (a9)
@@ -1748,5 +1755,123 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
         }
     }
 }
+
+#ifndef KS_HOST_EMULATION
+// ------------------------------------------------------------------------------------
+// Column groups: the double column phases of a step (COL_RESID, COL_UPDATE, outside the subspace)
+// on several columns of one loop at a time.  A block of 128 threads holds 128 butterflies of the
+// radix-4 passes: one column of 128 points gives 32, so three warps in four waited at the
+// barriers (256 ragged loops: 54 us a column launch).  The arithmetic and the orders of the sums
+// are those of col_item, so the results are the same bits.
+// ------------------------------------------------------------------------------------
+struct ColTile {
+    int b, j0, n;  // loop, first column, columns
+};
+constexpr int CG_THREADS = 128;
+constexpr int CG_MAX = 16;        // columns of a group
+// columns of ns points in a group: 512 points, so 128 butterflies
+KS_HDX int cg_cols(int ns) { return ns >= 512 ? 1 : (512 / ns < CG_MAX ? 512 / ns : CG_MAX); }
+// shared memory after the two transform buffers: warp sums (J, L per 32 accumulators of a column),
+// scales
+constexpr size_t CG_EXTRA = (2 * 4 * CG_MAX) * sizeof(double) + CG_MAX * sizeof(int);
+
+template <int MODE>
+__device__ __forceinline__ void col_group(const Dims& d, const Bufs<double>& p, const ColTile& t,
+                                          unsigned char* smem, int pts) {
+    typedef cpx<double> C;
+    const int b = t.b, ns = p.ns[b], lg = p.lgns[b], ks = p.ks[b], nk = 2 * ks + 1;
+    const int tid = threadIdx.x, total = t.n << lg;
+    C* A = reinterpret_cast<C*>(smem);
+    C* Bf = A + pts;
+    double* red = reinterpret_cast<double*>(Bf + pts);
+    int* sc = reinterpret_cast<int*>(red + 2 * 4 * CG_MAX);
+    C* const col = p.M + p.moff[b] + (size_t)t.j0 * ns;
+    const size_t bo = (size_t)p.boff[b] + (size_t)t.j0 * nk;
+    for (int i = tid; i < total; i += CG_THREADS) A[i] = col[i];
+    __syncthreads();
+    C* F = fft_fx(A, Bf, lg, t.n, -1, p.tw, sc, 0, lg);
+    C* X = F == A ? Bf : A;
+    const double w_over_T = p.wT[(size_t)p.par * d.B + b];
+    if constexpr (MODE == COL_RESID) {
+        // element n of a column goes to accumulator n mod 128; a warp holds 32 accumulators of one
+        // column (ns >= 32) or the whole of one or more columns
+        const int w = ns < 32 ? ns : 32, seg = ns <= 128 ? ns : 128;
+        for (int i0 = tid; i0 < t.n * seg; i0 += CG_THREADS) {  // whole warps: n seg is a multiple of 32
+            const int q = i0 / seg, n0 = i0 - q * seg, j = t.j0 + q;
+            const double a_lin = p.lin[j], rq = p.qv[j];
+            ColAcc<double> acc;
+            for (int n = n0; n < ns; n += seg) {
+                const int i = (q << lg) + n, k = n < (ns >> 1) ? n : n - ns;
+                C x = mk<double>(0, 0);
+                if (k >= -ks && k <= ks) {
+                    const size_t e = bo + (size_t)q * nk + (k + ks);
+                    const C u = p.uh[e];
+                    const C r = symbol_add(a_lin, -(double)k * w_over_T, u, neg(F[i]));  // a5
+                    p.rh[e] = r;
+                    acc.add(u, r, k);                                                    // a6
+                    x = mk<double>(-rq * r.y, rq * r.x);                                 // a7
+                }
+                X[i] = x;
+            }
+            for (int o = w >> 1; o > 0; o >>= 1) {
+                acc.J += __shfl_xor_sync(0xffffffffu, acc.J, o);
+                acc.L += __shfl_xor_sync(0xffffffffu, acc.L, o);
+            }
+            if ((tid & (w - 1)) == 0) {
+                const int g = (n0 / w) + 4 * q;
+                red[2 * g] = acc.J;
+                red[2 * g + 1] = acc.L;
+            }
+        }
+        __syncthreads();
+        if (tid < t.n) {
+            // the warps' sums: distances 2 and 1, over those that exist
+            const double* s = red + 8 * tid;
+            const int m = seg / w, j = t.j0 + tid;
+            ColAcc<double> acc;
+            if (m == 4) {
+                acc.J = (s[0] + s[4]) + (s[2] + s[6]);
+                acc.L = (s[1] + s[5]) + (s[3] + s[7]);
+            } else if (m == 2) {
+                acc.J = s[0] + s[2];
+                acc.L = s[1] + s[3];
+            } else {
+                acc.J = s[0];
+                acc.L = s[1];
+            }
+            const double wj = j == 0 ? 1.0 : 2.0;
+            p.Jpart[(size_t)b * d.nkx + j] = acc.part_J(wj);
+            p.L2part[(size_t)b * d.nkx + j] = acc.part_L(wj);
+        }
+    } else {
+        // by (k, -k) pairs, which share the IMEX factor; the rest of the spectrum is zeroed apart
+        const double wT2 = w_over_T * w_over_T;
+        const int nh = ks + 1;
+        for (int i = tid; i < t.n * nh; i += CG_THREADS) {
+            const int q = i / nh, k = i - q * nh, j = t.j0 + q;
+            const double a_lin = p.lin[j];
+            const double f = d.scheme == 1 ? imex_factor(d.dtau, k, wT2, p.cq[j]) : d.dtau;
+            auto upd = [&](int kk, int n) {
+                const size_t e = bo + (size_t)q * nk + (kk + ks);
+                const C G = symbol_add(a_lin, (double)kk * w_over_T, p.rh[e], F[(q << lg) + n]);  // a9
+                const C u = step_along(p.uh[e], G, f);                                             // a10
+                p.uh[e] = u;
+                X[(q << lg) + n] = u;
+            };
+            upd(k, k);
+            if (k > 0) upd(-k, ns - k);
+        }
+        const int gap = ns - nk;
+        for (int i = tid; i < t.n * gap; i += CG_THREADS) {
+            const int q = i / gap;
+            X[(q << lg) + ks + 1 + (i - q * gap)] = mk<double>(0, 0);
+        }
+        __syncthreads();
+    }
+    const C* v = fft_fx(X, F, lg, t.n, +1, p.tw, sc);
+    for (int i = tid; i < total; i += CG_THREADS) col[i] = v[i];
+    __syncthreads();
+}
+#endif
 
 }  // namespace ks

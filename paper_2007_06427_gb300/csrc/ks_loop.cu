@@ -78,6 +78,30 @@ __global__ void __launch_bounds__(256) k_cols(Dims d, Bufs<R> p, int nitems, int
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) col_item<R, MODE, true>(d, q, it, smem, q.par);
 }
 
+// The double column phases of a step by groups of columns (col_group).
+template <int MODE>
+__global__ void __launch_bounds__(CG_THREADS) k_cols_g(Dims d, Bufs<double> p, const ColTile* tiles, int ntiles,
+                                                       int pts, int tw_off, int nm) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const Bufs<double> q = stage_twiddles(p, smem, tw_off, nm);
+    for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
+        const ColTile t = tiles[it];
+        if constexpr (MODE == COL_RESID) {
+            if (!loop_live(q, t.b)) continue;
+        } else {
+            if (q.check_active && q.prec[t.b] != q.myprec) continue;
+            if (q.check_active && q.status[t.b] != ST_RUNNING) {
+                if (t.j0 == 0 && threadIdx.x == 0) {
+                    q.T[(size_t)(q.par ^ 1) * d.B + t.b] = q.T[(size_t)q.par * d.B + t.b];
+                    q.wT[(size_t)(q.par ^ 1) * d.B + t.b] = q.wT[(size_t)q.par * d.B + t.b];
+                }
+                continue;
+            }
+        }
+        col_group<MODE>(d, q, t, smem, pts);
+    }
+}
+
 // double band -> float band (every loop)
 __global__ void k_band_d2f(const cpx<double>* src, cpx<float>* dst, long long n) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -344,6 +368,10 @@ struct ks_loop {
     Work st;   // resident descent state
     Work api;  // scratch for ks_residual / ks_adjoint_grad
     Launch lrow[2], lcol[2];
+    // double column phases by groups of columns (none: see setup_cg)
+    int ncg = 0, cg_pts = 0;
+    size_t cg_tw_off = 0, cg_smem = 0;
+    ColTile* d_cg = nullptr;
     // float phases with the transforms in registers (ks_reg.cuh): tiles, or none where a length is
     // not covered
     int rg_nrow = 0, rg_ncol = 0, rg_ntab = 0;
@@ -654,6 +682,39 @@ int setup_rg(ks_loop* h) {
     return KS_OK;
 }
 
+// Groups of columns for the double column phases: where they leave every SM at least two blocks
+// (a single loop's few columns run faster one to a block), in colorder.
+int setup_cg(ks_loop* h) {
+    std::vector<ColTile> tiles;
+    bool grouped = false;
+    for (int b : h->colorder) {
+        const int g = cg_cols(h->ns[b]);
+        grouped |= g > 1;
+        for (int j = 0; j < h->d.nkx; j += g) tiles.push_back(ColTile{b, j, std::min(g, h->d.nkx - j)});
+    }
+    if (!grouped || tiles.size() < 2 * 152) return KS_OK;
+    for (int n : h->ns)
+        if (n < 32) return KS_OK;  // a group's accumulators fill whole warps
+    h->cg_pts = std::max(512, h->nsmax);
+    h->cg_tw_off = (2 * (size_t)h->cg_pts * sizeof(cpx<double>) + CG_EXTRA + 15) & ~(size_t)15;
+    h->cg_smem = h->cg_tw_off + twiddle_bytes<double>(h->nsmax, true);
+    KS_CUDA(cudaFuncSetAttribute(k_cols_g<COL_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->cg_smem));
+    KS_CUDA(cudaFuncSetAttribute(k_cols_g<COL_UPDATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->cg_smem));
+    KS_TRY(upload(h, &h->d_cg, tiles));
+    h->ncg = (int)tiles.size();
+    return KS_OK;
+}
+
+template <int MODE>
+int launch_cols_g(ks_loop* h, const Bufs<double>& p, cudaStream_t s) {
+    LaunchScope ls(h, s, kColNames[MODE], prec_suffix(P64));
+    k_cols_g<MODE><<<h->ncg, CG_THREADS, h->cg_smem, s>>>(h->d, p, h->d_cg, h->ncg, h->cg_pts, (int)h->cg_tw_off,
+                                                          h->nsmax);
+    KS_CUDA(cudaGetLastError());
+    ls.done();
+    return KS_OK;
+}
+
 template <typename R, int MODE>
 int launch_rows(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const int pr = std::is_same<R, double>::value ? P64 : P32;
@@ -674,6 +735,8 @@ int launch_cols(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const int pr = std::is_same<R, double>::value ? P64 : P32;
     if constexpr (std::is_same<R, float>::value && (MODE == COL_RESID || MODE == COL_UPDATE))
         if (use_rg(h)) return launch_rg_cols<MODE>(h, p, s);
+    if constexpr (std::is_same<R, double>::value && (MODE == COL_RESID || MODE == COL_UPDATE))
+        if (h->ncg > 0 && !h->xi) return launch_cols_g<MODE>(h, p, s);
     const Launch& l = h->lcol[pr];
     const int n = col_item_count(h->d, h->xi, MODE);
     LaunchScope ls(h, s, kColNames[MODE], prec_suffix(pr));
@@ -1228,7 +1291,9 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
     // small batches get smaller tiles so that at least two row items exist per SM.
     {
         long long rows_total = go / cfg->nx;
-        h->rows_per_tile = 8;
+        // Rows of up to 64 points take tiles of 16: the row pairs' transforms then fill a block of
+        // 128 threads (16 butterflies each).
+        h->rows_per_tile = h->d.nx <= 64 ? 16 : 8;
         while (h->rows_per_tile > 2 &&
                (2 * (size_t)h->rows_per_tile * cfg->nx * sizeof(cpx<double>) > 96 * 1024 ||
                 rows_total / h->rows_per_tile < 2 * 152))
@@ -1339,6 +1404,7 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
     }
     if ((rc = set_smem_attrs<double>(h)) || (rc = set_smem_attrs<float>(h))) return cleanup(rc);
     if (h->need[P32] && (rc = setup_rg(h))) return cleanup(rc);
+    if (h->need[P64] && (rc = setup_cg(h))) return cleanup(rc);
     if ((rc = setup_persistent<double>(h)) || (rc = setup_persistent<float>(h))) return cleanup(rc);
     if ((rc = setup_cluster<double, double>(h)) || (rc = setup_cluster<float, float>(h)) ||
         (h->mode == KS_MIXED && (rc = setup_cluster<double, float>(h))))

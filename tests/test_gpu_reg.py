@@ -65,3 +65,24 @@ def test_explicit_steps_and_frozen_loops():
             for p in (1, 2))
     assert all(np.array_equal(x, y) for x, y in zip(a, b))
     assert (a[5] == K.KS_CONVERGED).any() and (a[5] == K.KS_RUNNING).any()
+
+
+@pytest.mark.parametrize("nx,ns", [(64, [32] * 40 + [64] * 30 + [128, 256] * 20 + [512]), (64, [64] * 120),
+                                   (32, [128, 256] * 60), (128, [1024] * 5 + [32] * 90)])
+def test_column_groups_have_the_items_bits(nx, ns):
+    """The double column phases by groups of columns (large batches) against the items."""
+    outs = []
+    L = 22.0 * nx / 64
+    us, Ts = zip(*[spectral_loop(i, nx, L, ns=n, T_range=(20.0, 90.0))[:2] for i, n in enumerate(ns)])
+    for path in (2, 1):
+        u = torch.tensor(np.concatenate([v.ravel() for v in us]), device="cuda")
+        T = torch.tensor(Ts, dtype=torch.float64, device="cuda")
+        sq = torch.zeros(len(ns), dtype=torch.float64, device="cuda")
+        with K.KSLoop(L, nx, ns, K.KS_FP64, K.KS_IMEX, 0.1) as h:
+            K.ks_set_option(h.handle, "path", path)
+            K.ks_set_state(h.handle, u, T)
+            K.ks_step(h.handle, 3, 0.0)
+            K.ks_get_state(h.handle, u, T, None, sq)
+        outs.append([x.cpu().numpy() for x in (u, T, sq)])
+    for x, y in zip(*outs):
+        assert np.isfinite(x).all() and np.array_equal(x, y)
