@@ -521,6 +521,31 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                         Ul[(size_t)(t0 + 2 * pr + 1) * nx + m] = ub;
                         Y[i] = mk<R>(ua * uxa, ub * uxb);
                     }
+                } else if constexpr (sizeof(R) == 8) {
+                    // u of the row pairs, then u^2 (residual_at)
+                    const int lgq = lgnr - 1;
+                    for (int i = wtid; i < np * nx; i += ntw) {
+                        const int J = i >> lgq, pr = i & (np - 1);
+                        cpx<R> zz = mk<R>(0, 0);
+                        if (J <= kx) {
+                            const cpx<R>* src = Rin + (size_t)J * rmax + t0 + 2 * pr;
+                            zz = src[0] + mul_i(src[1], 1);
+                        } else if (J >= nx - kx) {
+                            const cpx<R>* src = Rin + (size_t)(nx - J) * rmax + t0 + 2 * pr;
+                            zz = conj(src[0]) + mul_i(conj(src[1]), 1);
+                        }
+                        A[(size_t)pr * nx + J] = zz;
+                    }
+                    __syncthreads();
+                    z = fft_warp<R, true>(A, Bf, lgnx, np, +1, tws, fsc);
+                    Y = (z == A) ? Bf : A;
+                    for (int i = wtid; i < np * nx; i += ntw) {
+                        const int pr = i >> lgnx, m = i & (nx - 1);
+                        const cpx<R> u = z[i];
+                        Ul[(size_t)(t0 + 2 * pr) * nx + m] = u.x;
+                        Ul[(size_t)(t0 + 2 * pr + 1) * nx + m] = u.y;
+                        Y[i] = mk<R>(u.x * u.x, u.y * u.y);
+                    }
                 } else {
                     for (int i = wtid; i < nr * nx; i += ntw) {
                         const int J = i >> lgnr, r = i & (nr - 1);
@@ -640,7 +665,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                                     const cpx<R> ph = Mloc[(q << lg) + n];
                                     const cpx<R> u = uhl[q * nk + k + ks];
                                     const R bk = -(R)k * wTr;
-                                    const cpx<R> r = symbol_add(a_lin, bk, u, neg(ph));
+                                    const cpx<R> r = residual_at(a_lin, bk, u, ph, rq);
                                     rhl[q * nk + k + ks] = r;
                                     acc[t].add(u, r, k);
                                     x = mk<R>(-rq * r.y, rq * r.x);

@@ -19,6 +19,7 @@
 // array M[b][j][n] (x-mode j, time sample n).  A step is four phases, each a set of
 // independent CTA work items:
 //   ROW_NONLIN  (rows)    : M = v (u_hat s-inverted) -> u, u_x rows -> U grid, p = u u_x -> M = P
+//                           (double, outside the subspace: u rows, p = u^2, see residual_at)
 //   COL_RESID   (columns) : M = P -> r_hat (a5), partial J / L^dag_2 (a6), M = s-inverse of i q r_hat
 //   ROW_ADJ     (rows)    : M = rho -> r_x rows, w = u r_x -> M = W
 //   COL_UPDATE  (columns) : M = W -> G_hat (a9), update (a10), M = s-inverse of the new u_hat
@@ -119,6 +120,22 @@ KS_HD cpx<R> cfma(cpx<R> v0, cpx<R> w, cpx<R> v) {
 template <typename R>
 KS_HD cpx<R> symbol_add(R a, R b, cpx<R> v, cpx<R> c) {
     return mk<R>(fmx(a, v.x, -mul_rn(b, v.y)) + c.x, fmx(a, v.y, mul_rn(b, v.x)) + c.y);
+}
+// r_hat from u_hat and the transformed product (a5).  Float: F holds the spectrum of u u_x, r_hat =
+// (a + i b) u_hat - F.  Double: F holds the spectrum of u^2 and u u_x = (u^2)_x / 2, so its own is
+// i q / 2 F (the truncated products are exact projections of the continuous ones, so this is the same
+// quantity): no transform for u_x.  The factor q / 2 multiplies the white noise of the forward
+// transform, which in fixed point is so far below the double transform's that r and G come out 5 to 20
+// times closer to a long double evaluation than with a double transform of u u_x; in float the
+// noise at the band's edge would grow by the factor.
+template <typename R>
+KS_HD cpx<R> residual_at(R a, R b, cpx<R> u, cpx<R> F, R q) {
+    if constexpr (sizeof(R) == 8) {
+        const R h = (R)0.5 * q;
+        return mk<R>(fmx(h, F.y, fmx(a, u.x, -mul_rn(b, u.y))), fmx(-h, F.x, fmx(a, u.y, mul_rn(b, u.x))));
+    } else {
+        return symbol_add(a, b, u, neg(F));
+    }
 }
 // u - f G
 template <typename R>
@@ -1113,10 +1130,11 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
     const int n0 = it.n0, nr = it.nr, lgnr = it.lgnr;
     const int lgp = lgnr - 1, npairs = nr >> 1;
     cpx<R>* A = reinterpret_cast<cpx<R>*>(smem);
-    cpx<R>* Bf = A + (size_t)nr * nx;
+    // double transforms take row pairs throughout, float ones up to a transform per row
+    cpx<R>* Bf = A + (size_t)(sizeof(R) == 8 ? npairs : nr) * nx;
     cpx<R>* Mb = p.M + p.moff[b];
     R* Ub = p.U + p.goff[b];
-    int* sc = reinterpret_cast<int*>(Bf + (size_t)nr * nx);  // scales of double transforms
+    int* sc = reinterpret_cast<int*>(Bf + (size_t)npairs * nx);  // scales of double transforms
     constexpr bool kHot = MODE == ROW_NONLIN || MODE == ROW_ADJ;
     R* Ib = p.io ? p.io + p.goff[b] : nullptr;
 
@@ -1183,6 +1201,28 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
             }
             KS_SYNC();
             cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, yv, lgnx, npairs, -1, p.tw, sc, 0, p.twsh, lgnx + 1);  // a4 (x-pass)
+            store_pair_spectra(d, F, Mb, ns, n0, lgp);
+            KS_SYNC();
+            return;
+        }
+        if constexpr (sizeof(R) == 8) {
+            // u of the row pairs, then u^2: its spectrum gives that of u u_x (residual_at)
+            load_pair_spectra(d, Mb, ns, n0, lgp, A);
+            KS_SYNC();
+            cpx<R>* z = fft_any<R, kHot, SWZ, true, false>(A, Bf, lgnx, npairs, +1, p.tw, sc, 0, p.twsh);
+            cpx<R>* Y = (z == A) ? Bf : A;
+            const int tp = npairs * nx;
+            for (int i = KS_TID; i < tp; i += KS_NT) {
+                const int pr = i >> lgnx;
+                const int m = i & (nx - 1);
+                R* ua = Ub + (size_t)(n0 + 2 * pr) * nx;
+                const cpx<R> u = z[i];
+                ua[m] = u.x;
+                ua[nx + m] = u.y;
+                Y[i] = mk<R>(u.x * u.x, u.y * u.y);
+            }
+            KS_SYNC();
+            cpx<R>* F = fft_any<R, kHot, SWZ, false, true>(Y, z, lgnx, npairs, -1, p.tw, sc, 0, p.twsh, lgnx + 1);
             store_pair_spectra(d, F, Mb, ns, n0, lgp);
             KS_SYNC();
             return;
@@ -1652,8 +1692,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                     const cpx<R> ph = norm(F[i], ins);
                     const cpx<R> u = p.uh[bo + (k + ks)];
                     const R bk = -(R)k * w_over_T;            // -omega_k / T
-                    // r_hat = (a + i bk) u_hat - p_hat                                    (a5)
-                    const cpx<R> r = symbol_add(a_lin, bk, u, neg(ph));
+                    const cpx<R> r = residual_at(a_lin, bk, u, ph, rq);  // a5
                     p.rh[bo + (k + ks)] = r;
                     if (fused) acc.add(u, r, k);              // a6: |r|^2, k Im(conj(u) r)
                     x = MODE == COL_RESID_R ? r : mk<R>(-rq * r.y, rq * r.x);  // i q_j r_hat    (a7)
@@ -1794,8 +1833,8 @@ __device__ __forceinline__ void col_group(const Dims& d, const Bufs<double>& p, 
     const double w_over_T = p.wT[(size_t)p.par * d.B + b];
     if constexpr (MODE == COL_RESID) {
         // element n of a column goes to accumulator n mod 128; a warp holds 32 accumulators of one
-        // column (ns >= 32) or the whole of one or more columns
-        const int w = ns < 32 ? ns : 32, seg = ns <= 128 ? ns : 128;
+        // column (ns >= 32)
+        const int seg = ns <= 128 ? ns : 128;
         for (int i0 = tid; i0 < t.n * seg; i0 += CG_THREADS) {  // whole warps: n seg is a multiple of 32
             const int q = i0 / seg, n0 = i0 - q * seg, j = t.j0 + q;
             const double a_lin = p.lin[j], rq = p.qv[j];
@@ -1806,28 +1845,24 @@ __device__ __forceinline__ void col_group(const Dims& d, const Bufs<double>& p, 
                 if (k >= -ks && k <= ks) {
                     const size_t e = bo + (size_t)q * nk + (k + ks);
                     const C u = p.uh[e];
-                    const C r = symbol_add(a_lin, -(double)k * w_over_T, u, neg(F[i]));  // a5
+                    const C r = residual_at(a_lin, -(double)k * w_over_T, u, F[i], rq);  // a5
                     p.rh[e] = r;
                     acc.add(u, r, k);                                                    // a6
                     x = mk<double>(-rq * r.y, rq * r.x);                                 // a7
                 }
                 X[i] = x;
             }
-            for (int o = w >> 1; o > 0; o >>= 1) {
-                acc.J += __shfl_xor_sync(0xffffffffu, acc.J, o);
-                acc.L += __shfl_xor_sync(0xffffffffu, acc.L, o);
-            }
-            if ((tid & (w - 1)) == 0) {
-                const int g = (n0 / w) + 4 * q;
-                red[2 * g] = acc.J;
-                red[2 * g + 1] = acc.L;
-            }
+            const double s2[2] = {acc.J, acc.L};
+            const double k2 = xor_sum_scatter<2>(s2, 16);
+            const int g = (n0 >> 5) + 4 * q;
+            if ((tid & 31) == 0) red[2 * g] = k2;
+            if ((tid & 31) == 16) red[2 * g + 1] = k2;
         }
         __syncthreads();
         if (tid < t.n) {
             // the warps' sums: distances 2 and 1, over those that exist
             const double* s = red + 8 * tid;
-            const int m = seg / w, j = t.j0 + tid;
+            const int m = seg >> 5, j = t.j0 + tid;
             ColAcc<double> acc;
             if (m == 4) {
                 acc.J = (s[0] + s[4]) + (s[2] + s[6]);

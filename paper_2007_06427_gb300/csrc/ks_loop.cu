@@ -724,7 +724,7 @@ int launch_rows(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const int n = (int)h->rows.size();
     LaunchScope ls(h, s, kRowNames[MODE], prec_suffix(pr));
     k_rows<R, MODE><<<std::min(n, l.grid), l.threads, l.smem, s>>>(h->d, p, n, (int)l.tw_off,
-                                                                     std::max(h->d.nx, h->nsmax));
+                                                                     h->d.nx);
     KS_CUDA(cudaGetLastError());
     ls.done();
     return KS_OK;
@@ -741,7 +741,7 @@ int launch_cols(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const int n = col_item_count(h->d, h->xi, MODE);
     LaunchScope ls(h, s, kColNames[MODE], prec_suffix(pr));
     k_cols<R, MODE><<<std::min(n, l.grid), l.threads, l.smem, s>>>(h->d, p, n, (int)l.tw_off,
-                                                                     std::max(h->d.nx, h->nsmax));
+                                                                     h->nsmax);
     KS_CUDA(cudaGetLastError());
     ls.done();
     return KS_OK;
@@ -875,11 +875,9 @@ int cluster_block(const ks_loop* h, int slot, const ClusterPlan& cp) {
     if (h->cthreads != 128) return h->cthreads;
     if (slot == 1) return 160;  // float: warp-owned transforms, never more rounds with 5 warps
     const int nx = h->d.nx;
-    const int lgnx = ilog2(nx);
-    const int zb = cp.rt * ((lgnx & 1) ? nx / 2 : nx / 4);  // transform of u + i u_x, one per row
-    const int pb = (cp.rt / 2) * (nx / 2);                   // row pairs
-    const int cb = cp.ncmax * (cp.nsmax / 2);                // columns (or column pairs)
-    return (zb <= 128 && pb <= 128 && cb <= 128) ? 160 : 128;
+    const int pb = (cp.rt / 2) * (nx / 4);     // row pairs
+    const int cb = cp.ncmax * (cp.nsmax / 4);  // columns (or column pairs)
+    return (pb <= 128 && cb <= 128) ? 160 : 128;
 }
 
 // the cluster kernel of a column scheme and launch-bound variant (see k_cluster)
@@ -1389,17 +1387,17 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
     const int ncolitems = B * h->d.nkx;
     for (int pr = 0; pr < 2; ++pr) {
         const size_t cs = pr == P64 ? sizeof(cpx<double>) : sizeof(cpx<float>);
-        const int nm = std::max(h->d.nx, h->nsmax);
-        const size_t tw_bytes = pr == P64 ? twiddle_bytes<double>(nm, true) : twiddle_bytes<float>(nm, true);
+        auto tw_bytes = [&](int nm) { return pr == P64 ? twiddle_bytes<double>(nm, true) : twiddle_bytes<float>(nm, true); };
         Launch& lr = h->lrow[pr];
         lr.threads = h->d.nx >= 256 ? 256 : 128;
-        lr.tw_off = 2 * (size_t)h->rows_per_tile * h->d.nx * cs + row_extra_bytes(h->rows_per_tile);  // 16-aligned
-        lr.smem = lr.tw_off + tw_bytes;
+        // two buffers of a row pair each (double) or of a row (float), 16-aligned
+        lr.tw_off = (size_t)(pr == P64 ? 1 : 2) * h->rows_per_tile * h->d.nx * cs + row_extra_bytes(h->rows_per_tile);
+        lr.smem = lr.tw_off + tw_bytes(h->d.nx);
         lr.grid = 152 * 16;
         Launch& lc = h->lcol[pr];
         lc.threads = (ncolitems < 152 && h->nsmax >= 256) ? 256 : 128;
         lc.tw_off = (2 * (size_t)h->nsmax * cs + COL_RED_DOUBLES * sizeof(double) + 15) & ~(size_t)15;
-        lc.smem = lc.tw_off + tw_bytes;
+        lc.smem = lc.tw_off + tw_bytes(h->nsmax);
         lc.grid = 152 * 16;
     }
     if ((rc = set_smem_attrs<double>(h)) || (rc = set_smem_attrs<float>(h))) return cleanup(rc);
