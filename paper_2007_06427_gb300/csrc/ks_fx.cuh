@@ -52,14 +52,6 @@ inline fxw fx_words(long double c, long double s) {
     fx_word(s, w.ih, w.il);
     return w;
 }
-// exp(2 pi i t / m), 0 <= t < m (host)
-inline fxw fx_twiddle(int t, int m) {
-    const long double c[4] = {1, 0, -1, 0};
-    if (4 * t % m == 0) return fx_words(c[4 * t / m], c[(4 * t / m + 3) & 3]);
-    const long double a = 6.283185307179586476925286766559006L * t / m;
-    return fx_words(cosl(a), sinl(a));
-}
-
 // The twiddles in the order the passes read them, w_m^t = exp(2 pi i t / m): for each power of
 // four s = 4, 16, 64, 256 the radix-2 pass that ends a transform of length 2 s (w_{2s}^j, j < s),
 // then the radix-4 pass of span s (w_{4s}^{q jm}, q = 1, 2, 3, for jm = 0 .. s - 1: three
@@ -86,21 +78,39 @@ KS_HDX void fx_table_entry(int i, int& t, int& m) {  // entry i is exp(2 pi i t 
     }
 }
 
-inline std::vector<fxw> fx_table() {  // host
-    std::vector<fxw> w(FX_TABLE);
-    for (int i = 0; i < FX_TABLE; ++i) {
-        int t, m;
-        fx_table_entry(i, t, m);
-        w[i] = fx_twiddle(t, m);
-    }
-    return w;
+// The table (host), built once per process: long double functions are software on some machines (1.0 ms for
+// the 1360 entries of each handle on Arm), so 129 angles of the first octant serve all of them.
+inline const std::vector<fxw>& fx_table() {
+    static const std::vector<fxw> table = [] {
+        constexpr int N = 1024, Q = N / 4;
+        std::vector<long double> c(Q + 1), s(Q + 1);
+        for (int t = 0; t <= Q / 2; ++t) {
+            const long double a = 6.283185307179586476925286766559006L * t / N;
+            c[t] = s[Q - t] = t ? cosl(a) : 1;
+            s[t] = c[Q - t] = t ? sinl(a) : 0;
+        }
+        std::vector<fxw> w(FX_TABLE);
+        for (int i = 0; i < FX_TABLE; ++i) {
+            int t, m;
+            fx_table_entry(i, t, m);
+            t *= N / m;
+            const long double x = c[t % Q], y = s[t % Q];
+            switch (t / Q) {
+            case 0: w[i] = fx_words(x, y); break;
+            case 1: w[i] = fx_words(-y, x); break;
+            case 2: w[i] = fx_words(-x, -y); break;
+            default: w[i] = fx_words(y, -x); break;
+            }
+        }
+        return w;
+    }();
+    return table;
 }
 
 // Entry i of the table at tw (the host build of the items has its own).
 KS_HD fxw fx_tw(const cpx<double>* tw, int i) {
 #ifdef KS_HOST_EMULATION
-    static const std::vector<fxw> w = fx_table();
-    return w[i];
+    return fx_table()[i];
 #else
     return reinterpret_cast<const fxw*>(tw)[i];
 #endif

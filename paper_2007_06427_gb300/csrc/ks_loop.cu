@@ -1323,7 +1323,7 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
     {
         std::vector<double> re, im;
         twiddles(re, im);
-        const std::vector<fxw> t64 = fx_table();  // the double transforms' twiddles (ks_fx.cuh)
+        const std::vector<fxw>& t64 = fx_table();  // the double transforms' twiddles (ks_fx.cuh)
         std::vector<cpx<float>> t32(NMAX);
         for (int t = 0; t < NMAX; ++t) {
             t32[t].x = (float)re[t];

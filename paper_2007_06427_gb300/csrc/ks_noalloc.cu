@@ -193,7 +193,7 @@ int na_setup(int dev, unsigned char** base) {
         cudaGetLastError();
         return na_fail(KS_ERR_CUDA, "cudaGetSymbolAddress of the scratch array failed");
     }
-    const std::vector<fxw> tw = fx_table();
+    const std::vector<fxw>& tw = fx_table();
     e = cudaMemcpy(static_cast<unsigned char*>(ptr) + O_TW, tw.data(), tw.size() * sizeof(fxw), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return na_fail(KS_ERR_CUDA, "twiddle upload failed");
     const int rs = (int)(2 * NA_ROWS * NA_NXMAX * sizeof(cpx<double>) + row_extra_bytes(NA_ROWS) + twiddle_bytes<double>(NA_NSMAX, true));
