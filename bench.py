@@ -164,7 +164,7 @@ def kernel_source_hash() -> str:
     kernel), comments and layout excluded; host-side changes leave it unchanged."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("ks_items.cuh", "ks_cluster.cuh"):
+    for f in ("ks_items.cuh", "ks_fx.cuh", "ks_cluster.cuh"):
         with open(os.path.join(ROOT, "paper_2007_06427_gb300", "csrc", f)) as fh:
             h.update(code_tokens(fh.read()).encode())
     return h.hexdigest()[:16]
@@ -415,7 +415,7 @@ def annotate_sms(roof, K, h, mode, batch, dev):
     """For the cluster-resident kernel: the SMs a launch occupies (one CTA per SM; C CTAs per
     loop) and the roofline fraction against the peak of those SMs alone."""
     import torch
-    if not roof or K.ks_get_option(h.handle, "path") != 0:
+    if not roof or K.ks_get_option(h.handle, "path") != 0 or not roof.get("kernel", "cluster").startswith("cluster"):
         return roof
     C = K.ks_get_option(h.handle, "cluster_f32" if mode == K.KS_FP32 else "cluster_f64")
     if C <= 0:
@@ -440,7 +440,7 @@ def add_probe(roof, probe):
 
 def launch_shape(K, h, mode, autotuned):
     sfx = "f32" if mode == K.KS_FP32 else "f64"
-    path = K.ks_get_option(h.handle, "path")
+    path = K.ks_get_option(h.handle, "form_" + sfx)
     cl = path == 0 and K.ks_get_option(h.handle, "cluster_" + sfx) > 0  # the cluster kernel runs
     return {"path": path,
             "cluster": K.ks_get_option(h.handle, "cluster_" + sfx),

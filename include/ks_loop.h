@@ -203,12 +203,17 @@ KS_API int ks_profile_read(ks_loop_t h, int n, char* names, double* ms, long lon
  *                    "graph").  All three give bit-identical results.
  *   "path_f64", "path_f32"  the same for the double or the float steps alone (the loops of a
  *                    KS_MIXED batch in each precision are stepped by their own precision's form).
- *                    Default at create, with P = Nx * max Ns (the faster form in measurements on
- *                    GB300): 2 for ragged batches (unequal Ns) of 64 or more loops; double: 2
- *                    when P >= 16384, or P >= 8192 in batches of 8 or more, or when the cluster
- *                    plan has 1 or 2 CTAs per loop on P >= 4096 in a batch; float: 2 when
- *                    P >= 32768, or P >= 16384 in batches of 64 or more; else 0.  ks_autotune
+ *                    Value at create, with P = Nx * max Ns: 2 for ragged batches (unequal Ns) of
+ *                    64 or more loops; double: 2 when P >= 16384, or P >= 8192 in batches of 8 or
+ *                    more, or when the cluster plan has 1 or 2 CTAs per loop on P >= 4096; float:
+ *                    2 when P >= 32768, or P >= 16384 in batches of 64 or more; else 0.  Until one
+ *                    of these knobs is set, the steps take the faster of forms 0 and 2 by a rule on
+ *                    the points of a loop per CTA of its cluster (see "form_f64").  ks_autotune
  *                    replaces the bulk precision's form (float for KS_MIXED) by timing.
+ *   "path_auto"      bit 0 (double) and bit 1 (float): that precision's path has not been set.
+ *                    Setting a path clears its bit; setting the bit returns to the rule.
+ *   "form_f64", "form_f32"  (read only) the form the steps of that precision take now, with the
+ *                    fallbacks of path 0 and 1 applied
  *   "persistent"     1: path 1, 0: path 2 (older spelling of "path")
  *   "row_threads", "col_threads"  path 2: threads per block of the row and column items, 128
  *                    or 256 (results are bit-identical: a column's partials of J and L^dag_2

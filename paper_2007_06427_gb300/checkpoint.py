@@ -31,7 +31,7 @@ VERSION = 2
 # knobs of ks_set_option that change how the descent proceeds (saved and restored)
 KNOBS = ("symmetry", "extrapolate", "extrapolate_start_ppm", "extrapolate_drop_ppm",
          "stall_window", "stall_drop_ppm", "finish_f32_adjoint", "switch_probe",
-         "switch_probe_steps", "chunk", "path_f64", "path_f32", "graph")
+         "switch_probe_steps", "chunk", "path_f64", "path_f32", "path_auto", "graph")
 
 
 def save(loop: "K.KSLoop", path: str, tol: float = 1e-10, switch_tol: float = 0.0) -> None:

@@ -336,6 +336,7 @@ struct ks_loop {
     // launch path of each precision (index P64, P32): 0 = cluster-resident kernel when its plan
     // fits, else 1; 1 = grid-persistent cooperative kernel; 2 = four launches per tau-step
     int path[2] = {0, 0};
+    int path_auto = 0;              // bit pr: path[pr] has not been set, the steps take auto_form
     int force_cluster = 0;          // 0: choose the cluster size; else use this one
     int cexchange = 1;              // cluster kernel: mbarrier exchanges where the plan has room
     int force_mb = 0;               // cluster kernel variant: 0 by occupancy, 1 or 2 forced
@@ -958,23 +959,10 @@ int setup_cluster(ks_loop* h) {
     return KS_OK;
 }
 
-// Default launch form of each precision's steps (the "path" knob, set per precision), from
-// steady-state step times on GB300 of the cluster-resident kernel against the four-launch form
-// replayed as graphs, over loops of 32x64 to 256x1024 points in batches of 1-128 (and ragged
-// batches of 64-1024 loops).  All forms compute the same bits, so this only sets the speed.
-// P = Nx * max Ns, the points of the longest loop:
-//   * ragged batches (loops of unequal Ns) of 64 or more loops: four launches per step.  One
-//     cluster per loop leaves the SMs that hold the long loops working while the rest idle;
-//   * double: four launches once P >= 16384, or P >= 8192 in batches of 8 or more, or when the
-//     cluster plan has 1 or 2 CTAs per loop on P >= 4096 in a batch.  A double loop of that size
-//     keeps each CTA of its cluster busy for long serial transforms (64x256 single loop: 54 us
-//     per step resident, 38 us in four launches; 256x256: 192 against 45);
-//   * float: four launches once P >= 32768, or P >= 16384 in batches of 64 or more (float
-//     transforms are short enough that the resident kernel's saved launches and round trips to
-//     memory win up to there: 64x256 x 32 loops 29.7 against 30.4 us; 256x1024 x 8 loops 305
-//     against 83);
-//   * otherwise the cluster-resident kernel.
-// ks_autotune replaces the choice of the handle's bulk precision by timing.
+// The "path" knob a handle is created with, per precision (P = Nx * max Ns): 2 for ragged batches of
+// 64 or more loops; double: P >= 16384, P >= 8192 in batches of 8 or more, or 1 or 2 CTAs a loop on
+// P >= 4096; float: P >= 32768, or P >= 16384 in batches of 64 or more; else 0.  Callers read it; until
+// it is set, the steps take the form of auto_form.
 int default_path(const ks_loop* h, int pr) {
     const int B = h->d.B;
     bool ragged = false;
@@ -990,10 +978,40 @@ int default_path(const ks_loop* h, int pr) {
     return (P >= 32768 || (P >= 16384 && B >= 64)) ? 2 : 0;
 }
 
+// The form of a handle whose "path" knob is not set, from step times on GB300 over loops of 32x32 to
+// 256x512 points, batches of 1 to 2048, in and outside the subspace.  All forms compute the same bits.
+//   * Ragged batches of 64 or more loops: four launches.  One cluster a loop leaves the SMs of the long
+//     loops working while the rest idle.
+//   * Otherwise by the points of a CTA's share of a loop, Q = P / C, and by whether all clusters of the
+//     batch are resident.  The cluster kernel's step grows with Q, its transforms shared by four warps,
+//     and with the waves; four launches have a floor (double 40 us, float 18 to 28) and fill the GPU.
+//     Double: four launches from Q = 2048 on (us a step, cluster against four launches: Q = 1024: one
+//     64x256 loop 29.3 / 43.0, 32 64x128 loops 35.8 / 47.7; Q = 2048: one 128x256 loop 51.2 / 44.6, 256
+//     32x64 loops 71.3 / 62.8), and from 512 on where the clusters take several waves (16 64x256 loops
+//     65.6 / 48.6, 1024 16x32 loops 92.3 / 61.9, but 1024 16x16 loops 68.4 / 94.1).
+//     Float, with its phases in registers (use_rg): from Q = 4096 on (256 64x64 loops 60.3 / 26.3, one
+//     256x256 loop 39.0 / 28.9), from Q = 2048 on in clusters of fewer than 16 CTAs or in waves (256
+//     64x32 loops 38.3 / 25.8, 64 256x32 loops 38.9 / 24.5, 16 128x256 loops 47.3 / 29.7, but one 128x256
+//     loop 20.5 / 27.1) and from 1024 on in waves (512 32x32 loops 46.9 / 30.9).  Float with the items
+//     (the subspace): from Q = 4096 on (256 64x128 loops 129 / 58), and from Q = 2048 on in waves.
+int auto_form(const ks_loop* h, int pr) {
+    const int B = h->d.B;
+    const ClusterPlan& cp = h->cplan[pr];
+    bool ragged = false;
+    for (int b = 1; b < B; ++b) ragged |= (h->ns[b] != h->ns[0]);
+    if (ragged && B >= 64) return 2;
+    if (h->force_cluster || !cp.bytes) return h->path[pr];
+    const long long Q = (long long)h->d.nx * h->nsmax / cp.C;
+    const bool waves = h->cgrid[pr] < cp.C * B;
+    if (pr == P64) return Q >= (waves ? 512 : 2048) ? 2 : 0;
+    if (use_rg(h)) return Q >= (waves ? 1024 : cp.C < 16 ? 2048 : 4096) ? 2 : 0;
+    return Q >= (waves ? 2048 : 4096) ? 2 : 0;
+}
+
 // the launch form precision pr's steps take: 0 cluster-resident (where its plan fits), 1
 // grid-persistent (where its cooperative grid fits), 2 four launches per step
 int form_of(const ks_loop* h, int pr) {
-    const int p = h->path[pr];
+    const int p = h->path_auto >> pr & 1 ? auto_form(h, pr) : h->path[pr];
     if (p == 0 && h->cplan[pr].bytes > 0) return 0;
     if (p <= 1 && h->pgrid[pr] > 0) return 1;
     return 2;
@@ -1413,6 +1431,7 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
     h->h_steps.assign(B, 0);
     h->path[P64] = default_path(h, P64);
     h->path[P32] = default_path(h, P32);
+    h->path_auto = 3;
     if (h->autotune && (rc = ks_autotune_impl(h))) return cleanup(rc);
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cleanup(fail(KS_ERR_CUDA, cudaGetErrorString(e)));
@@ -2437,10 +2456,17 @@ extern "C" int ks_set_option(ks_loop_t h, const char* key, long long value) {
     const std::string k(key);
     if (k == "persistent") {
         h->path[P64] = h->path[P32] = value ? 1 : 2;
+        h->path_auto = 0;
     } else if (k == "path" || k == "path_f64" || k == "path_f32") {
         if (value < 0 || value > 2) return fail(KS_ERR_ARG, "path must be 0, 1 or 2");
-        if (k != "path_f32") h->path[P64] = (int)value;
-        if (k != "path_f64") h->path[P32] = (int)value;
+        for (int pr : {P64, P32})
+            if (k != (pr == P64 ? "path_f32" : "path_f64")) {
+                h->path[pr] = (int)value;
+                h->path_auto &= ~(1 << pr);
+            }
+    } else if (k == "path_auto") {
+        if (value < 0 || value > 3) return fail(KS_ERR_ARG, "path_auto must be 0..3 (bit 0 double, bit 1 float)");
+        h->path_auto = (int)value;
     } else if (k == "cluster") {
         if (value < 0 || value > 16) return fail(KS_ERR_ARG, "cluster must be 0 (auto) or 1..16");
         h->force_cluster = (int)value;
@@ -2510,6 +2536,9 @@ extern "C" int ks_get_option(ks_loop_t h, const char* key, long long* value) {
     if (k == "path") *value = h->path[h->mode == KS_FP64 ? P64 : P32];
     else if (k == "path_f64") *value = h->path[P64];
     else if (k == "path_f32") *value = h->path[P32];
+    else if (k == "path_auto") *value = h->path_auto;
+    else if (k == "form_f64") *value = form_of(h, P64);
+    else if (k == "form_f32") *value = form_of(h, P32);
     else if (k == "cluster_f64") *value = h->cplan[0].bytes ? h->cplan[0].C : 0;
     else if (k == "cluster_f32") *value = h->cplan[1].bytes ? h->cplan[1].C : 0;
     else if (k == "cluster_smem_f64") *value = h->cplan[0].bytes;
@@ -2627,6 +2656,7 @@ void cache_store(const std::string& key, const TuneChoice& c) {
 int apply_choice(ks_loop* h, const TuneChoice& c) {
     h->path[P32] = c.path;
     if (h->mode != KS_MIXED) h->path[P64] = c.path;
+    h->path_auto &= h->mode != KS_MIXED ? 0 : 1 << P64;
     h->force_cluster = c.cluster;
     h->cthreads = c.threads;
     KS_TRY((setup_cluster<double, double>(h)));
