@@ -598,6 +598,12 @@ __device__ __forceinline__ void cp_async(void* smem_dst, const void* gsrc) {
 
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
+// Launches linked to the one in front of them (launch_linked): wait until it has completed and its
+// stores are visible; let the one behind start as soon as this launch's blocks are all resident.
+// Without the link the first does nothing.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;\n"); }
+
 // The twiddles a transform of length n <= nm reads: entries t of exp(2 pi i t / NMAX) with t a
 // multiple of NMAX / n (every pass indexes the table by multiples of NMAX / (4 span) or more, and
 // 4 span <= n), hence of NMAX / nm.  Only those entries are copied into the shared-memory copy

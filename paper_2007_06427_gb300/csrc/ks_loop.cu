@@ -29,6 +29,7 @@ using namespace ks;
 // Per-phase launches.  Each CTA first copies the twiddles its transforms read (nm entries,
 // nm = the longest transform) into a compact bank-swizzled table at tw_off, after its item
 // buffers; the items read them there (the same values as the global table: the same bits).
+// The tables are constant, so they are staged before the wait for the launch in front (launch_linked).
 template <typename R>
 __device__ __forceinline__ Bufs<R> stage_twiddles(const Bufs<R>& p, unsigned char* smem,
                                                   int tw_off, int nm) {
@@ -36,6 +37,7 @@ __device__ __forceinline__ Bufs<R> stage_twiddles(const Bufs<R>& p, unsigned cha
     load_twiddles_compact(tws, p.tw, nm);
     cp_async_wait();
     __syncthreads();
+    grid_wait();
     Bufs<R> q = p;
     q.tw = tws;
     q.twsh = __ffs(NMAX / nm) - 1;
@@ -45,6 +47,7 @@ __device__ __forceinline__ Bufs<R> stage_twiddles(const Bufs<R>& p, unsigned cha
 template <typename R, int MODE>
 __global__ void __launch_bounds__(256) k_rows(Dims d, Bufs<R> p, int nitems, int tw_off, int nm) {
     extern __shared__ __align__(16) unsigned char smem[];
+    grid_trigger();
     const Bufs<R> q = stage_twiddles(p, smem, tw_off, nm);
     if constexpr (MODE == ROW_ANALYZE) {
         if (p.Tin)
@@ -74,6 +77,7 @@ __global__ void __launch_bounds__(256) k_rows(Dims d, Bufs<R> p, int nitems, int
 template <typename R, int MODE>
 __global__ void __launch_bounds__(256) k_cols(Dims d, Bufs<R> p, int nitems, int tw_off, int nm) {
     extern __shared__ __align__(16) unsigned char smem[];
+    grid_trigger();
     const Bufs<R> q = stage_twiddles(p, smem, tw_off, nm);
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) col_item<R, MODE, true>(d, q, it, smem, q.par);
 }
@@ -83,6 +87,7 @@ template <int MODE>
 __global__ void __launch_bounds__(CG_THREADS) k_cols_g(Dims d, Bufs<double> p, const ColTile* tiles, int ntiles,
                                                        int pts, int tw_off, int nm) {
     extern __shared__ __align__(16) unsigned char smem[];
+    grid_trigger();
     const Bufs<double> q = stage_twiddles(p, smem, tw_off, nm);
     for (int it = blockIdx.x; it < ntiles; it += gridDim.x) {
         const ColTile t = tiles[it];
@@ -336,6 +341,7 @@ struct ks_loop {
     // launch path of each precision (index P64, P32): 0 = cluster-resident kernel when its plan
     // fits, else 1; 1 = grid-persistent cooperative kernel; 2 = four launches per tau-step
     int path[2] = {0, 0};
+    bool linked = false;            // see launch_linked
     int path_auto = 0;              // bit pr: path[pr] has not been set, the steps take auto_form
     int force_cluster = 0;          // 0: choose the cluster size; else use this one
     int cexchange = 1;              // cluster kernel: mbarrier exchanges where the plan has room
@@ -611,6 +617,36 @@ struct LaunchScope {
     }
 };
 
+// Launch of a phase kernel.  linked: the launch in front of it in stream s is a phase kernel too; it may
+// then start while that one ends (programmatic dependent launch): its blocks stage their tables and
+// wait (grid_wait, in every phase kernel) until the launch in front has completed, which had waited
+// for its own.  A 32x32 residual, five launches: 36.9 -> 29.3 us a call; 40 double steps of 256 ragged
+// loops: 5921 -> 5837.  The float phases link launches of at most a block per SM: larger ones place
+// their early blocks on the SMs that happen to be free first, and stay uneven (120 float steps of the
+// ragged loops, some 450 blocks a launch: 6106 -> 6572 us).
+template <typename R, typename... KA, typename... A>
+cudaError_t launch_linked(const ks_loop* h, void (*k)(KA...), int grid, int block, size_t smem, cudaStream_t s,
+                          const A&... a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = h->linked && !h->prof && (sizeof(R) == 8 || grid <= 152) ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, KA(a)...);
+}
+
+// The launches while this lives are linked.
+struct Linked {
+    ks_loop* h;
+    explicit Linked(ks_loop* h_) : h(h_) { h->linked = true; }
+    ~Linked() { h->linked = false; }
+};
+
 const char* prec_suffix(int pr) { return pr == 0 ? "_f64" : "_f32"; }
 
 // The float phases of a step take the register kernels wherever their lengths are covered, except
@@ -623,14 +659,12 @@ template <int MODE>
 int launch_rg_rows(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
     const int n = h->rg_nrow, per = RG_THREADS / 32, g = (n + per - 1) / per;
     LaunchScope ls(h, s, kRowNames[MODE], prec_suffix(P32));
-    switch (h->d.lgnx) {
-    case 5: k_rg_rows<MODE, 5><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
-    case 6: k_rg_rows<MODE, 6><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
-    case 7: k_rg_rows<MODE, 7><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
-    case 8: k_rg_rows<MODE, 8><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
-    default: k_rg_rows<MODE, 9><<<g, RG_THREADS, 0, s>>>(h->d, p, h->d_rg_rows, n, h->d_rg_tab); break;
-    }
-    KS_CUDA(cudaGetLastError());
+    auto* const k = h->d.lgnx == 5   ? k_rg_rows<MODE, 5>
+                    : h->d.lgnx == 6 ? k_rg_rows<MODE, 6>
+                    : h->d.lgnx == 7 ? k_rg_rows<MODE, 7>
+                    : h->d.lgnx == 8 ? k_rg_rows<MODE, 8>
+                                     : k_rg_rows<MODE, 9>;
+    KS_CUDA(launch_linked<float>(h, k, g, RG_THREADS, 0, s, h->d, p, h->d_rg_rows, n, h->d_rg_tab));
     ls.done();
     return KS_OK;
 }
@@ -640,8 +674,8 @@ int launch_rg_cols(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
     const int n = h->rg_ncol, per = RG_THREADS / 64, g = (n + per - 1) / per;
     LaunchScope ls(h, s, kColNames[MODE], prec_suffix(P32));
     const size_t smem = (size_t)h->rg_ntab * sizeof(rgv) + (size_t)per * RG_XBYTES;
-    k_rg_cols<MODE><<<g, RG_THREADS, smem, s>>>(h->d, p, h->d_rg_cols, n, h->d_rg_tab, h->rg_ntab);
-    KS_CUDA(cudaGetLastError());
+    KS_CUDA(launch_linked<float>(h, k_rg_cols<MODE>, g, RG_THREADS, smem, s, h->d, p, h->d_rg_cols, n, h->d_rg_tab,
+                          h->rg_ntab));
     ls.done();
     return KS_OK;
 }
@@ -709,9 +743,8 @@ int setup_cg(ks_loop* h) {
 template <int MODE>
 int launch_cols_g(ks_loop* h, const Bufs<double>& p, cudaStream_t s) {
     LaunchScope ls(h, s, kColNames[MODE], prec_suffix(P64));
-    k_cols_g<MODE><<<h->ncg, CG_THREADS, h->cg_smem, s>>>(h->d, p, h->d_cg, h->ncg, h->cg_pts, (int)h->cg_tw_off,
-                                                          h->nsmax);
-    KS_CUDA(cudaGetLastError());
+    KS_CUDA(launch_linked<double>(h, k_cols_g<MODE>, h->ncg, CG_THREADS, h->cg_smem, s, h->d, p, h->d_cg, h->ncg, h->cg_pts,
+                          (int)h->cg_tw_off, h->nsmax));
     ls.done();
     return KS_OK;
 }
@@ -724,9 +757,8 @@ int launch_rows(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const Launch& l = h->lrow[pr];
     const int n = (int)h->rows.size();
     LaunchScope ls(h, s, kRowNames[MODE], prec_suffix(pr));
-    k_rows<R, MODE><<<std::min(n, l.grid), l.threads, l.smem, s>>>(h->d, p, n, (int)l.tw_off,
-                                                                     h->d.nx);
-    KS_CUDA(cudaGetLastError());
+    KS_CUDA(launch_linked<R>(h, k_rows<R, MODE>, std::min(n, l.grid), l.threads, l.smem, s, h->d, p, n, (int)l.tw_off,
+                          h->d.nx));
     ls.done();
     return KS_OK;
 }
@@ -741,9 +773,8 @@ int launch_cols(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const Launch& l = h->lcol[pr];
     const int n = col_item_count(h->d, h->xi, MODE);
     LaunchScope ls(h, s, kColNames[MODE], prec_suffix(pr));
-    k_cols<R, MODE><<<std::min(n, l.grid), l.threads, l.smem, s>>>(h->d, p, n, (int)l.tw_off,
-                                                                     h->nsmax);
-    KS_CUDA(cudaGetLastError());
+    KS_CUDA(launch_linked<R>(h, k_cols<R, MODE>, std::min(n, l.grid), l.threads, l.smem, s, h->d, p, n, (int)l.tw_off,
+                          h->nsmax));
     ls.done();
     return KS_OK;
 }
@@ -1083,6 +1114,7 @@ int run_analyze(ks_loop* h, Work& w, double* io, const float* iof, const double*
     p.iof = iof;
     p.uhf = iof ? (cpx<float>*)w.uh[P32] : nullptr;
     KS_TRY((launch_rows<double, ROW_ANALYZE>(h, p, s)));
+    const Linked linked(h);
     const bool fuse = prime && !iof && !h->xi;
     if (fuse) KS_TRY((launch_cols<double, COL_ANALYZE_U>(h, p, s)));
     else KS_TRY((launch_cols<double, COL_ANALYZE>(h, p, s)));
@@ -1111,11 +1143,15 @@ int run_prime(ks_loop* h, Work& w, int pr, cudaStream_t s) {
     return KS_OK;
 }
 
-// one tau-step of every live loop of precision pr (M must hold s-inverse of u_hat)
+// one tau-step of every live loop of precision pr (M must hold s-inverse of u_hat); chained: the launch
+// in front of it in s is the end of the step before
 template <typename R>
-int run_step(ks_loop* h, Work& w, int pr, double tol, double switch_tol, cudaStream_t s) {
+int run_step(ks_loop* h, Work& w, int pr, double tol, double switch_tol, cudaStream_t s, bool chained) {
     Bufs<R> p = make_bufs<R>(h, w, pr, 1, tol, switch_tol, (R*)nullptr);
+    const Linked linked(h);
+    h->linked = chained;
     KS_TRY((launch_rows<R, ROW_NONLIN>(h, p, s)));
+    h->linked = true;
     KS_TRY((launch_cols<R, COL_RESID>(h, p, s)));
     KS_TRY((launch_rows<R, ROW_ADJ>(h, p, s)));
     KS_TRY((launch_cols<R, COL_UPDATE>(h, p, s)));
@@ -1125,13 +1161,18 @@ int run_step(ks_loop* h, Work& w, int pr, double tol, double switch_tol, cudaStr
 // residual pass (no update): J partials and r_hat for every loop of the workspace; M holds the
 // s-inverse of u_hat when mix_valid says so.  CMODE: COL_RESID (M = the input of ROW_ADJ),
 // COL_RESID_R (M = s-inverse of r_hat) or COL_RESID_J (the rest alone); in the subspace COL_RESID
-// stands in for all.
+// stands in for all.  chained: the launch in front in s is a phase kernel (the analysis).
 template <typename R, int CMODE>
-int run_residual(ks_loop* h, Work& w, int pr, cudaStream_t s) {
+int run_residual(ks_loop* h, Work& w, int pr, cudaStream_t s, bool chained = false) {
     Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, (R*)nullptr);
-    if (!w.mix_valid[pr]) KS_TRY((launch_cols<R, COL_SYNTH_U>(h, p, s)));
+    const bool primed = w.mix_valid[pr];
+    const Linked linked(h);
+    h->linked = chained;
+    if (!primed) KS_TRY((launch_cols<R, COL_SYNTH_U>(h, p, s)));
+    h->linked = chained || !primed;
     w.mix_valid[pr] = false;
     KS_TRY((launch_rows<R, ROW_NONLIN>(h, p, s)));
+    h->linked = true;
     if (h->xi) KS_TRY((launch_cols<R, COL_RESID>(h, p, s)));
     else KS_TRY((launch_cols<R, CMODE>(h, p, s)));
     return KS_OK;
@@ -1140,7 +1181,8 @@ int run_residual(ks_loop* h, Work& w, int pr, cudaStream_t s) {
 // M = the s-inverse of G_hat, for the synthesis of G
 template <typename R>
 int run_gradient(ks_loop* h, Work& w, int pr, cudaStream_t s) {
-    KS_TRY((run_residual<R, COL_RESID>(h, w, pr, s)));
+    KS_TRY((run_residual<R, COL_RESID>(h, w, pr, s, true)));
+    const Linked linked(h);
     Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, (R*)nullptr);
     KS_TRY((launch_rows<R, ROW_ADJ>(h, p, s)));
     if (!h->xi) return launch_cols<R, COL_GRAD_G>(h, p, s);
@@ -1155,6 +1197,7 @@ int run_rows_out(ks_loop* h, Work& w, int pr, R* io, double* J, double* dJdT, cu
     p.fin = 1;
     p.Jout = J;
     p.dJdTout = dJdT;
+    const Linked linked(h);
     return launch_rows<R, ROW_SYNTH>(h, p, s);
 }
 
@@ -1469,10 +1512,10 @@ double* out_ptr(double* user, double* own) { return user && is_device_ptr(user) 
 template <typename R>
 int residual_call(ks_loop* h, Work& w, int pr, void* r, double* J, cudaStream_t s) {
     if (!r) {
-        KS_TRY((run_residual<R, COL_RESID_J>(h, w, pr, s)));
+        KS_TRY((run_residual<R, COL_RESID_J>(h, w, pr, s, true)));
         return J ? run_finalize(h, w, w.T, pr, 0, s, J) : KS_OK;
     }
-    KS_TRY((run_residual<R, COL_RESID_R>(h, w, pr, s)));
+    KS_TRY((run_residual<R, COL_RESID_R>(h, w, pr, s, true)));
     if (h->xi) {
         Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, (R*)nullptr);
         KS_TRY((launch_cols<R, COL_SYNTH_R>(h, p, s)));
@@ -1661,8 +1704,8 @@ int step_graph(ks_loop* h, Work& w, const bool* live, double tol, double swt, in
             }
             s64 = h->gcap2;
         }
-        if (live[P32]) rc = run_step<float>(h, w, P32, tol, swt, h->gcap);
-        if (rc == KS_OK && live[P64]) rc = run_step<double>(h, w, P64, tol, 0.0, s64);
+        if (live[P32]) rc = run_step<float>(h, w, P32, tol, swt, h->gcap, i > 0 && !both);
+        if (rc == KS_OK && live[P64]) rc = run_step<double>(h, w, P64, tol, 0.0, s64, i > 0 && !both);
         if (rc == KS_OK && both &&
             (cudaEventRecord(h->gjoin, h->gcap2) != cudaSuccess ||
              cudaStreamWaitEvent(h->gcap, h->gjoin, 0) != cudaSuccess))
@@ -1719,8 +1762,8 @@ int phase_steps(ks_loop* h, Work& w, const bool* live, long long n, double tol, 
         }
     }
     for (; i < n; ++i) {
-        if (live[P32]) KS_TRY(run_step<float>(h, w, P32, tol, swt, s));
-        if (live[P64]) KS_TRY(run_step<double>(h, w, P64, tol, 0.0, s));
+        if (live[P32]) KS_TRY(run_step<float>(h, w, P32, tol, swt, s, false));
+        if (live[P64]) KS_TRY(run_step<double>(h, w, P64, tol, 0.0, s, false));
         w.par ^= 1;
     }
     return KS_OK;

@@ -318,8 +318,10 @@ __global__ void __launch_bounds__(RG_THREADS) k_rg_rows(Dims d, Bufs<float> p, c
                                                         const rgv* tab) {
     __shared__ rgv xs[RG_THREADS / 64 * (RG_XBYTES / 8)];
     __shared__ rgv tws[rg_len(LGX)];
+    grid_trigger();
     for (int i = threadIdx.x; i < rg_len(LGX); i += RG_THREADS) tws[i] = tab[rg_at(LGX) + i];
     __syncthreads();
+    grid_wait();
     const int w = threadIdx.x >> 5;
     rgv* x = xs + w * (RG_XBYTES / 16);
     for (int it = blockIdx.x * (RG_THREADS / 32) + w; it < ntiles; it += gridDim.x * (RG_THREADS / 32)) {
@@ -500,8 +502,10 @@ __global__ void __launch_bounds__(RG_THREADS) k_rg_cols(Dims d, Bufs<float> p, c
     extern __shared__ __align__(16) unsigned char smem[];
     rgv* tws = reinterpret_cast<rgv*>(smem);
     rgv* xs = tws + ntab;
+    grid_trigger();
     for (int i = threadIdx.x; i < ntab; i += RG_THREADS) tws[i] = tab[i];
     __syncthreads();
+    grid_wait();
     const int half = threadIdx.x >> 6, w = (threadIdx.x >> 5) & 1;
     for (int it = blockIdx.x * (RG_THREADS / 64) + half; it < npairs; it += gridDim.x * (RG_THREADS / 64)) {
         const bool both = p.lgns[tiles[2 * it].b] == 10;
