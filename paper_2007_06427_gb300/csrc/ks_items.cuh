@@ -193,7 +193,12 @@ KS_HD ff two_sum(float a, float b) {
 KS_HD ff ff_add(ff a, ff b) {
     const ff s = two_sum(a.hi, b.hi);
     const float e = s.lo + (a.lo + b.lo);
-    return two_sum(s.hi, e);
+    // s.hi is a multiple of the last place of e (or 0), so three operations give the exact error of
+    // the last sum, as the six of two_sum would
+    ff r;
+    r.hi = s.hi + e;
+    r.lo = e - (r.hi - s.hi);
+    return r;
 }
 KS_HD ff two_prod(float a, float b) {
     const float p = mul_rn(a, b);

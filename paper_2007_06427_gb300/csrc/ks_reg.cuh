@@ -496,8 +496,12 @@ struct RgCol {
     int b, j0;
 };
 
+//
+// Three blocks an SM (168 registers, a 48-byte spill in COL_RESID): left at 222 to 231 registers two fit,
+// and the 352 blocks of 256 ragged loops or the 344 of eight 256x1024 loops took a second wave for the
+// last 40 (120 and 60 steps: 6093 -> 5253 us, 3269 -> 2680 us, ff_add's shorter sum included).
 template <int MODE>
-__global__ void __launch_bounds__(RG_THREADS) k_rg_cols(Dims d, Bufs<float> p, const RgCol* tiles, int npairs,
+__global__ void __launch_bounds__(RG_THREADS, 3) k_rg_cols(Dims d, Bufs<float> p, const RgCol* tiles, int npairs,
                                                         const rgv* tab, int ntab) {
     extern __shared__ __align__(16) unsigned char smem[];
     rgv* tws = reinterpret_cast<rgv*>(smem);
