@@ -218,9 +218,9 @@ KS_API int ks_profile_read(ks_loop_t h, int n, char* names, double* ms, long lon
  *   "row_threads", "col_threads"  path 2: threads per block of the row and column items, 128
  *                    or 256 (results are bit-identical: a column's partials of J and L^dag_2
  *                    keep 128 accumulators at either size).  Default at create: 256-thread rows
- *                    for Nx >= 256; 256-thread columns when the batch has fewer than 152 column
- *                    items (loops x retained x-modes, one per SM of a GB300) and max Ns >= 256;
- *                    else 128.
+ *                    for Nx >= 256; 256-thread columns for max Ns >= 256 when the batch has fewer
+ *                    than 152 column items (loops x retained x-modes, one per SM of a GB300), in
+ *                    double also when it has fewer than 400 or max Ns = 1024; else 128.
  *   "cluster"        0 (default): cluster size chosen per precision; 1..16: force this size
  *                    (KS_ERR_ARG when no plan of that size fits the batch)
  *   "cluster_exchange" 1 (default): the cluster kernel's DSMEM exchanges are asynchronous

@@ -1456,7 +1456,10 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
         lr.smem = lr.tw_off + tw_bytes(h->d.nx);
         lr.grid = 152 * 16;
         Launch& lc = h->lcol[pr];
-        lc.threads = (ncolitems < 152 && h->nsmax >= 256) ? 256 : 128;
+        // 256 threads where the columns are few for the SMs or long. Double, us a step of four launches
+        // with 128 and 256 threads: 8 loops of 128x512 (344 columns) 99.5 / 73.3, 8 of 256x1024 (688)
+        // 183 / 159, 4 of 128x256 (172) 57.4 / 51.8, but 32 of 64x512 (704) 101.7 / 108.1.
+        lc.threads = h->nsmax >= 256 && (ncolitems < 152 || (pr == P64 && (ncolitems < 400 || h->nsmax >= 1024))) ? 256 : 128;
         lc.tw_off = (2 * (size_t)h->nsmax * cs + COL_RED_DOUBLES * sizeof(double) + 15) & ~(size_t)15;
         lc.smem = lc.tw_off + tw_bytes(h->nsmax);
         lc.grid = 152 * 16;
