@@ -141,6 +141,29 @@ __device__ void dns_coefficients(double* coef, int nh, double L, double dt) {
 // dependent FP64 instructions a pass where one thread takes six, on twice the warps.  The values
 // are the same.
 //
+// That is where the block has the threads for it (SPLIT). Where a pass has more butterflies, a thread
+// takes whole ones: their loads and index arithmetic are shared, and its two chains overlap (us a step
+// with one thread a component and a thread a butterfly: 1216 trajectories of 64 modes 33.2 / 27.7, 400 of
+// 128 modes 36.9 / 30.5, 64 of 256 modes 40.5 / 33.4).
+//
+// n butterflies over the block: f(i, c) computes component c of butterfly i, put(i, c, o) stores it.
+template <bool SPLIT, typename F, typename P>
+__device__ __forceinline__ void dns_each(int n, F f, P put) {
+    for (int t = threadIdx.x; t < (SPLIT ? 2 * n : n); t += blockDim.x) {
+        if constexpr (SPLIT) {
+            double o[2];
+            f(t >> 1, t & 1, o);
+            put(t >> 1, t & 1, o);
+        } else {
+            double o[2], q[2];
+            f(t, 0, o);
+            f(t, 1, q);
+            put(t, 0, o);
+            put(t, 1, q);
+        }
+    }
+}
+
 // One component of a butterfly's outputs (c = 0 real, 1 imaginary).
 __device__ __forceinline__ void dns_bfly(cpx<double> v0, cpx<double> v1, cpx<double> w, int c, double& o0,
                                          double& o1) {
@@ -150,28 +173,32 @@ __device__ __forceinline__ void dns_bfly(cpx<double> v0, cpx<double> v1, cpx<dou
 }
 
 // Passes first <= span < last of cnt transforms at a (b scratch); returns where the data is.
+template <bool SPLIT>
 __device__ __forceinline__ cpx<double>* dns_passes(cpx<double>* a, cpx<double>* b, int lg, int cnt, int dir,
                                                    const cpx<double>* tw, int twsh, int first, int last) {
     const int n = 1 << lg, nb = n >> 1;
     for (int span = first; span < last; span <<= 1) {
         const int tu = NMAX / (span * 2);
-        for (int i = threadIdx.x; i < cnt << lg; i += blockDim.x) {
-            const int f = i >> lg, j = (i >> 1) & (nb - 1), c = i & 1;
-            const cpx<double>* s = a + (f << lg);
-            double* d = reinterpret_cast<double*>(b + (f << lg)) + c;
-            const int jm = j & (span - 1), od = ((j - jm) << 1) + jm;
-            if (span > 1) {
-                double o0, o1;
-                dns_bfly(s[j], s[j + nb], twid<double, true>(tw, jm * tu, dir, twsh), c, o0, o1);
-                d[2 * od] = o0;
-                d[2 * (od + span)] = o1;
-            } else {
-                const double v0 = reinterpret_cast<const double*>(s + j)[c];
-                const double v1 = reinterpret_cast<const double*>(s + j + nb)[c];
-                d[2 * od] = v0 + v1;
-                d[2 * od + 2] = v0 - v1;
-            }
-        }
+        dns_each<SPLIT>(
+            cnt << (lg - 1),
+            [&](int i, int c, double (&o)[2]) {
+                const int f = i >> (lg - 1), j = i & (nb - 1);
+                const cpx<double>* s = a + (f << lg);
+                if (span > 1) {
+                    dns_bfly(s[j], s[j + nb], twid<double, true>(tw, (j & (span - 1)) * tu, dir, twsh), c, o[0], o[1]);
+                } else {
+                    const double v0 = reinterpret_cast<const double*>(s + j)[c];
+                    const double v1 = reinterpret_cast<const double*>(s + j + nb)[c];
+                    o[0] = v0 + v1;
+                    o[1] = v0 - v1;
+                }
+            },
+            [&](int i, int c, const double (&o)[2]) {
+                const int f = i >> (lg - 1), j = i & (nb - 1), jm = j & (span - 1), od = ((j - jm) << 1) + jm;
+                double* d = reinterpret_cast<double*>(b + (f << lg)) + c;
+                d[2 * od] = o[0];
+                d[2 * (od + span)] = o[1];
+            });
         __syncthreads();
         cpx<double>* t = a;
         a = b;
@@ -207,7 +234,7 @@ __device__ void dns_norms(const cpx<double>* Y, int nx, int ntraj, double* red) 
 // split into the two members), handed to use(t, j, c, N): component c of mode j of trajectory t.
 // The first pass forms the pair's spectrum as it reads it, the last inverse pass squares what it
 // writes, so that neither takes a round trip of its own.
-template <typename Use>
+template <bool SPLIT, typename Use>
 __device__ __forceinline__ void dns_eval(const DnsArgs& a, int tr0, int ntraj, cpx<double>* fftb,
                                          cpx<double>* specs, const cpx<double>* tw, const double* coef,
                                          double* red, int src, long long isave, bool end, Use use) {
@@ -216,48 +243,58 @@ __device__ __forceinline__ void dns_eval(const DnsArgs& a, int tr0, int ntraj, c
     const int twsh = LGNMAX - lgnx;
     cpx<double>* A = fftb;
     cpx<double>* Bf = fftb + (size_t)a.pairs * nx;
-    for (int i = threadIdx.x; i < np * nx; i += blockDim.x) {
-        const int pr = i >> lgnx, j = (i >> 1) & (nb - 1), c = i & 1;
-        const int ta = 2 * pr, tb = ta + 1;
-        const bool hb = tb < ntraj;
-        const double* sa = reinterpret_cast<const double*>(spec(specs, nh, ta, src));
-        const double* sb = reinterpret_cast<const double*>(spec(specs, nh, tb, src));
-        auto z = [&](int J) {  // component c of v_a + i v_b, or of conj v_a + i conj v_b
-            if (J <= kx) {
-                const double x = sa[2 * J + c], y = hb ? sb[2 * J + 1 - c] : 0.0;
-                return c ? x + y : x - y;
-            }
-            if (J >= nx - kx) {
-                const double x = sa[2 * (nx - J) + c], y = hb ? sb[2 * (nx - J) + 1 - c] : 0.0;
-                return c ? -x + y : x + y;
-            }
-            return 0.0;
-        };
-        const double v0 = z(j), v1 = z(j + nb);
-        double* d = reinterpret_cast<double*>(A + (pr << lgnx) + 2 * j) + c;
-        d[0] = v0 + v1;
-        d[2] = v0 - v1;
-    }
+    dns_each<SPLIT>(
+        np * nb,
+        [&](int i, int c, double (&o)[2]) {
+            const int pr = i >> (lgnx - 1), j = i & (nb - 1);
+            const int ta = 2 * pr, tb = ta + 1;
+            const bool hb = tb < ntraj;
+            const double* sa = reinterpret_cast<const double*>(spec(specs, nh, ta, src));
+            const double* sb = reinterpret_cast<const double*>(spec(specs, nh, tb, src));
+            auto z = [&](int J) {  // component c of v_a + i v_b, or of conj v_a + i conj v_b
+                if (J <= kx) {
+                    const double x = sa[2 * J + c], y = hb ? sb[2 * J + 1 - c] : 0.0;
+                    return c ? x + y : x - y;
+                }
+                if (J >= nx - kx) {
+                    const double x = sa[2 * (nx - J) + c], y = hb ? sb[2 * (nx - J) + 1 - c] : 0.0;
+                    return c ? -x + y : x + y;
+                }
+                return 0.0;
+            };
+            const double v0 = z(j), v1 = z(j + nb);
+            o[0] = v0 + v1;
+            o[1] = v0 - v1;
+        },
+        [&](int i, int c, const double (&o)[2]) {
+            const int pr = i >> (lgnx - 1), j = i & (nb - 1);
+            double* d = reinterpret_cast<double*>(A + (pr << lgnx) + 2 * j) + c;
+            d[0] = o[0];
+            d[2] = o[1];
+        });
     __syncthreads();
-    cpx<double>* Z = dns_passes(A, Bf, lgnx, np, +1, tw, twsh, 2, nb);
+    cpx<double>* Z = dns_passes<SPLIT>(A, Bf, lgnx, np, +1, tw, twsh, 2, nb);
     cpx<double>* Y = Z == A ? Bf : A;
     const double inx = 1.0 / (double)nx;  // exact: nx is a power of two
     const bool save = isave >= 0;
-    for (int i = threadIdx.x; i < np * nx; i += blockDim.x) {  // the pass of span nb
-        const int pr = i >> lgnx, j = (i >> 1) & (nb - 1), c = i & 1;
-        double o[2];
-        dns_bfly(Z[(pr << lgnx) + j], Z[(pr << lgnx) + j + nb],
-                 twid<double, true>(tw, j * (NMAX / nx), +1, twsh), c, o[0], o[1]);
-        const int t = 2 * pr + c;
+    dns_each<SPLIT>(  // the pass of span nb
+        np * nb,
+        [&](int i, int c, double (&o)[2]) {
+            const int pr = i >> (lgnx - 1), j = i & (nb - 1);
+            dns_bfly(Z[(pr << lgnx) + j], Z[(pr << lgnx) + j + nb],
+                     twid<double, true>(tw, j * (NMAX / nx), +1, twsh), c, o[0], o[1]);
+        },
+        [&](int i, int c, const double (&o)[2]) {
+            const int pr = i >> (lgnx - 1), j = i & (nb - 1), t = 2 * pr + c;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int m = j + q * nb;
-            const double u = o[q] * inx;
-            reinterpret_cast<double*>(Y + (pr << lgnx) + m)[c] = u * u;
-            if (save && a.u_saved && t < ntraj) a.u_saved[((size_t)(tr0 + t) * a.nsave + isave) * nx + m] = u;
-            if (end && a.u_end && t < ntraj) a.u_end[(size_t)(tr0 + t) * nx + m] = u;
-        }
-    }
+            for (int q = 0; q < 2; ++q) {
+                const int m = j + q * nb;
+                const double u = o[q] * inx;
+                reinterpret_cast<double*>(Y + (pr << lgnx) + m)[c] = u * u;
+                if (save && a.u_saved && t < ntraj) a.u_saved[((size_t)(tr0 + t) * a.nsave + isave) * nx + m] = u;
+                if (end && a.u_end && t < ntraj) a.u_end[(size_t)(tr0 + t) * nx + m] = u;
+            }
+        });
     __syncthreads();
     if (save && a.norms) {
         dns_norms(Y, nx, ntraj, red);
@@ -266,20 +303,29 @@ __device__ __forceinline__ void dns_eval(const DnsArgs& a, int tr0, int ntraj, c
             a.norms[(size_t)(tr0 + threadIdx.x) * a.nsave + isave] = sqrt(a.L * red[threadIdx.x] * inx);
     }
     if (end) return;
-    const cpx<double>* F = dns_passes(Y, Z, lgnx, np, -1, tw, twsh, 1, nx);
+    const cpx<double>* F = dns_passes<SPLIT>(Y, Z, lgnx, np, -1, tw, twsh, 1, nx);
     const double* g = coef + 6 * nh;
-    for (int i = threadIdx.x; i < ntraj * nh * 2; i += blockDim.x) {
-        const int c = i & 1, t = (i >> 1) / nh, j = (i >> 1) - t * nh;
+    auto give = [&](int t, int j, int c) {
         const cpx<double> P = F[((t >> 1) << lgnx) + j], Q = F[((t >> 1) << lgnx) + ((nx - j) & (nx - 1))];
         // W_a = (P + conj Q) / 2, W_b = (P - conj Q) / (2 i); N = i g W
         const double h = (c ^ (t & 1)) ? P.x : P.y, k = (c ^ (t & 1)) ? Q.x : Q.y;
         // a: W.x = (P.x + Q.x) / 2, W.y = (P.y - Q.y) / 2; b: W.x = (P.y + Q.y) / 2, W.y = -(P.x - Q.x) / 2
         const double W = c ? 0.5 * (h + k) : ((t & 1) ? -0.5 : 0.5) * (h - k);
         use(t, j, c, (c ? g[j] : -g[j]) * W);
+    };
+    for (int i = threadIdx.x; i < ntraj * nh * (SPLIT ? 2 : 1); i += blockDim.x) {
+        const int tj = SPLIT ? i >> 1 : i, t = tj / nh, j = tj - t * nh;
+        if constexpr (SPLIT) {
+            give(t, j, i & 1);
+        } else {
+            give(t, j, 0);
+            give(t, j, 1);
+        }
     }
     __syncthreads();
 }
 
+template <bool SPLIT>
 __global__ void __launch_bounds__(DNS_THREADS) k_dns(DnsArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const DnsPlan pl = dns_plan(a.nx, a.nh, a.pairs);
@@ -313,7 +359,7 @@ __global__ void __launch_bounds__(DNS_THREADS) k_dns(DnsArgs a) {
     }
     __syncthreads();
     {
-        cpx<double>* F = dns_passes(A, Bf, lgnx, np, -1, tw, twsh, 1, nx);
+        cpx<double>* F = dns_passes<SPLIT>(A, Bf, lgnx, np, -1, tw, twsh, 1, nx);
         for (int i = threadIdx.x; i < np * nh; i += blockDim.x) {
             const int pr = i / nh, j = i - pr * nh;
             const cpx<double> P = F[(size_t)pr * nx + j];
@@ -342,21 +388,21 @@ __global__ void __launch_bounds__(DNS_THREADS) k_dns(DnsArgs a) {
     };
     for (long long n = 0; n < a.nsteps; ++n) {
         const long long isave = (n % a.save_every == 0) ? n / a.save_every : -1;
-        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SV, isave, false, [&](int t, int j, int c, double N) {
+        dns_eval<SPLIT>(a, tr0, ntraj, fftb, specs, tw, coef, red, SV, isave, false, [&](int t, int j, int c, double N) {
             at(t, SNV, j, c) = N;
             at(t, SA, j, c) = E2[j] * at(t, SV, j, c) + Q[j] * N;  // a = E2 v + Q Nv
         });
-        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SA, -1, false, [&](int t, int j, int c, double N) {
+        dns_eval<SPLIT>(a, tr0, ntraj, fftb, specs, tw, coef, red, SA, -1, false, [&](int t, int j, int c, double N) {
             at(t, SNA, j, c) = N;
             at(t, SS, j, c) = E2[j] * at(t, SV, j, c) + Q[j] * N;  // b = E2 v + Q Na
         });
-        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SS, -1, false, [&](int t, int j, int c, double N) {
+        dns_eval<SPLIT>(a, tr0, ntraj, fftb, specs, tw, coef, red, SS, -1, false, [&](int t, int j, int c, double N) {
             at(t, SNB, j, c) = N;
             const double d2 = 2.0 * N - at(t, SNV, j, c);          // c = E2 a + Q (2 Nb - Nv)
             at(t, SS, j, c) = E2[j] * at(t, SA, j, c) + Q[j] * d2;
         });
         // v' = E v + f1 Nv + 2 f2 (Na + Nb) + f3 Nc; in the subspace the real parts are zeroed
-        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SS, -1, false, [&](int t, int j, int c, double N) {
+        dns_eval<SPLIT>(a, tr0, ntraj, fftb, specs, tw, coef, red, SS, -1, false, [&](int t, int j, int c, double N) {
             const double w2 = 2.0 * f2[j];
             const double v = at(t, SV, j, c), Nv = at(t, SNV, j, c), Na = at(t, SNA, j, c), Nb = at(t, SNB, j, c);
             const double vn = E[j] * v + f1[j] * Nv + w2 * (Na + Nb) + f3[j] * N;
@@ -365,7 +411,7 @@ __global__ void __launch_bounds__(DNS_THREADS) k_dns(DnsArgs a) {
     }
     const bool save_last = (a.nsteps % a.save_every == 0);
     if (save_last || a.u_end)
-        dns_eval(a, tr0, ntraj, fftb, specs, tw, coef, red, SV, save_last ? a.nsteps / a.save_every : -1, true,
+        dns_eval<SPLIT>(a, tr0, ntraj, fftb, specs, tw, coef, red, SV, save_last ? a.nsteps / a.save_every : -1, true,
                  [](int, int, int, double) {});
 }
 
@@ -511,12 +557,14 @@ extern "C" int ks_dns(double L, int nx, int batch, double dt, long long nsteps, 
     a.u_saved = static_cast<double*>(ssv.dev);
     a.norms = static_cast<double*>(snm.dev);
     a.u_end = static_cast<double*>(sue.dev);
-    if (cudaFuncSetAttribute(k_dns, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.bytes) != cudaSuccess) {
+    // a thread per butterfly component where the block has one for each
+    auto* const kern = pairs * nx <= DNS_THREADS ? k_dns<true> : k_dns<false>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.bytes) != cudaSuccess) {
         cudaGetLastError();
         return dns_fail(KS_ERR_CUDA, "shared-memory attribute of the DNS kernel failed");
     }
     const int grid = (batch + 2 * pairs - 1) / (2 * pairs);
-    k_dns<<<grid, DNS_THREADS, pl.bytes, s>>>(a);
+    kern<<<grid, DNS_THREADS, pl.bytes, s>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return dns_fail(KS_ERR_CUDA, cudaGetErrorString(e));
     rc = su0.finish(s);
