@@ -143,23 +143,28 @@ __device__ void dns_coefficients(double* coef, int nh, double L, double dt) {
 //
 // That is where the block has the threads for it (SPLIT). Where a pass has more butterflies, a thread
 // takes whole ones: their loads and index arithmetic are shared, and its two chains overlap (us a step
-// with one thread a component and a thread a butterfly: 1216 trajectories of 64 modes 33.2 / 27.7, 400 of
-// 128 modes 36.9 / 30.5, 64 of 256 modes 40.5 / 33.4).
+// with one thread a component and a thread a butterfly: 1216 trajectories of 64 modes 33.2 / 26.3, 400 of
+// 128 modes 36.9 / 28.9, 64 of 256 modes 40.5 / 31.6).
 //
-// n butterflies over the block: f(i, c) computes component c of butterfly i, put(i, c, o) stores it.
-template <bool SPLIT, typename F, typename P>
-__device__ __forceinline__ void dns_each(int n, F f, P put) {
+// n butterflies over the block: f(i, c, o) computes component c of the two outputs of butterfly i, which
+// go to at(i, 0) and at(i, 1); extra(i, c, o) sees them before.
+template <bool SPLIT, typename F, typename A, typename E>
+__device__ __forceinline__ void dns_each(int n, F f, A at, E extra) {
     for (int t = threadIdx.x; t < (SPLIT ? 2 * n : n); t += blockDim.x) {
         if constexpr (SPLIT) {
             double o[2];
             f(t >> 1, t & 1, o);
-            put(t >> 1, t & 1, o);
+            extra(t >> 1, t & 1, o);
+            reinterpret_cast<double*>(at(t >> 1, 0))[t & 1] = o[0];
+            reinterpret_cast<double*>(at(t >> 1, 1))[t & 1] = o[1];
         } else {
             double o[2], q[2];
             f(t, 0, o);
             f(t, 1, q);
-            put(t, 0, o);
-            put(t, 1, q);
+            extra(t, 0, o);
+            extra(t, 1, q);
+            *at(t, 0) = mk<double>(o[0], q[0]);
+            *at(t, 1) = mk<double>(o[1], q[1]);
         }
     }
 }
@@ -193,12 +198,11 @@ __device__ __forceinline__ cpx<double>* dns_passes(cpx<double>* a, cpx<double>* 
                     o[1] = v0 - v1;
                 }
             },
-            [&](int i, int c, const double (&o)[2]) {
-                const int f = i >> (lg - 1), j = i & (nb - 1), jm = j & (span - 1), od = ((j - jm) << 1) + jm;
-                double* d = reinterpret_cast<double*>(b + (f << lg)) + c;
-                d[2 * od] = o[0];
-                d[2 * (od + span)] = o[1];
-            });
+            [&](int i, int q) {
+                const int f = i >> (lg - 1), j = i & (nb - 1), jm = j & (span - 1);
+                return b + (f << lg) + ((j - jm) << 1) + jm + (q ? span : 0);
+            },
+            [](int, int, double (&)[2]) {});
         __syncthreads();
         cpx<double>* t = a;
         a = b;
@@ -266,12 +270,7 @@ __device__ __forceinline__ void dns_eval(const DnsArgs& a, int tr0, int ntraj, c
             o[0] = v0 + v1;
             o[1] = v0 - v1;
         },
-        [&](int i, int c, const double (&o)[2]) {
-            const int pr = i >> (lgnx - 1), j = i & (nb - 1);
-            double* d = reinterpret_cast<double*>(A + (pr << lgnx) + 2 * j) + c;
-            d[0] = o[0];
-            d[2] = o[1];
-        });
+        [&](int i, int q) { return A + 2 * i + q; }, [](int, int, double (&)[2]) {});
     __syncthreads();
     cpx<double>* Z = dns_passes<SPLIT>(A, Bf, lgnx, np, +1, tw, twsh, 2, nb);
     cpx<double>* Y = Z == A ? Bf : A;
@@ -284,13 +283,14 @@ __device__ __forceinline__ void dns_eval(const DnsArgs& a, int tr0, int ntraj, c
             dns_bfly(Z[(pr << lgnx) + j], Z[(pr << lgnx) + j + nb],
                      twid<double, true>(tw, j * (NMAX / nx), +1, twsh), c, o[0], o[1]);
         },
-        [&](int i, int c, const double (&o)[2]) {
+        [&](int i, int q) { return Y + ((i >> (lgnx - 1)) << lgnx) + (i & (nb - 1)) + (q ? nb : 0); },
+        [&](int i, int c, double (&o)[2]) {
             const int pr = i >> (lgnx - 1), j = i & (nb - 1), t = 2 * pr + c;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const int m = j + q * nb;
                 const double u = o[q] * inx;
-                reinterpret_cast<double*>(Y + (pr << lgnx) + m)[c] = u * u;
+                o[q] = u * u;
                 if (save && a.u_saved && t < ntraj) a.u_saved[((size_t)(tr0 + t) * a.nsave + isave) * nx + m] = u;
                 if (end && a.u_end && t < ntraj) a.u_end[(size_t)(tr0 + t) * nx + m] = u;
             }
