@@ -15,9 +15,10 @@
 // puts 9/8 S just below 2^63: no pass can overflow and no pass needs a scaling of its own.  The
 // quantum, of the input and of the rounding of each twiddle product, is at most 9/4 2^-63 S,
 // against rounding relative to each intermediate value in 53-bit arithmetic.  Measured over
-// flat, decaying and single-mode random inputs against long double, the 2-norm error over that of
-// the double radix-4 transform lies between 0.38 and 0.99 (0.42 for flat inputs of 64 to 256
-// points, where the rounding of the results to double is all of it, 0.6 at 1024).
+// flat, decaying and single-mode random inputs of several amplitudes (9/8 S lies anywhere between
+// two powers of two) against long double, the 2-norm error over that of the double radix-4
+// transform lies between 0.27 and 0.83: flat inputs of 64 to 256 points 0.30 to 0.48 (the rounding
+// of the results to double is most of it), of 512 0.49 to 0.83, of 1024 0.41 to 0.75.
 //
 // A transform that holds an infinity or a NaN returns NaN in every element (each output depends on
 // each input); inputs below 2^-913 count as zero.
@@ -138,7 +139,7 @@ KS_HD int fx_top(long long v) { return (int)((unsigned long long)v >> 32); }
 // middle products enter by their high words, an error of 1.2 units rms; twelve products and 32-bit
 // sums, 58 clocks a warp (124 with the middle products in one 64-bit sum).  FINE = true: their sums
 // are rounded to the unit, at 1024 points, where the coarse products would take the error of flat
-// inputs above that of the double transform (0.9 to 1.6 times; 0.5 to 0.6 so).
+// inputs above that of the double transform (up to 1.6 times; 0.41 to 0.75 so).
 template <bool FINE>
 KS_HD fxc fx_mul(fxc v, fxw w) {
     const int al = (int)v.x, ah = fx_top(v.x) + (int)((unsigned)al >> 31);
@@ -146,11 +147,12 @@ KS_HD fxc fx_mul(fxc v, fxw w) {
     if constexpr (FINE) {
         const long long r1 = fx_wide(al, w.rh) - fx_wide(bl, w.ih), r2 = fx_wide(ah, w.rl) - fx_wide(bh, w.il);
         const long long i1 = fx_wide(al, w.ih) + fx_wide(bl, w.rh), i2 = fx_wide(ah, w.il) + fx_wide(bh, w.rl);
-        const unsigned fr = ((unsigned)r1 >> 1) + ((unsigned)r2 >> 1) + (1u << 29);
-        const unsigned fi = ((unsigned)i1 >> 1) + ((unsigned)i2 >> 1) + (1u << 29);
-        const long long x = fx_wide(ah, w.rh) - fx_wide(bh, w.ih) + fx_top(r1) + fx_top(r2) + (fr >> 31);
-        const long long y = fx_wide(ah, w.ih) + fx_wide(bh, w.rh) + fx_top(i1) + fx_top(i2) + (fi >> 31);
-        return fxc{-(x + x + ((fr >> 30) & 1)), -(y + y + ((fi >> 30) & 1))};
+        // the low words of the sums as 30 bits each, so that they and the half fit 32; bit 29 is the unit
+        const unsigned fr = ((unsigned)r1 >> 2) + ((unsigned)r2 >> 2) + (1u << 28);
+        const unsigned fi = ((unsigned)i1 >> 2) + ((unsigned)i2 >> 2) + (1u << 28);
+        const long long x = fx_wide(ah, w.rh) - fx_wide(bh, w.ih) + fx_top(r1) + fx_top(r2);
+        const long long y = fx_wide(ah, w.ih) + fx_wide(bh, w.rh) + fx_top(i1) + fx_top(i2);
+        return fxc{-(x + x + (fr >> 29)), -(y + y + (fi >> 29))};
     }
     const int r1 = fx_top(fx_wide(al, w.rh)) - fx_top(fx_wide(bl, w.ih));
     const int r2 = fx_top(fx_wide(ah, w.rl)) - fx_top(fx_wide(bh, w.il));
