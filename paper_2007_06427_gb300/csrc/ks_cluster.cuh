@@ -148,12 +148,12 @@ __host__ __device__ inline int cluster_rows_per_rank(int ns, int C) {
 
 // FFT of `cnt` columns stored [q][n] at `a` with `b` as scratch; the result is left in `a`.
 // nthr > 0: a double transform run by the first nthr threads only (see fft_fx), which alone
-// call this; otherwise every thread of the block calls it.
+// call this; otherwise every thread of the block calls it.  A double forward transform comes out
+// divided by its length, as in the items.
 template <typename R>
 __device__ __forceinline__ void col_fft_inplace(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir,
                                                 const cpx<R>* tw, int* sc, int nthr = 0) {
-    cpx<R>* r = nthr > 0 ? fft_warp<R, true>(a, b, lg, cnt, dir, tw, sc, nthr)
-                         : fft_warp<R, true>(a, b, lg, cnt, dir, tw, sc);
+    cpx<R>* r = fft_warp<R, true>(a, b, lg, cnt, dir, tw, sc, nthr, dir < 0 ? lg : 0);
     if (r != a) {
         const int n = cnt << lg;
         const int NT = nthr > 0 ? nthr : (int)blockDim.x;
@@ -261,8 +261,10 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
     cpx<RA>* tws_a = kSame ? reinterpret_cast<cpx<RA>*>(tws) : reinterpret_cast<cpx<RA>*>(smem + cp.off_tw_a);
     // 1/(2 Nx) of the row split; per loop it is multiplied by 1/Ns, the normalisation of the
     // forward s-transform that the column phases would otherwise apply (both powers of two, so
-    // the product is exact and scaling before the transform gives the same bits as after it); a
-    // double transform applies both itself (norm)
+    // the product is exact and scaling before the transform gives the same bits as after it).  The
+    // double transforms apply each factor in the transform it belongs to (norm), as in the items:
+    // their scale is no function of the ratio alone (fx_sum_ok), so a factor moved from one
+    // transform to another can change the last bits
     const R h0 = (R)d.hx;
     const RA h0_a = (RA)d.hx;
     // the per-x-mode tables, read in every phase, live in shared memory
@@ -567,7 +569,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                     }
                 }
                 __syncthreads();
-                cpx<R>* F = fft_warp<R, true>(Y, z, lgnx, np, -1, tws, fsc, 0, lgnx + 1 + lg);
+                cpx<R>* F = fft_warp<R, true>(Y, z, lgnx, np, -1, tws, fsc, 0, lgnx + 1);
                 const int lgp = lgnr - 1;
                 for (int i = wtid; i < (nkx << lgp); i += ntw) {
                     const int j = i >> lgp, pr = i & (np - 1);
@@ -732,7 +734,7 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
                                   (RA)Ul[(size_t)(t0 + 2 * pr + 1) * nx + m] * rx.y);
                 }
                 wsync();
-                cpx<RA>* F = fft_warp<RA, true>(Y, z, lgnx, np, -1, tws_a, fsc, wn, lgnx + 1 + lg);
+                cpx<RA>* F = fft_warp<RA, true>(Y, z, lgnx, np, -1, tws_a, fsc, wn, lgnx + 1);
                 for (int i = wtid; i < (nkx << lgp); i += ntw) {
                     const int j = i >> lgp, pr = i & (np - 1);
                     if (xi && j == 0) continue;
