@@ -617,13 +617,15 @@ struct LaunchScope {
     }
 };
 
-// Launch of a phase kernel.  linked: the launch in front of it in stream s is a phase kernel too; it may
-// then start while that one ends (programmatic dependent launch): its blocks stage their tables and
-// wait (grid_wait, in every phase kernel) until the launch in front has completed, which had waited
-// for its own.  A 32x32 residual, five launches: 36.9 -> 29.3 us a call; 40 double steps of 256 ragged
-// loops: 5921 -> 5837.  The float phases link launches of at most a block per SM: larger ones place
-// their early blocks on the SMs that happen to be free first, and stay uneven (120 float steps of the
-// ragged loops, some 450 blocks a launch: 6106 -> 6572 us).
+// Launch of a phase kernel.  linked (the boundary calls: load, residual, gradient): the launch in front of
+// it in stream s is a phase kernel too; it may then start while that one ends (programmatic dependent
+// launch): its blocks stage their tables and wait (grid_wait, in every phase kernel) until the launch in
+// front has completed, which had waited for its own.  A 32x32 residual, five launches: 36.9 -> 29.3 us a
+// call.  Its early blocks are placed on the SMs that happen to be free first, and stay uneven: float
+// launches of more than a block per SM are not linked, and neither are the steps, which gained 1 to 4 %
+// on single small loops and on 256 ragged ones and lost up to half elsewhere (linked / not, us a step,
+// four-launch form: double 128x1024 89.5 / 60.0, 18 of 128x256 102 / 62, two of 64x512 in the
+// subspace 80 / 51; float 64 of 64x128 33.3 / 26.7, two of 256x512 in the subspace 48.5 / 32.5).
 template <typename R, typename... KA, typename... A>
 cudaError_t launch_linked(const ks_loop* h, void (*k)(KA...), int grid, int block, size_t smem, cudaStream_t s,
                           const A&... a) {
@@ -1143,15 +1145,12 @@ int run_prime(ks_loop* h, Work& w, int pr, cudaStream_t s) {
     return KS_OK;
 }
 
-// one tau-step of every live loop of precision pr (M must hold s-inverse of u_hat); chained: the launch
-// in front of it in s is the end of the step before
+// one tau-step of every live loop of precision pr (M must hold s-inverse of u_hat); its launches are not
+// linked (see launch_linked)
 template <typename R>
-int run_step(ks_loop* h, Work& w, int pr, double tol, double switch_tol, cudaStream_t s, bool chained) {
+int run_step(ks_loop* h, Work& w, int pr, double tol, double switch_tol, cudaStream_t s) {
     Bufs<R> p = make_bufs<R>(h, w, pr, 1, tol, switch_tol, (R*)nullptr);
-    const Linked linked(h);
-    h->linked = chained;
     KS_TRY((launch_rows<R, ROW_NONLIN>(h, p, s)));
-    h->linked = true;
     KS_TRY((launch_cols<R, COL_RESID>(h, p, s)));
     KS_TRY((launch_rows<R, ROW_ADJ>(h, p, s)));
     KS_TRY((launch_cols<R, COL_UPDATE>(h, p, s)));
@@ -1707,8 +1706,8 @@ int step_graph(ks_loop* h, Work& w, const bool* live, double tol, double swt, in
             }
             s64 = h->gcap2;
         }
-        if (live[P32]) rc = run_step<float>(h, w, P32, tol, swt, h->gcap, i > 0 && !both);
-        if (rc == KS_OK && live[P64]) rc = run_step<double>(h, w, P64, tol, 0.0, s64, i > 0 && !both);
+        if (live[P32]) rc = run_step<float>(h, w, P32, tol, swt, h->gcap);
+        if (rc == KS_OK && live[P64]) rc = run_step<double>(h, w, P64, tol, 0.0, s64);
         if (rc == KS_OK && both &&
             (cudaEventRecord(h->gjoin, h->gcap2) != cudaSuccess ||
              cudaStreamWaitEvent(h->gcap, h->gjoin, 0) != cudaSuccess))
@@ -1765,8 +1764,8 @@ int phase_steps(ks_loop* h, Work& w, const bool* live, long long n, double tol, 
         }
     }
     for (; i < n; ++i) {
-        if (live[P32]) KS_TRY(run_step<float>(h, w, P32, tol, swt, s, false));
-        if (live[P64]) KS_TRY(run_step<double>(h, w, P64, tol, 0.0, s, false));
+        if (live[P32]) KS_TRY(run_step<float>(h, w, P32, tol, swt, s));
+        if (live[P64]) KS_TRY(run_step<double>(h, w, P64, tol, 0.0, s));
         w.par ^= 1;
     }
     return KS_OK;
