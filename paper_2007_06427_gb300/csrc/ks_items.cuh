@@ -493,10 +493,12 @@ KS_HD cpx<R> norm(cpx<R> v, R g) {
 }
 
 // The batched transform of every launch form: double in 64-bit fixed point (fft_fx, sc: room for
-// cnt scales), float in the radix-4 passes of fft_batch.  HOT: the phases of a tau-step, which take
-// the double transform inlined (256 ragged loops: 191 us a step, 229 through calls); the items at
-// the boundary of a call (analysis, synthesis, gradient) run once per call and share one copy of
-// it, which the launches of a call find in the instruction caches.
+// cnt scales), float in the radix-4 passes of fft_batch.  HOT: the phases of a tau-step in large
+// batches, which take the double transform inlined (256 ragged loops: 191 us a step, 229 through
+// calls); small ones (call_rows, call_cols), the persistent kernel, whose four phases follow one
+// another on the same SMs (one 64x128 loop 42.5 us a step inlined, 33.8 through calls), and the items
+// at the boundary of a call (analysis, synthesis, gradient) share one copy of it, which the launches
+// of a call find in the instruction caches.
 template <typename R, bool HOT, bool SWZ = false, bool SKI = false, bool SKO = false>
 KS_HD cpx<R>* fft_any(cpx<R>* a, cpx<R>* b, int lg, int cnt, int dir, const cpx<R>* tw, int* sc,
                       int nthr = 0, int twsh = 0, int down = 0) {
@@ -1129,7 +1131,8 @@ KS_HD void store_pair_spectra(const Dims& d, const cpx<R>* Y, cpx<R>* Mb, int ns
 // SWZ: p.tw is the bank-swizzled shared-memory copy of the twiddle table (load_twiddles).
 // par: step parity of the T arrays (the persistent kernel passes its step's; the per-phase
 // launches take p.par).
-template <typename R, int MODE, bool SWZ = false>
+// CALL: the double transforms of a tau-step through the shared copy (fft_any).
+template <typename R, int MODE, bool SWZ = false, bool CALL = false>
 KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* smem, int par = -1) {
     const RowItem it = p.rows[item];
     const int b = it.b;
@@ -1146,7 +1149,7 @@ KS_HD void row_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
     cpx<R>* Mb = p.M + p.moff[b];
     R* Ub = p.U + p.goff[b];
     int* sc = reinterpret_cast<int*>(Bf + (size_t)npairs * nx);  // scales of double transforms
-    constexpr bool kHot = MODE == ROW_NONLIN || MODE == ROW_ADJ;
+    constexpr bool kHot = !CALL && (MODE == ROW_NONLIN || MODE == ROW_ADJ);
     R* Ib = p.io ? p.io + p.goff[b] : nullptr;
 
     if constexpr (MODE == ROW_ANALYZE) {
@@ -1404,7 +1407,7 @@ KS_HD P zero_part() { return P{}; }
 // One pair of columns (ja, jb) of one loop; the modes of col_item that run on pairs.  Pair 0
 // also writes the zero column j = 0 (M and the partials) and takes the per-loop duties that
 // column 0 has in col_item (T, status, sqrt(J), the step counter).
-template <typename R, int MODE, bool SWZ = false>
+template <typename R, int MODE, bool SWZ = false, bool CALL = false>
 KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* smem, int par) {
     typedef typename PartT<R>::type Part;
     const int nkx = d.nkx, np = xi_npairs(d);
@@ -1418,7 +1421,7 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
     cpx<R>* Bf = A + ns;
     double* red = reinterpret_cast<double*>(Bf + ns);
     int* sc = reinterpret_cast<int*>(red + COL_RED_SC);
-    constexpr bool kHot = MODE == COL_RESID || MODE == COL_UPDATE;
+    constexpr bool kHot = !CALL && (MODE == COL_RESID || MODE == COL_UPDATE);
     cpx<R>* const M0 = p.M + p.moff[b];
     cpx<R>* const cola = M0 + (size_t)ja * ns;
     cpx<R>* const colb = M0 + (size_t)jb * ns;   // used only when hasb
@@ -1598,11 +1601,11 @@ KS_HD void col_pair_item(const Dims& d, const Bufs<R>& p, int item, unsigned cha
     }
 }
 
-template <typename R, int MODE, bool SWZ = false>
+template <typename R, int MODE, bool SWZ = false, bool CALL = false>
 KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* smem, int par) {
     if constexpr (col_paired(MODE)) {
         if (p.xi) {
-            col_pair_item<R, MODE, SWZ>(d, p, item, smem, par);
+            col_pair_item<R, MODE, SWZ, CALL>(d, p, item, smem, par);
             return;
         }
     }
@@ -1615,7 +1618,7 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
     cpx<R>* Bf = A + ns;
     double* red = reinterpret_cast<double*>(Bf + ns);
     int* sc = reinterpret_cast<int*>(red + COL_RED_SC);
-    constexpr bool kHot = MODE == COL_RESID || MODE == COL_UPDATE;
+    constexpr bool kHot = !CALL && (MODE == COL_RESID || MODE == COL_UPDATE);
     cpx<R>* col = p.M + p.moff[b] + (size_t)j * ns;
     const size_t bo = (size_t)p.boff[b] + (size_t)j * nk;
     const int B = d.B;

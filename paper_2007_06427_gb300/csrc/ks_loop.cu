@@ -44,7 +44,8 @@ __device__ __forceinline__ Bufs<R> stage_twiddles(const Bufs<R>& p, unsigned cha
     return q;
 }
 
-template <typename R, int MODE>
+// CALL: double transforms through the shared copy (call_copy).
+template <typename R, int MODE, bool CALL = false>
 __global__ void __launch_bounds__(256) k_rows(Dims d, Bufs<R> p, int nitems, int tw_off, int nm) {
     extern __shared__ __align__(16) unsigned char smem[];
     grid_trigger();
@@ -70,16 +71,16 @@ __global__ void __launch_bounds__(256) k_rows(Dims d, Bufs<R> p, int nitems, int
                 loop_costs(p.Jpart + (size_t)b * d.nkx, p.L2part + (size_t)b * d.nkx, d.nkx, d.L, p.T[b],
                            p.Jout ? p.Jout + b : nullptr, p.dJdTout ? p.dJdTout + b : nullptr, nullptr);
     }
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x) row_item<R, MODE, true>(d, q, it, smem);
+    for (int it = blockIdx.x; it < nitems; it += gridDim.x) row_item<R, MODE, true, CALL>(d, q, it, smem);
     if constexpr (MODE == ROW_ADJ) loops_scalars(d, q, q.par, blockIdx.x, gridDim.x);
 }
 
-template <typename R, int MODE>
+template <typename R, int MODE, bool CALL = false>
 __global__ void __launch_bounds__(256) k_cols(Dims d, Bufs<R> p, int nitems, int tw_off, int nm) {
     extern __shared__ __align__(16) unsigned char smem[];
     grid_trigger();
     const Bufs<R> q = stage_twiddles(p, smem, tw_off, nm);
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x) col_item<R, MODE, true>(d, q, it, smem, q.par);
+    for (int it = blockIdx.x; it < nitems; it += gridDim.x) col_item<R, MODE, true, CALL>(d, q, it, smem, q.par);
 }
 
 // The double column phases of a step by groups of columns (col_group).
@@ -187,7 +188,7 @@ __device__ __forceinline__ bool grid_sync(const GridBar& g) {
 // to shared memory at tw_off once per launch; the items then read them there instead of from
 // the global table (the same values, so the same bits as the per-phase launches).
 // Launch bounds: always COL_ACC_LANES = 128 threads; six resident blocks per SM caps the
-// registers at 85 (80 used, no spills; with (256) alone ptxas chose 64 and spilled).
+// registers at 85 (80 used, 8 bytes spilled around the calls of the double transforms).
 template <typename R>
 __global__ void __launch_bounds__(128, 6) k_persist(Dims d, Bufs<R> p, int nsteps, int par0,
                                                  int nrow, int ncol, GridBar bar, int tw_off,
@@ -205,14 +206,14 @@ __global__ void __launch_bounds__(128, 6) k_persist(Dims d, Bufs<R> p, int nstep
     const int ncol_u = min(ncol, col_item_count(d, p.xi, COL_UPDATE));
     for (int s = 0; s < nsteps; ++s) {
         const int par = (par0 + s) & 1;
-        for (int it = blockIdx.x; it < nrow; it += gridDim.x) row_item<R, ROW_NONLIN, true>(d, q, it, smem);
+        for (int it = blockIdx.x; it < nrow; it += gridDim.x) row_item<R, ROW_NONLIN, true, true>(d, q, it, smem);
         if (!grid_sync(bar)) return;
-        for (int it = blockIdx.x; it < ncol_r; it += gridDim.x) col_item<R, COL_RESID, true>(d, q, it, smem, par);
+        for (int it = blockIdx.x; it < ncol_r; it += gridDim.x) col_item<R, COL_RESID, true, true>(d, q, it, smem, par);
         if (!grid_sync(bar)) return;
-        for (int it = blockIdx.x; it < nrow; it += gridDim.x) row_item<R, ROW_ADJ, true>(d, q, it, smem, par);
+        for (int it = blockIdx.x; it < nrow; it += gridDim.x) row_item<R, ROW_ADJ, true, true>(d, q, it, smem, par);
         loops_scalars(d, q, par, blockIdx.x, gridDim.x);
         if (!grid_sync(bar)) return;
-        for (int it = blockIdx.x; it < ncol_u; it += gridDim.x) col_item<R, COL_UPDATE, true>(d, q, it, smem, par);
+        for (int it = blockIdx.x; it < ncol_u; it += gridDim.x) col_item<R, COL_UPDATE, true, true>(d, q, it, smem, par);
         if (s + 1 < nsteps && !grid_sync(bar)) return;
     }
 }
@@ -751,6 +752,22 @@ int launch_cols_g(ks_loop* h, const Bufs<double>& p, cudaStream_t s) {
     return KS_OK;
 }
 
+// Which double phases of a step take their transforms through the shared copy (CALL) and which inlined.
+// A launch of few or short transforms is bound by the fetch of its code: the shared copy is one loop
+// nest for both transforms of the phase, and gives two threads to a butterfly.  A launch of many takes
+// them inlined: a call's registers cost resident blocks.  Time with the copy over inlined, four-launch
+// form: rows of up to 64 points 0.87 to 0.97 up to 600 items and 1.08 at 1200, of 128 points 0.94 to
+// 1.01 and 1.11, of 256 points (256 threads) 0.96 up to 288 items, 1.04 at 320, 1.13 at 512; columns of
+// up to 64 points 0.87 to 0.92, of 128 points 0.94 to 1.00, of 256 points 0.96 where they fill no wave
+// of blocks and 1.01 beyond, of 512 points 0.99 to 1.05; in the subspace, whose items are pairs of
+// columns, of up to 64 points 0.92 to 0.99, 1.03 from 2800 items on, of 128 points 1.01 to 1.07.
+bool call_rows(const ks_loop* h, int n) { return n <= (h->d.nx >= 256 ? 2 : 4) * 152; }
+bool call_cols(const ks_loop* h, int n) {
+    if (n > 16 * 152) return false;
+    if (h->xi) return h->nsmax <= 64;
+    return h->nsmax <= 128 || (h->nsmax <= 256 && n <= 152);
+}
+
 template <typename R, int MODE>
 int launch_rows(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const int pr = std::is_same<R, double>::value ? P64 : P32;
@@ -759,7 +776,10 @@ int launch_rows(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const Launch& l = h->lrow[pr];
     const int n = (int)h->rows.size();
     LaunchScope ls(h, s, kRowNames[MODE], prec_suffix(pr));
-    KS_CUDA(launch_linked<R>(h, k_rows<R, MODE>, std::min(n, l.grid), l.threads, l.smem, s, h->d, p, n, (int)l.tw_off,
+    auto* k = k_rows<R, MODE>;
+    if constexpr (std::is_same<R, double>::value && (MODE == ROW_NONLIN || MODE == ROW_ADJ))
+        if (call_rows(h, n)) k = k_rows<R, MODE, true>;
+    KS_CUDA(launch_linked<R>(h, k, std::min(n, l.grid), l.threads, l.smem, s, h->d, p, n, (int)l.tw_off,
                           h->d.nx));
     ls.done();
     return KS_OK;
@@ -775,7 +795,10 @@ int launch_cols(ks_loop* h, const Bufs<R>& p, cudaStream_t s) {
     const Launch& l = h->lcol[pr];
     const int n = col_item_count(h->d, h->xi, MODE);
     LaunchScope ls(h, s, kColNames[MODE], prec_suffix(pr));
-    KS_CUDA(launch_linked<R>(h, k_cols<R, MODE>, std::min(n, l.grid), l.threads, l.smem, s, h->d, p, n, (int)l.tw_off,
+    auto* k = k_cols<R, MODE>;
+    if constexpr (std::is_same<R, double>::value && (MODE == COL_RESID || MODE == COL_UPDATE))
+        if (call_cols(h, n)) k = k_cols<R, MODE, true>;
+    KS_CUDA(launch_linked<R>(h, k, std::min(n, l.grid), l.threads, l.smem, s, h->d, p, n, (int)l.tw_off,
                           h->nsmax));
     ls.done();
     return KS_OK;
@@ -802,6 +825,12 @@ int set_smem_attrs(ks_loop* h) {
     KS_ATTR((k_cols<R, COL_RESID_R>), cs);
     KS_ATTR((k_cols<R, COL_RESID_J>), cs);
     KS_ATTR((k_cols<R, COL_GRAD_G>), cs);
+    if constexpr (std::is_same<R, double>::value) {
+        KS_ATTR((k_rows<R, ROW_NONLIN, true>), rs);
+        KS_ATTR((k_rows<R, ROW_ADJ, true>), rs);
+        KS_ATTR((k_cols<R, COL_RESID, true>), cs);
+        KS_ATTR((k_cols<R, COL_UPDATE, true>), cs);
+    }
 #undef KS_ATTR
     return KS_OK;
 }
