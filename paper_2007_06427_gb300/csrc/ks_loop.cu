@@ -652,7 +652,7 @@ struct Linked {
 
 const char* prec_suffix(int pr) { return pr == 0 ? "_f64" : "_f32"; }
 
-// The float phases of a step take the register kernels wherever their lengths are covered, except
+// The float phases of a step take the register kernels wherever setup_rg has made their tiles, except
 // in the centre-symmetric subspace (whose transforms pair rows and columns differently).  The two
 // row phases agree on the layout of U, so they must come from the same family: the choice depends
 // on nothing that changes between them.
@@ -683,7 +683,13 @@ int launch_rg_cols(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
     return KS_OK;
 }
 
-// Tiles and twiddles of the register kernels: row lengths 32 .. 512, column lengths 32 .. 1024.
+// Tiles and twiddles of the register kernels: row lengths 32 .. 512, column lengths 32 .. 1024, in
+// batches that give their row phases a block or so for every second SM.  A warp's chain over sixteen
+// points a thread is long, and below that line the items' many short ones end sooner (us a step in four
+// launches, register kernels / items, at their blocks of rows: one 256x256 loop, 16, 29.1 / 22.0; one
+// 128x512, 16, 27.9 / 23.9; 18 of 64x256, 72, 27.4 / 24.5; 40 of 32x64, 20, 23.2 / 19.7; beyond it 18 of
+// 64x512, 144, 27.6 / 32.1; 18 of 256x128, 144, 28.3 / 34.4; 64 of 64x128, 128, 26.7 / 29.6; with columns
+// of up to 64 points 300 of 32x32, 75, 29.1 / 33.6; 40 of 128x64, 80, 21.9 / 30.6).
 int setup_rg(ks_loop* h) {
     const int nx = h->d.nx;
     if (nx < 32 || nx > 512) return KS_OK;
@@ -693,6 +699,7 @@ int setup_rg(ks_loop* h) {
     const int step = 1024 / nx;  // 2 F rows, F = 32 / (nx / 16) pairs a warp
     for (int b = 0; b < h->d.B; ++b)
         for (int n0 = 0; n0 < h->ns[b]; n0 += step) rows.push_back(RgTile{b, n0});
+    if ((int)rows.size() <= (h->nsmax <= 64 ? 63 : 95) * (RG_THREADS / 32)) return KS_OK;
     std::vector<RgCol> cols;  // in colorder: the 1024-point loops come first
     for (int b : h->colorder) {
         const int F = std::max(1, 512 / h->ns[b]);
