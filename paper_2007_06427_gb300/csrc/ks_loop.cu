@@ -1047,22 +1047,26 @@ int default_path(const ks_loop* h, int pr) {
     return (P >= 32768 || (P >= 16384 && B >= 64)) ? 2 : 0;
 }
 
-// The form of a handle whose "path" knob is not set, from step times on GB300 over loops of 32x32 to
-// 256x512 points, batches of 1 to 2048, in and outside the subspace.  All forms compute the same bits.
+// The form of a handle whose "path" knob is not set, from step times on GB300 over loops of 16x16 to
+// 1024x256 and 32x1024 points, batches of 1 to 1000, in and outside the subspace.  All forms compute the same bits.
 //   * Ragged batches of 64 or more loops: four launches.  One cluster a loop leaves the SMs of the long
 //     loops working while the rest idle.
 //   * Otherwise by the points of a CTA's share of a loop, Q = P / C, and by whether all clusters of the
 //     batch are resident.  The cluster kernel's step grows with Q, its transforms shared by four warps,
-//     and with the waves; four launches have a floor (double 40 us, float 18 to 28) and fill the GPU.
-//     Double: four launches from Q = 2048 on (us a step, cluster against four launches: Q = 1024: one
-//     64x256 loop 29.3 / 43.0, 32 64x128 loops 35.8 / 47.7; Q = 2048: one 128x256 loop 51.2 / 44.6, 256
-//     32x64 loops 71.3 / 62.8), and from 512 on where the clusters take several waves (16 64x256 loops
-//     65.6 / 48.6, 1024 16x32 loops 92.3 / 61.9, but 1024 16x16 loops 68.4 / 94.1).
-//     Float, with its phases in registers (use_rg): from Q = 4096 on (256 64x64 loops 60.3 / 26.3, one
-//     256x256 loop 39.0 / 28.9), from Q = 2048 on in clusters of fewer than 16 CTAs or in waves (256
-//     64x32 loops 38.3 / 25.8, 64 256x32 loops 38.9 / 24.5, 16 128x256 loops 47.3 / 29.7, but one 128x256
-//     loop 20.5 / 27.1) and from 1024 on in waves (512 32x32 loops 46.9 / 30.9).  Float with the items
-//     (the subspace): from Q = 4096 on (256 64x128 loops 129 / 58), and from Q = 2048 on in waves.
+//     and with the waves; four launches have a floor (double 33 us, float 17 to 25) and fill the GPU.
+//     Double: four launches from Q = 2048 on (us a step, cluster / four launches: Q = 1024: one 64x256
+//     loop 28.7 / 36.1, 40 64x64 loops 34.4 / 37.2; Q = 2048: one 128x256 loop 50.2 / 40.8, 300 32x64
+//     loops 68.7 / 64.0), and from 512 on where the clusters take several waves (18 64x256 loops
+//     64.9 / 48.9, 1000 32x32 loops 141 / 83).
+//     Float outside the subspace: from Q = 4096 on (one 256x256 loop 38.4 / 22.0); from Q = 2048 on in
+//     batches of 8 or more of one length (300 64x32 loops 36.5 / 25.4, 8 256x128 loops 28.0 / 25.7, but
+//     4 of them 21.2 / 22.0, 32 ragged 64x{32 .. 256} loops 23.5 / 24.4), with transforms of 512 points or
+//     more (one 32x1024 loop 39.2 / 25.8, one 64x512 25.5 / 22.1) or in waves; with the register kernels
+//     from 1024 on in waves (512 32x32 loops 46.9 / 30.9).
+//     Float in the subspace: from Q = 4096 on (64 64x256 loops 40.3 / 33.9), with columns of less than 64
+//     points, whose many small items cost most, from 8192 on (300 128x32 loops 58.0 / 68.3), and from 2048
+//     on with transforms of 1024 points (one 32x1024 loop 40.3 / 28.4, but one 64x512 23.6 / 23.6, one
+//     128x256 18.6 / 22.3) or in waves.
 int auto_form(const ks_loop* h, int pr) {
     const int B = h->d.B;
     const ClusterPlan& cp = h->cplan[pr];
@@ -1073,8 +1077,10 @@ int auto_form(const ks_loop* h, int pr) {
     const long long Q = (long long)h->d.nx * h->nsmax / cp.C;
     const bool waves = h->cgrid[pr] < cp.C * B;
     if (pr == P64) return Q >= (waves ? 512 : 2048) ? 2 : 0;
-    if (use_rg(h)) return Q >= (waves ? 1024 : cp.C < 16 ? 2048 : 4096) ? 2 : 0;
-    return Q >= (waves ? 2048 : 4096) ? 2 : 0;
+    const int m = std::max(h->d.nx, h->nsmax);
+    if (h->xi) return Q >= (waves || m >= 1024 ? 2048 : h->nsmax < 64 ? 8192 : 4096) ? 2 : 0;
+    if (waves) return Q >= (use_rg(h) ? 1024 : 2048) ? 2 : 0;
+    return Q >= (m >= 512 || (B >= 8 && !ragged && h->nsmax >= 32) ? 2048 : 4096) ? 2 : 0;
 }
 
 // the launch form precision pr's steps take: 0 cluster-resident (where its plan fits), 1
