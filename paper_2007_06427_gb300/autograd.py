@@ -48,21 +48,28 @@ class KSLoopJ(torch.autograd.Function):
 
 def loop_index(loop, device):
     """Loop of each packed grid value (a gather by it needs no host read of the lengths)."""
-    key = ("index", str(device))
-    cache = loop.__dict__.setdefault("_cache", {})
-    if key not in cache:
+    def make():
         sizes = torch.tensor([n * loop.nx for n in loop.ns], dtype=torch.int64, device=device)
-        cache[key] = torch.repeat_interleave(torch.arange(loop.batch, device=device), sizes)
-    return cache[key]
+        return torch.repeat_interleave(torch.arange(loop.batch, device=device), sizes)
+    return _constant(loop, "index", device, make)
 
 
 def loop_factor(loop, device):
     """2 L / (Nx Ns_b) per loop."""
-    key = ("factor", str(device))
+    return _constant(loop, "factor", device, lambda: torch.tensor(
+        [2.0 * loop.L / (loop.nx * n) for n in loop.ns], dtype=torch.float64, device=device))
+
+
+def _constant(loop, name, device, make):
+    """A tensor kept with the handle.  It is complete before any other call can see it: the stream
+    of the first backward made it, and a later one may run on another that is not ordered behind."""
     cache = loop.__dict__.setdefault("_cache", {})
+    key = (name, str(device))
     if key not in cache:
-        cache[key] = torch.tensor([2.0 * loop.L / (loop.nx * n) for n in loop.ns], dtype=torch.float64,
-                                  device=device)
+        value = make()
+        if value.is_cuda:
+            torch.cuda.current_stream(value.device).synchronize()
+        cache[key] = value
     return cache[key]
 
 
