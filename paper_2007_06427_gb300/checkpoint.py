@@ -74,8 +74,14 @@ def resume(path: str, info: bool = False, **create_kw):
             loop.close()
             raise ValueError(f"checkpoint {path} does not match its own configuration")
         for k in KNOBS:
-            if f"knob_{k}" in z.files:
-                K.ks_set_option(loop.handle, k, int(z[f"knob_{k}"]))
+            if f"knob_{k}" not in z.files:
+                continue
+            # a file from before "path_auto" holds a handle's own value of an unset path: setting it
+            # would fix that form in place of the rule
+            if (k in ("path_f64", "path_f32") and "knob_path_auto" not in z.files
+                    and int(z[f"knob_{k}"]) == K.ks_get_option(loop.handle, k)):
+                continue
+            K.ks_set_option(loop.handle, k, int(z[f"knob_{k}"]))
         K.ks_set_band(loop.handle, band, np.ascontiguousarray(z["T"], dtype=np.float64),
                       np.ascontiguousarray(z["prec"], dtype=np.int32),
                       np.ascontiguousarray(z["steps"], dtype=np.int64))
