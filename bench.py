@@ -415,7 +415,7 @@ def annotate_sms(roof, K, h, mode, batch, dev):
     """For the cluster-resident kernel: the SMs a launch occupies (one CTA per SM; C CTAs per
     loop) and the roofline fraction against the peak of those SMs alone."""
     import torch
-    if not roof or K.ks_get_option(h.handle, "path") != 0 or not roof.get("kernel", "cluster").startswith("cluster"):
+    if not roof or not roof.get("kernel", "").startswith("cluster"):  # the kernel the profile saw, not the knob
         return roof
     C = K.ks_get_option(h.handle, "cluster_f32" if mode == K.KS_FP32 else "cluster_f64")
     if C <= 0:
