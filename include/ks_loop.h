@@ -208,8 +208,9 @@ KS_API int ks_profile_read(ks_loop_t h, int n, char* names, double* ms, long lon
  *                    more, or when the cluster plan has 1 or 2 CTAs per loop on P >= 4096; float:
  *                    2 when P >= 32768, or P >= 16384 in batches of 64 or more; else 0.  Until one
  *                    of these knobs is set, the steps take the faster of forms 0 and 2 by a rule on
- *                    the points of a loop per CTA of its cluster (see "form_f64").  ks_autotune
- *                    replaces the bulk precision's form (float for KS_MIXED) by timing.
+ *                    the points of a loop per CTA of its cluster, so a value read here is not the
+ *                    form in use (that is "form_f64") and setting it again fixes that form.
+ *                    ks_autotune replaces the bulk precision's form (float for KS_MIXED) by timing.
  *   "path_auto"      bit 0 (double) and bit 1 (float): that precision's path has not been set.
  *                    Setting a path clears its bit; setting the bit returns to the rule.
  *   "form_f64", "form_f32"  (read only) the form the steps of that precision take now, with the
@@ -218,9 +219,14 @@ KS_API int ks_profile_read(ks_loop_t h, int n, char* names, double* ms, long lon
  *   "row_threads", "col_threads"  path 2: threads per block of the row and column items, 128
  *                    or 256 (results are bit-identical: a column's partials of J and L^dag_2
  *                    keep 128 accumulators at either size).  Default at create: 256-thread rows
- *                    for Nx >= 256; 256-thread columns for max Ns >= 256 when the batch has fewer
- *                    than 152 column items (loops x retained x-modes, one per SM of a GB300), in
- *                    double also when it has fewer than 400 or max Ns = 1024; else 128.
+ *                    for Nx >= 256; 256-thread columns for max Ns = 1024, and for max Ns >= 256
+ *                    when the batch has fewer than 304 column items (loops x retained x-modes,
+ *                    two per SM of a GB300); else 128.  Two kinds of steps have kernels of their
+ *                    own outside the centre-symmetric subspace, with 128 threads whatever the
+ *                    knobs say: float steps of batches with more than 252 tiles of 1024 points
+ *                    (380 where max Ns > 64), all Ns >= 32 and Nx 32..512; and the double columns
+ *                    of batches with at least 304 groups of up to 512 points or 16 columns, all
+ *                    Ns >= 32 and some Ns < 512.
  *   "cluster"        0 (default): cluster size chosen per precision; 1..16: force this size
  *                    (KS_ERR_ARG when no plan of that size fits the batch)
  *   "cluster_exchange" 1 (default): the cluster kernel's DSMEM exchanges are asynchronous

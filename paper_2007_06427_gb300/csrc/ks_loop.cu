@@ -1481,11 +1481,14 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
     bool api_need[2] = {true, h->api_prec == P32};
     if ((rc = alloc_work(h, h->st, st_need)) || (rc = alloc_work(h, h->api, api_need)))
         return cleanup(rc);
-    // launch shapes.  Block sizes from step times of the four-launch form on GB300: 256-thread
-    // row items for rows of 256 points or more (256 x 1024, 8 loops: 505 against 546 us per
-    // double step), 256-thread column items only when the columns are fewer than the SMs and
-    // long (one 256 x 1024 loop: 102 against 113 us); batches with more column items run
-    // them faster at 128 threads (ragged 64 x {32..256}, 256 loops: 405 against 479 us).
+    // launch shapes of the items, the same in both precisions (the knobs "row_threads" and "col_threads" hold
+    // one value each), from step times of the four-launch form on GB300 with blocks of 256 over 128 threads:
+    //   * rows: of 256 points 0.97 to 0.99 (double) and 0.96 to 1.00 (float), of 512 points 0.94 to 0.98 and
+    //     0.92 to 1.01; of 64 and 128 points 1.00 to 1.27 and 0.97 to 1.03;
+    //   * columns of 256 and 512 points: double 0.94 to 0.99 up to 176 items, 1.01 to 1.03 at 344, 1.2 at
+    //     700 (64x512); float 0.94 to 0.98 up to 172, 0.98 to 1.03 at 350 to 1400, 1.14 at 2750;
+    //   * columns of 1024 points: double 0.86 to 0.98 at every count from 11 to 1408 (8 loops of 256x1024
+    //     180.8 / 160.3 us a step), float 0.82 to 0.98; pairs of columns in the subspace alike.
     const int ncolitems = B * h->d.nkx;
     for (int pr = 0; pr < 2; ++pr) {
         const size_t cs = pr == P64 ? sizeof(cpx<double>) : sizeof(cpx<float>);
@@ -1497,10 +1500,7 @@ extern "C" int ks_loop_create(const ks_config* cfg, ks_loop_t* out) {
         lr.smem = lr.tw_off + tw_bytes(h->d.nx);
         lr.grid = 152 * 16;
         Launch& lc = h->lcol[pr];
-        // 256 threads where the columns are few for the SMs or long. Double, us a step of four launches
-        // with 128 and 256 threads: 8 loops of 128x512 (344 columns) 99.5 / 73.3, 8 of 256x1024 (688)
-        // 183 / 159, 4 of 128x256 (172) 57.4 / 51.8, but 32 of 64x512 (704) 101.7 / 108.1.
-        lc.threads = h->nsmax >= 256 && (ncolitems < 152 || (pr == P64 && (ncolitems < 400 || h->nsmax >= 1024))) ? 256 : 128;
+        lc.threads = h->nsmax >= 1024 || (h->nsmax >= 256 && ncolitems < 2 * 152) ? 256 : 128;
         lc.tw_off = (2 * (size_t)h->nsmax * cs + COL_RED_DOUBLES * sizeof(double) + 15) & ~(size_t)15;
         lc.smem = lc.tw_off + tw_bytes(h->nsmax);
         lc.grid = 152 * 16;

@@ -48,3 +48,35 @@ def test_forms_agree_across_the_line(exponent, nx, nss, xi):
     for path in (0, 1):
         for x, y in zip(stepped(us, Ts, nx, nss, L, path, xi), ref):
             assert np.array_equal(x, y)
+
+
+def relative(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+@pytest.mark.parametrize("nx,nss", [(32, [32, 16]), (64, [128, 64, 8]), (256, [256]), (128, [512, 32]), (32, [1024])])
+@pytest.mark.parametrize("amps", [(1e-33,), (1e-40,), (1e33,), (1.0, 1e-33, 1e33)])
+def test_residual_and_gradient_outside_the_float_range(nx, nss, amps):
+    """Amplitudes where every scale, or that of a neighbouring loop, comes from the exponents, at lengths on
+    both sides of 128 (where the scale has a pass of its own), against the oracle: 1e-12 of each
+    loop's norm, as for ordinary loops."""
+    from oracle import ks_oracle as ko
+    L = 22.0 * max(1.0, nx / 64)
+    nss = nss * len(amps)
+    us, Ts = loops(nx, nss, L, amps, decay=(max(2.0, (nx // 3) / 10.0), 2.0))
+    u = torch.tensor(np.concatenate([a.ravel() for a in us]), device="cuda")
+    T = torch.tensor(Ts, dtype=torch.float64, device="cuda")
+    r, G = torch.empty_like(u), torch.empty_like(u)
+    J, dJ = torch.empty_like(T), torch.empty_like(T)
+    with K.KSLoop(L, nx, nss, K.KS_FP64) as h:
+        K.ks_residual(h.handle, u, T, r, J)
+        K.ks_adjoint_grad(h.handle, u, T, G, dJ)
+    at = 0
+    for b, n in enumerate(nss):
+        ref = ko.adjoint_grad(us[b], Ts[b], L)
+        r_ref = ko.grid(nx, n, L).real_grid(ref["rh"])
+        cut = slice(at, at + n * nx)
+        at += n * nx
+        assert relative(r.cpu().numpy()[cut], r_ref.ravel()) < 1e-12
+        assert relative(G.cpu().numpy()[cut], ref["G"].ravel()) < 1e-12
+        assert abs(J[b].item() - ref["J"]) <= 1e-12 * ref["J"]
