@@ -125,7 +125,7 @@ KS_HD cpx<R> symbol_add(R a, R b, cpx<R> v, cpx<R> c) {
 // (a + i b) u_hat - F.  Double: F holds the spectrum of u^2 and u u_x = (u^2)_x / 2, so its own is
 // i q / 2 F (the truncated products are exact projections of the continuous ones, so this is the same
 // quantity): no transform for u_x.  The factor q / 2 multiplies the white noise of the forward
-// transform, which in fixed point is so far below the double transform's that r and G come out 5 to 20
+// transform, which in fixed point is so far below the double transform's that r and G come out 3 to 19
 // times closer to a long double evaluation than with a double transform of u u_x; in float the
 // noise at the band's edge would grow by the factor.
 template <typename R>
