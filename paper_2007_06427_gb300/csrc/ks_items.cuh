@@ -316,7 +316,7 @@ struct Bufs {
     int prec_new;           // precision), or null
     const float* iof;       // ROW_ANALYZE, double: float grid to analyse in place of io, or null
     cpx<float>* uhf;        // COL_ANALYZE: band rounded to float, stored in place of uh, or null
-    int fin;                // ROW_SYNTH: 1: also form J, dJ/dT and sqrt(J) from the column partials
+    int fin;                // ROW_SYNTH: 1: also form J and dJ/dT from the column partials
     double* Jout;           // [B] (fin), each nullable
     double* dJdTout;
     int step_scalars;       // 1 (tau-steps): the ROW_ADJ launch forms each running loop's step
@@ -1735,23 +1735,13 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                     const cpx<R> r = p.rh[bo + (k + ks)];
                     const R bk = (R)k * w_over_T;             // +omega_k / T
                     const cpx<R> G = symbol_add(a_lin, bk, r, wh);
-                    if (p.xi) X[i] = G;
-                    else if constexpr (MODE == COL_GRAD) p.gh[bo + (k + ks)] = G;
+                    if constexpr (MODE == COL_GRAD) p.gh[bo + (k + ks)] = G;  // the host build of the items
                     x = G;
                 }
                 if constexpr (MODE == COL_GRAD_G) X[i] = x;
             }
             if constexpr (MODE == COL_GRAD_G) back(X, F);
             KS_SYNC();
-            if (p.xi) {
-                // gradient within the Xi subspace: the projected G_hat
-                for (int i = KS_TID; i < ns; i += KS_NT) {
-                    const int k = (i < (ns >> 1)) ? i : i - ns;
-                    if (k >= -ks && k <= ks)
-                        p.gh[bo + (k + ks)] = (j == 0) ? mk<R>(0, 0) : xi_pair(X[i], X[(ns - i) & (ns - 1)]);
-                }
-                KS_SYNC();
-            }
         } else if constexpr (MODE == COL_UPDATE) {
             // J, the freeze decision and the next T of this step were formed once for the loop
             // by the ROW_ADJ launch (loop_scalars): a loop that froze now is in p.status
@@ -1759,36 +1749,15 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
             const R dt = (R)d.dtau;
             const R cqj = p.cq[j];
             const R wT2 = w_over_T * w_over_T;
-            if (p.xi) {
-                // Xi subspace: G_hat of every k into X first; the update below takes the
-                // projected pair (j, k), (j, -k) from there
-                for (int i = KS_TID; i < ns; i += KS_NT) {
-                    const int k = (i < (ns >> 1)) ? i : i - ns;
-                    if (k >= -ks && k <= ks) {
-                        const cpx<R> wh = norm(F[i], ins);
-                        const cpx<R> r = p.rh[bo + (k + ks)];
-                        const R bk = (R)k * w_over_T;
-                        X[i] = symbol_add(a_lin, bk, r, wh);
-                    }
-                }
-                KS_SYNC();
-            }
-            // the new u_hat goes to X, or to F (free once G_hat is formed) in the Xi subspace
-            cpx<R>* Y = p.xi ? F : X;
             for (int i = KS_TID; i < ns; i += KS_NT) {
                 const int k = (i < (ns >> 1)) ? i : i - ns;
                 cpx<R> x = mk<R>(0, 0);
                 if (k >= -ks && k <= ks) {
-                    cpx<R> G;
-                    if (p.xi) {
-                        G = (j == 0) ? mk<R>(0, 0) : xi_pair(X[i], X[(ns - i) & (ns - 1)]);
-                    } else {
-                        const cpx<R> wh = norm(F[i], ins);
-                        const cpx<R> r = p.rh[bo + (k + ks)];
-                        const R bk = (R)k * w_over_T;
-                        // G_hat = (a + i omega/T) r_hat + F[P(u r_x)]                      (a9)
-                        G = symbol_add(a_lin, bk, r, wh);
-                    }
+                    const cpx<R> wh = norm(F[i], ins);
+                    const cpx<R> r = p.rh[bo + (k + ks)];
+                    const R bk = (R)k * w_over_T;
+                    // G_hat = (a + i omega/T) r_hat + F[P(u r_x)]                          (a9)
+                    const cpx<R> G = symbol_add(a_lin, bk, r, wh);
                     R f = dt;
                     if (d.scheme == 1) {
                         // IMEX: dtau / (1 - dtau Lambda), Lambda = -(omega/T)^2 - q^4 (q^2-1)^2  (a10)
@@ -1799,11 +1768,9 @@ KS_HD void col_item(const Dims& d, const Bufs<R>& p, int item, unsigned char* sm
                     p.uh[bo + (k + ks)] = u;
                     x = u;
                 }
-                Y[i] = x;
+                X[i] = x;
             }
-            KS_SYNC();
-            cpx<R>* v = fft_any<R, kHot, SWZ>(Y, p.xi ? X : F, lg, 1, +1, p.tw, sc, 0, p.twsh);
-            for (int i = KS_TID; i < ns; i += KS_NT) col[i] = v[i];
+            back(X, F);
             KS_SYNC();
         }
     }
