@@ -14,7 +14,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "libks_loop.so")
-SOURCES = ["ks_loop.cu", "ks_noalloc.cu", "ks_probe.cu", "ks_dns.cu"]
+SOURCES = ["ks_loop.cu", "ks_cluster.cu", "ks_reg.cu", "ks_noalloc.cu", "ks_probe.cu", "ks_dns.cu"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 
@@ -26,7 +26,8 @@ def nvcc() -> str:
 
 
 def build(verbose: bool = False, extra=()) -> str:
-    cmd = [nvcc(), ARCH, "-O3", "-lineinfo", "-std=c++17", "--shared", "-Xcompiler", "-fPIC",
+    # the translation units compile side by side
+    cmd = [nvcc(), ARCH, "-t", str(len(SOURCES)), "-O3", "-lineinfo", "-std=c++17", "--shared", "-Xcompiler", "-fPIC",
            "-Xcompiler", "-fvisibility=hidden", "-I", INCLUDE, "-I", CSRC,
            "-DKS_BUILD_SO", "-o", LIB + ".tmp"]
     cmd += list(extra)

@@ -931,4 +931,11 @@ __global__ void __launch_bounds__(256, MB) k_cluster(Dims d, Bufs<R> p, AdjTable
     cp_async_wait();  // a cluster whose loops were all skipped still has its table copies
 }
 
+// the cluster kernel of a column scheme and launch-bound variant (see k_cluster); ks_cluster.cu holds
+// the kernels, for <double, double>, <float, float> and <double, float>
+template <typename R, typename RA>
+using ClusterFn = void (*)(Dims, Bufs<R>, AdjTables<RA>, ClusterPlan, int, int, int);
+template <typename R, typename RA>
+ClusterFn<R, RA> cluster_fn(bool xi, int mb);
+
 }  // namespace ks

@@ -662,12 +662,7 @@ template <int MODE>
 int launch_rg_rows(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
     const int n = h->rg_nrow, per = RG_THREADS / 32, g = (n + per - 1) / per;
     LaunchScope ls(h, s, kRowNames[MODE], prec_suffix(P32));
-    auto* const k = h->d.lgnx == 5   ? k_rg_rows<MODE, 5>
-                    : h->d.lgnx == 6 ? k_rg_rows<MODE, 6>
-                    : h->d.lgnx == 7 ? k_rg_rows<MODE, 7>
-                    : h->d.lgnx == 8 ? k_rg_rows<MODE, 8>
-                                     : k_rg_rows<MODE, 9>;
-    KS_CUDA(launch_linked<float>(h, k, g, RG_THREADS, 0, s, h->d, p, h->d_rg_rows, n, h->d_rg_tab));
+    KS_CUDA(launch_linked<float>(h, rg_rows_fn(MODE, h->d.lgnx), g, RG_THREADS, 0, s, h->d, p, h->d_rg_rows, n, h->d_rg_tab));
     ls.done();
     return KS_OK;
 }
@@ -677,7 +672,7 @@ int launch_rg_cols(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
     const int n = h->rg_ncol, per = RG_THREADS / 64, g = (n + per - 1) / per;
     LaunchScope ls(h, s, kColNames[MODE], prec_suffix(P32));
     const size_t smem = (size_t)h->rg_ntab * sizeof(rgv) + (size_t)per * RG_XBYTES;
-    KS_CUDA(launch_linked<float>(h, k_rg_cols<MODE>, g, RG_THREADS, smem, s, h->d, p, h->d_rg_cols, n, h->d_rg_tab,
+    KS_CUDA(launch_linked<float>(h, rg_cols_fn(MODE), g, RG_THREADS, smem, s, h->d, p, h->d_rg_cols, n, h->d_rg_tab,
                           h->rg_ntab));
     ls.done();
     return KS_OK;
@@ -948,15 +943,6 @@ int cluster_block(const ks_loop* h, int slot, const ClusterPlan& cp) {
     const int pb = (cp.rt / 2) * (nx / 4);     // row pairs
     const int cb = cp.ncmax * (cp.nsmax / 4);  // columns (or column pairs)
     return (pb <= 128 && cb <= 128) ? 160 : 128;
-}
-
-// the cluster kernel of a column scheme and launch-bound variant (see k_cluster)
-template <typename R, typename RA>
-using ClusterFn = void (*)(Dims, Bufs<R>, AdjTables<RA>, ClusterPlan, int, int, int);
-template <typename R, typename RA>
-ClusterFn<R, RA> cluster_fn(bool xi, int mb) {
-    if (mb == 2) return xi ? k_cluster<R, RA, true, 2> : k_cluster<R, RA, false, 2>;
-    return xi ? k_cluster<R, RA, true, 1> : k_cluster<R, RA, false, 1>;
 }
 
 // pick the cluster size: enough CTAs to cover the GPU (about two per SM), at most 16, and a

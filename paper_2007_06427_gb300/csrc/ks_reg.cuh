@@ -540,6 +540,13 @@ __global__ void __launch_bounds__(RG_THREADS, 3) k_rg_cols(Dims d, Bufs<float> p
         }
     }
 }
+
+// the kernels, held by ks_reg.cu: mode ROW_NONLIN or ROW_ADJ and rows of 2^lgnx points; mode COL_RESID or
+// COL_UPDATE
+using RgRowsFn = void (*)(Dims, Bufs<float>, const RgTile*, int, const rgv*);
+using RgColsFn = void (*)(Dims, Bufs<float>, const RgCol*, int, const rgv*, int);
+RgRowsFn rg_rows_fn(int mode, int lgnx);
+RgColsFn rg_cols_fn(int mode);
 #endif  // KS_HOST_EMULATION
 
 }  // namespace ks
