@@ -224,7 +224,7 @@ KS_API int ks_profile_read(ks_loop_t h, int n, char* names, double* ms, long lon
  *                    two per SM of a GB300); else 128.  Two kinds of steps have kernels of their
  *                    own outside the centre-symmetric subspace, with 128 threads whatever the
  *                    knobs say: float steps of batches with more than 252 tiles of 1024 points
- *                    (380 where max Ns > 64), all Ns >= 32 and Nx 32..512; and the double columns
+ *                    (380 where 64 < max Ns < 512), all Ns >= 32, Nx 32..512; and the double columns
  *                    of batches with at least 304 groups of up to 512 points or 16 columns, all
  *                    Ns >= 32 and some Ns < 512.
  *   "cluster"        0 (default): cluster size chosen per precision; 1..16: force this size

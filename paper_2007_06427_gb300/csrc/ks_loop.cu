@@ -383,6 +383,8 @@ struct ks_loop {
     // float phases with the transforms in registers (ks_reg.cuh): tiles, or none where a length is
     // not covered
     int rg_nrow = 0, rg_ncol = 0, rg_ntab = 0;
+    bool rg_steps = false;  // the steps take them too (see setup_rg)
+    bool stepping = false;  // the launches belong to a step
     RgTile* d_rg_rows = nullptr;
     RgCol* d_rg_cols = nullptr;
     rgv* d_rg_tab = nullptr;
@@ -643,20 +645,20 @@ cudaError_t launch_linked(const ks_loop* h, void (*k)(KA...), int grid, int bloc
     return cudaLaunchKernelEx(&cfg, k, KA(a)...);
 }
 
-// The launches while this lives are linked.
-struct Linked {
-    ks_loop* h;
-    explicit Linked(ks_loop* h_) : h(h_) { h->linked = true; }
-    ~Linked() { h->linked = false; }
+// A flag of the handle that is set while this lives.
+struct Flag {
+    bool& f;
+    explicit Flag(bool& f_) : f(f_) { f = true; }
+    ~Flag() { f = false; }
 };
 
 const char* prec_suffix(int pr) { return pr == 0 ? "_f64" : "_f32"; }
 
-// The float phases of a step take the register kernels wherever setup_rg has made their tiles, except
-// in the centre-symmetric subspace (whose transforms pair rows and columns differently).  The two
-// row phases agree on the layout of U, so they must come from the same family: the choice depends
-// on nothing that changes between them.
-bool use_rg(const ks_loop* h) { return h->rg_nrow > 0 && !h->xi; }
+// The float phases take the register kernels where setup_rg has made their tiles, in the steps of large
+// batches only, and except in the centre-symmetric subspace (whose transforms pair rows and columns
+// differently).  The two row phases agree on the layout of U, so they must come from the same family:
+// both are launched by a step, or both by a boundary call.
+bool use_rg(const ks_loop* h) { return h->rg_nrow > 0 && !h->xi && (h->rg_steps || !h->stepping); }
 
 template <int MODE>
 int launch_rg_rows(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
@@ -678,13 +680,14 @@ int launch_rg_cols(ks_loop* h, const Bufs<float>& p, cudaStream_t s) {
     return KS_OK;
 }
 
-// Tiles and twiddles of the register kernels: row lengths 32 .. 512, column lengths 32 .. 1024, in
-// batches that give their row phases a block or so for every second SM.  A warp's chain over sixteen
-// points a thread is long, and below that line the items' many short ones end sooner (us a step in four
-// launches, register kernels / items, at their blocks of rows: one 256x256 loop, 16, 29.1 / 22.0; one
-// 128x512, 16, 27.9 / 23.9; 18 of 64x256, 72, 27.4 / 24.5; 40 of 32x64, 20, 23.2 / 19.7; beyond it 18 of
-// 64x512, 144, 27.6 / 32.1; 18 of 256x128, 144, 28.3 / 34.4; 64 of 64x128, 128, 26.7 / 29.6; with columns
-// of up to 64 points 300 of 32x32, 75, 29.1 / 33.6; 40 of 128x64, 80, 21.9 / 30.6).
+// Tiles and twiddles of the register kernels: row lengths 32 .. 512, column lengths 32 .. 1024.  Steps take
+// them in batches that give their row phases a block or so for every second SM.  A warp's chain over
+// sixteen points a thread is long, and below that line the items' many short ones end sooner (us a step in
+// four launches, register kernels / items, at their blocks of rows: one 256x256 loop, 16, 29.1 / 22.0; one
+// 128x512, 16, 27.9 / 23.9; 40 of 32x64, 20, 23.2 / 19.7).  With columns of up to 64 points, or of 512 and
+// more, which a block of items holds long, the line is 64 blocks (40 of 128x64, 80, 21.9 / 30.6; 300 of
+// 32x32, 75, 29.1 / 33.6; two of 256x512, 64, 28.8 / 30.2; 8 of 32x1024, 64, 29.2 / 27.7), with those
+// between 96 (18 of 64x256, 72, 27.4 / 24.5; 40 of 64x128, 80, 26.5 / 25.3; 64 of 64x128, 128, 26.7 / 29.6).
 int setup_rg(ks_loop* h) {
     const int nx = h->d.nx;
     if (nx < 32 || nx > 512) return KS_OK;
@@ -694,7 +697,7 @@ int setup_rg(ks_loop* h) {
     const int step = 1024 / nx;  // 2 F rows, F = 32 / (nx / 16) pairs a warp
     for (int b = 0; b < h->d.B; ++b)
         for (int n0 = 0; n0 < h->ns[b]; n0 += step) rows.push_back(RgTile{b, n0});
-    if ((int)rows.size() <= (h->nsmax <= 64 ? 63 : 95) * (RG_THREADS / 32)) return KS_OK;
+    h->rg_steps = (int)rows.size() > (h->nsmax > 64 && h->nsmax < 512 ? 95 : 63) * (RG_THREADS / 32);
     std::vector<RgCol> cols;  // in colorder: the 1024-point loops come first
     for (int b : h->colorder) {
         const int F = std::max(1, 512 / h->ns[b]);
@@ -1065,7 +1068,7 @@ int auto_form(const ks_loop* h, int pr) {
     if (pr == P64) return Q >= (waves ? 512 : 2048) ? 2 : 0;
     const int m = std::max(h->d.nx, h->nsmax);
     if (h->xi) return Q >= (waves || m >= 1024 ? 2048 : h->nsmax < 64 ? 8192 : 4096) ? 2 : 0;
-    if (waves) return Q >= (use_rg(h) ? 1024 : 2048) ? 2 : 0;
+    if (waves) return Q >= (h->rg_steps ? 1024 : 2048) ? 2 : 0;
     return Q >= (m >= 512 || (B >= 8 && !ragged && h->nsmax >= 32) ? 2048 : 4096) ? 2 : 0;
 }
 
@@ -1144,7 +1147,7 @@ int run_analyze(ks_loop* h, Work& w, double* io, const float* iof, const double*
     p.iof = iof;
     p.uhf = iof ? (cpx<float>*)w.uh[P32] : nullptr;
     KS_TRY((launch_rows<double, ROW_ANALYZE>(h, p, s)));
-    const Linked linked(h);
+    const Flag linked(h->linked);
     const bool fuse = prime && !iof && !h->xi;
     if (fuse) KS_TRY((launch_cols<double, COL_ANALYZE_U>(h, p, s)));
     else KS_TRY((launch_cols<double, COL_ANALYZE>(h, p, s)));
@@ -1178,6 +1181,7 @@ int run_prime(ks_loop* h, Work& w, int pr, cudaStream_t s) {
 template <typename R>
 int run_step(ks_loop* h, Work& w, int pr, double tol, double switch_tol, cudaStream_t s) {
     Bufs<R> p = make_bufs<R>(h, w, pr, 1, tol, switch_tol, (R*)nullptr);
+    const Flag stepping(h->stepping);
     KS_TRY((launch_rows<R, ROW_NONLIN>(h, p, s)));
     KS_TRY((launch_cols<R, COL_RESID>(h, p, s)));
     KS_TRY((launch_rows<R, ROW_ADJ>(h, p, s)));
@@ -1193,7 +1197,7 @@ template <typename R, int CMODE>
 int run_residual(ks_loop* h, Work& w, int pr, cudaStream_t s, bool chained = false) {
     Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, (R*)nullptr);
     const bool primed = w.mix_valid[pr];
-    const Linked linked(h);
+    const Flag linked(h->linked);
     h->linked = chained;
     if (!primed) KS_TRY((launch_cols<R, COL_SYNTH_U>(h, p, s)));
     h->linked = chained || !primed;
@@ -1209,7 +1213,7 @@ int run_residual(ks_loop* h, Work& w, int pr, cudaStream_t s, bool chained = fal
 template <typename R>
 int run_gradient(ks_loop* h, Work& w, int pr, cudaStream_t s) {
     KS_TRY((run_residual<R, COL_RESID>(h, w, pr, s, true)));
-    const Linked linked(h);
+    const Flag linked(h->linked);
     Bufs<R> p = make_bufs<R>(h, w, pr, 0, 0.0, 0.0, (R*)nullptr);
     KS_TRY((launch_rows<R, ROW_ADJ>(h, p, s)));
     if (!h->xi) return launch_cols<R, COL_GRAD_G>(h, p, s);
@@ -1224,7 +1228,7 @@ int run_rows_out(ks_loop* h, Work& w, int pr, R* io, double* J, double* dJdT, cu
     p.fin = 1;
     p.Jout = J;
     p.dJdTout = dJdT;
-    const Linked linked(h);
+    const Flag linked(h->linked);
     return launch_rows<R, ROW_SYNTH>(h, p, s);
 }
 

@@ -12,11 +12,13 @@ from paper_2007_06427_gb300.inputs import spectral_loop
 
 pytestmark = pytest.mark.gpu
 
-# tiles of 1024 points of rows: more than 252 (columns of up to 64 points) or 380 take the kernels
+# tiles of 1024 points of rows: more than 252 (columns of up to 64, or of 512 points and more) or 380 take
+# the kernels
 SHAPES = [(32, [32] * 300), (32, [64, 128, 32] * 60), (64, [32, 64, 128, 256] * 14), (64, [512] * 13),
           (128, [128, 32] * 40), (128, [1024, 64, 1024, 64, 1024]), (256, [256, 32] * 6),
           (512, [32, 64, 32] * 7), (512, [1024]),
-          (64, [64] * 63), (64, [64] * 64), (64, [128] * 47), (64, [128] * 48)]  # the line
+          (64, [64] * 63), (64, [64] * 64), (64, [128] * 47), (64, [128] * 48), (64, [512] * 7),
+          (64, [512] * 8)]  # the line
 
 
 def descend(nx, ns, path, steps, scheme=K.KS_IMEX, dtau=0.1, tol=0.0):
