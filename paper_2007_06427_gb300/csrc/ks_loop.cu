@@ -623,11 +623,13 @@ struct LaunchScope {
 // Launch of a phase kernel.  linked (the boundary calls: load, residual, gradient): the launch in front of
 // it in stream s is a phase kernel too; it may then start while that one ends (programmatic dependent
 // launch): its blocks stage their tables and wait (grid_wait, in every phase kernel) until the launch in
-// front has completed, which had waited for its own.  A 32x32 residual, five launches: 36.9 -> 29.3 us a
-// call.  Its early blocks are placed on the SMs that happen to be free first, and stay uneven: float
-// launches of more than a block per SM are not linked, and neither are the steps, which gained 1 to 4 %
-// on single small loops and on 256 ragged ones and lost up to half elsewhere (linked / not, us a step,
-// four-launch form: double 128x1024 89.5 / 60.0, 18 of 128x256 102 / 62, two of 64x512 in the
+// front has completed, which had waited for its own.  A 32x32 residual, five launches: 36.9 -> 27.2 us a
+// call.  Its early blocks are placed on the SMs that happen to be free first, and stay uneven, which long
+// blocks do not make up for: double launches of loops with transforms of 512 or 1024 points are not linked
+// (J alone of 8 loops of 32x512 linked / not, 1.3 of the time, of a 256x1024 loop in the subspace 1.31; up to
+// 256 points 0.92 in the median), nor are float launches of more than a block per SM.  Neither are the
+// steps, which gained 1 to 4 % on single small loops and on 256 ragged ones and lost up to half elsewhere
+// (us a step, four-launch form: double 128x1024 89.5 / 60.0, 18 of 128x256 102 / 62, two of 64x512 in the
 // subspace 80 / 51; float 64 of 64x128 33.3 / 26.7, two of 256x512 in the subspace 48.5 / 32.5).
 template <typename R, typename... KA, typename... A>
 cudaError_t launch_linked(const ks_loop* h, void (*k)(KA...), int grid, int block, size_t smem, cudaStream_t s,
@@ -641,7 +643,8 @@ cudaError_t launch_linked(const ks_loop* h, void (*k)(KA...), int grid, int bloc
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = h->linked && !h->prof && (sizeof(R) == 8 || grid <= 152) ? 1 : 0;
+    const bool even = sizeof(R) == 8 ? std::max(h->d.nx, h->nsmax) <= 256 : grid <= 152;
+    cfg.numAttrs = h->linked && !h->prof && even ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k, KA(a)...);
 }
 
