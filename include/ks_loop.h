@@ -24,7 +24,8 @@
  *    laid out [n][m] with the x-index m fastest; loops follow one another in batch order.
  *    Their element type is double for KS_FP64 and KS_MIXED handles and float for KS_FP32.
  *  - Every input field is first projected onto the 2/3 band; all results are those of the
- *    projected loop.
+ *    projected loop.  Double transforms take their scale from their inputs: infinities and NaN
+ *    give NaN throughout, and a transform whose inputs are all below 2^-913 (1e-275) gives zeros.
  *  - T and the per-loop outputs are double arrays of length `batch` (steps: long long,
  *    status: int).
  *  - Pointers may be device pointers or ordinary host pointers; the library tells them apart

@@ -499,7 +499,9 @@ struct RgCol {
 //
 // Three blocks an SM (168 registers, a 48-byte spill in COL_RESID): left at 222 to 231 registers two fit,
 // and the 352 blocks of 256 ragged loops or the 344 of eight 256x1024 loops took a second wave for the
-// last 40 (120 and 60 steps: 6093 -> 5253 us, 3269 -> 2680 us, ff_add's shorter sum included).
+// last 40 (120 and 60 steps: 6093 -> 5253 us, 3269 -> 2680 us, ff_add's shorter sum included).  Over 77
+// batches that take these kernels the step takes 0.79 to 1.01 of its time with two, below 0.93 where there
+// are more than two blocks an SM.
 template <int MODE>
 __global__ void __launch_bounds__(RG_THREADS, 3) k_rg_cols(Dims d, Bufs<float> p, const RgCol* tiles, int npairs,
                                                         const rgv* tab, int ntab) {
