@@ -35,42 +35,38 @@ class KSLoopJ(torch.autograd.Function):
         loop = ctx.loop
         G = torch.empty_like(u)
         dJdT = torch.empty_like(T)
-        K.ks_adjoint_grad(loop.handle, u, T, G, dJdT, torch.cuda.current_stream(u.device))
+        stream = torch.cuda.current_stream(u.device)
+        K.ks_adjoint_grad(loop.handle, u, T, G, dJdT, stream)
         gu = gT = None
         gJ = gJ.to(torch.float64)
         if ctx.needs_input_grad[0]:
-            per_loop = (gJ * loop_factor(loop, u.device)).to(G.dtype)
-            gu = G * per_loop.index_select(0, loop_index(loop, u.device))
+            factor, index = constants(loop, u.device, stream)
+            gu = G * (gJ * factor).to(G.dtype).index_select(0, index)
         if ctx.needs_input_grad[1]:
             gT = dJdT * gJ
         return gu, gT, None
 
 
-def loop_index(loop, device):
-    """Loop of each packed grid value (a gather by it needs no host read of the lengths)."""
-    def make():
-        sizes = torch.tensor([n * loop.nx for n in loop.ns], dtype=torch.int64, device=device)
-        return torch.repeat_interleave(torch.arange(loop.batch, device=device), sizes)
-    return _constant(loop, "index", device, make)
-
-
-def loop_factor(loop, device):
-    """2 L / (Nx Ns_b) per loop."""
-    return _constant(loop, "factor", device, lambda: torch.tensor(
-        [2.0 * loop.L / (loop.nx * n) for n in loop.ns], dtype=torch.float64, device=device))
-
-
-def _constant(loop, name, device, make):
-    """A tensor kept with the handle.  It is complete before any other call can see it: the stream
-    of the first backward made it, and a later one may run on another that is not ordered behind."""
+def constants(loop, device, stream):
+    """2 L / (Nx Ns_b) per loop and the loop of each packed grid value (a gather by it needs no host
+    read of the lengths), kept with the handle, once per stream: those that another stream made need
+    not be complete on this one.  Under capture, where they cannot be made, any that are there serve: a
+    capture starts behind all earlier work."""
     cache = loop.__dict__.setdefault("_cache", {})
-    key = (name, str(device))
+    key = (device, stream.cuda_stream)
     if key not in cache:
-        value = make()
-        if value.is_cuda:
-            torch.cuda.current_stream(value.device).synchronize()
-        cache[key] = value
+        made = [v for k, v in cache.items() if k[0] == device]
+        if made and torch.cuda.is_current_stream_capturing():
+            return made[0]
+        cache[key] = make_constants(loop, device)
     return cache[key]
+
+
+def make_constants(loop, device):
+    factor = torch.tensor([2.0 * loop.L / (loop.nx * n) for n in loop.ns], dtype=torch.float64,
+                          device=device)
+    sizes = torch.tensor([n * loop.nx for n in loop.ns], dtype=torch.int64, device=device)
+    return factor, torch.repeat_interleave(torch.arange(loop.batch, device=device), sizes)
 
 
 def cost(u: torch.Tensor, T: torch.Tensor, loop: "K.KSLoop") -> torch.Tensor:
